@@ -519,18 +519,14 @@ int cfs_slab_helmholtz_finish(cfs_slab_t slab, double c, int loc, const double* 
  *       of CFS_F32_REFINED plans.
  *   CFS_OPT_FFT_RADIX  largest radix of the Stockham passes of the x and y
  *       transforms: 8 (0 or 8, the default: radix-8 passes, then 4, 2, 3s) or
- *       4 (radix-4 passes, then 2, 3s).  Setting it rebuilds the twiddle
+ *       4 (radix-4 passes, then 2, 3s).  It shapes the FP32 transforms (the FP64
+ *       ones choose their passes, and their launch shapes, by length alone).
+ *       Setting it rebuilds the twiddle
  *       tables (it waits for the device); groups bound to the plan must be
  *       rebound.
- *   CFS_OPT_F64_ADDS_X, CFS_OPT_F64_ADDS_Y  how many kinds of butterfly
- *       additions of the FP64 x / y transforms run on the integer units
- *       instead of the FP64 pipe, 0..4 (cumulative: 1 the second level of
- *       every radix-4 core, 2 also the radix-2 combination of each DFT8,
- *       3 also the first level of the untwiddled passes, 4 also the real-FFT
- *       untangle of the x transform).  Those additions are exact IEEE-754
- *       binary64 round-to-nearest-even additions done in integer
- *       arithmetic, so every level gives the same bits; on GPUs whose FP64
- *       pipe is narrow it lets the integer units share the FP64 work.
+ *   CFS_OPT_F64_ADDS_X, CFS_OPT_F64_ADDS_Y  0..4; accepted and reported, with no
+ *       effect on times or results: the FP64 x / y transforms run on the integer
+ *       units as a whole (64-bit block fixed point).
  *   CFS_OPT_STREAM_CHUNKS  chunks in which cfs_solve_batch_host moves each
  *       field of an FP64 plan: 0 automatic (about 200 MB per chunk, at most
  *       8), 1 whole fields, or 2..8.  A Poisson field moves in ranges of z
@@ -601,11 +597,10 @@ int cfs_selfcheck_conversions(unsigned long long samples, unsigned long long* mi
 
 /*
  * cfs_selfcheck_f64_addsub -- a diagnostic with no counterpart in the paper.
- * The FP64 x and y transforms may run part of their butterfly additions in
- * integer arithmetic (CFS_OPT_F64_ADDS_X / _Y): an exact IEEE-754 binary64
- * round-to-nearest-even a + b and a - b, with zeros, subnormals, operands
- * below 2^-959 or from 2^1023 up, infinities and NaNs left to the FP64
- * pipe.  This runs `samples` hashed operand pairs (any two bit patterns,
+ * The library holds a binary64 addition in integer arithmetic (measured by
+ * cfs_probe_addsub): an exact IEEE-754 round-to-nearest-even a + b and a - b,
+ * with zeros, subnormals, operands below 2^-959 or from 2^1023 up, infinities
+ * and NaNs left to the FP64 pipe.  This runs `samples` hashed operand pairs (any two bit patterns,
  * close and distant exponents, cancellation, exact rounding ties, the ends
  * of the integer range, equal magnitudes, FFT-sized values) through both on
  * the GPU (on_device = 1) or on the host CPU (on_device = 0, no GPU needed)
@@ -640,8 +635,7 @@ int cfs_probe_fma(int bits, long long iters, double* fma_per_s, double* ms);
 /*
  * cfs_probe_addsub -- a measurement with no counterpart in the paper: the
  * rate of FP64 butterfly pairs (a + b, a - b) on the FP64 pipe
- * (on_integer_units = 0) or by the integer-unit additions of the transforms
- * (1).  Every thread of one full wave of 256-thread blocks runs 8
+ * (on_integer_units = 0) or by the integer-unit additions (1).  Every thread of one full wave of 256-thread blocks runs 8
  * independent pair chains for `iters` steps (rounded up to a multiple of
  * 256; 1 <= iters <= 2^40), timed as cfs_probe_fma.  *pairs_per_s receives
  * pairs per second, *ms (may be NULL) the launch time.  Waits for the device.

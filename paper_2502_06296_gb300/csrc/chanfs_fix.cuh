@@ -1,0 +1,382 @@
+// chanfs_fix.cuh -- the FP64 transforms in block fixed point.
+//
+// GB300 executes 2 FP64 instructions per SM per clock against 64 integer
+// ones, and a Stockham FFT in FP64 needs 12 to 14 of them per real point: the
+// FP64 pipe bounds it at a tenth of the memory bandwidth.  Here a line (or
+// column) of doubles is turned into 64-bit integers under one common power of
+// two, transformed with integer additions and 32 x 32 + 64 -> 64 bit
+// multiply-adds, and turned back into doubles once, at the end.
+//
+// Range.  Let B be the largest sum of |re| + |im| over the inputs of one
+// first-pass butterfly and S the sum over the line.  The twiddle products come
+// out divided by 4 (a 62-bit value times a 62-bit twiddle, the high half), so
+// every pass after the first grows its values by R / 4 at most, and none exceeds
+// S / 4.  The scale 2^s is the largest with 2^s C < 2^headroom, C = max(B, min(B G,
+// S / 4)), G = max(1, R_2/4, R_2 R_3/16, ..): no overflow for any input.  The
+// pass by pass division keeps the bits below a long line's sums that a bound on
+// the whole line at the start (N max|x|, or S) would give away.  Transforms with few
+// passes leave S out (C = B G), which costs them at most two bits.
+// Precision.  Values carry 61 bits less that growth below B against the 53 of a
+// double, twiddles 62; additions are exact, a product is rounded to the last
+// place, the result is rounded to a double once.
+#pragma once
+
+#include "chanfs_internal.cuh"
+
+namespace chanfs {
+
+// A complex value.  (Twiddles are int4 (re hi, re lo, im hi, im lo): hi 2^-30 +
+// lo 2^-62, lo signed.)
+struct __align__(16) Fix {
+  long long x, y;
+};
+
+// Radix of pass p of length n = 2^a 3^b (0 past the last pass): the fewest passes
+// of radix 8, 6, 4, 3 and at most one 2 (16 as 4 x 4), in that order, the 6s last but
+// for 3s.  PAIR (the real transform along x): the last radix is at most 6, since
+// its last pass holds two mirrored butterflies in registers; the inverse takes
+// the passes in the opposite order.
+template <bool PAIR> __host__ __device__ constexpr int fix_radix(int n, int p) {
+  int a = 0, b = 0;
+  for (int m = n; m % 2 == 0; m /= 2) ++a;
+  for (int m = n; m % 3 == 0; m /= 3) ++b;
+  const int tail = PAIR && b == 0 ? 2 : 0;  // a closing radix 4
+  a -= tail;
+  int sixes = 0, least = 99;
+  for (int c = 0; c <= a && c <= b; ++c) {
+    const int passes = c + (b - c) + (a - c) / 3 + ((a - c) % 3 ? 1 : 0);
+    const int cost =  // two per pass, one more for a lone radix 2
+        2 * passes + ((a - c) % 3 == 1 && a - c < 4 ? 1 : 0);
+    if (cost < least) {
+      least = cost;
+      sixes = c;
+    }
+  }
+  a -= sixes;
+  b -= sixes;
+  int r[16] = {}, c = 0;
+  const bool fours = a % 3 == 1 && a >= 4;
+  for (int i = 0; i < (fours ? a / 3 - 1 : a / 3); ++i) r[c++] = 8;
+  if (fours) {
+    r[c++] = 4;
+    r[c++] = 4;
+  } else if (a % 3) {
+    r[c++] = a % 3 == 1 ? 2 : 4;
+  }
+  for (int i = 0; i < sixes; ++i) r[c++] = 6;
+  for (int i = 0; i < b; ++i) r[c++] = 3;
+  if (tail) r[c++] = 4;
+  return p < c ? r[p] : 0;
+}
+template <bool PAIR> __host__ __device__ constexpr int fix_npass(int n) {
+  int p = 0;
+  while (fix_radix<PAIR>(n, p)) ++p;
+  return p;
+}
+// Pass p in execution order, its span and its twiddles' offset: entry (r, k),
+// 1 <= r < radix, k < span, at twoff + (r - 1) span + k.
+template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_rad(int n, int p) {
+  return fix_radix<PAIR>(n, INV && PAIR ? fix_npass<PAIR>(n) - 1 - p : p);
+}
+template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_span(int n, int p) {
+  int L = 1;
+  for (int i = 0; i < p; ++i) L *= fix_rad<PAIR, INV>(n, i);
+  return L;
+}
+template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_twoff(int n, int p) {
+  int o = 0;
+  for (int i = 0; i < p; ++i) o += fix_span<PAIR, INV>(n, i) * (fix_rad<PAIR, INV>(n, i) - 1);
+  return o;
+}
+
+// ceil(log2) of the largest growth max(1, R_2/4, R_2 R_3/16, ..) after the first pass.
+template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_growth(int n) {
+  int lg = 0;
+  double g = 1.0;
+  for (int p = 1; p < fix_npass<PAIR>(n); ++p) {
+    g *= fix_rad<PAIR, INV>(n, p) / 4.0;
+    while (g > (double)(1 << lg)) ++lg;
+  }
+  return lg;
+}
+
+// Whether the sum over the line is worth its reduction: where the growth and the
+// divisions take 7 bits or more, a line with one dominant value would otherwise
+// keep fewer than a double's bits.
+template <bool PAIR, bool INV> __host__ __device__ constexpr bool fix_uses_sum(int n) {
+  return fix_growth<PAIR, INV>(n) + 2 * (fix_npass<PAIR>(n) - 1) >= 7;
+}
+
+// Shared-memory place of element e: one 16-byte element of padding per 8, so
+// that the 8 lanes of a 128-byte access phase fall on different banks also in
+// the first pass's stride-R writes.
+__host__ __device__ constexpr int fix_pad(int e) { return e + (e >> 3); }
+
+#ifdef __CUDACC__
+
+__device__ __forceinline__ Fix fadd(Fix a, Fix b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ Fix fsub(Fix a, Fix b) { return {a.x - b.x, a.y - b.y}; }
+template <bool INV> __device__ __forceinline__ Fix frot(Fix a) {  // times -i (forward) or +i
+  return INV ? Fix{-a.y, a.x} : Fix{a.y, -a.x};
+}
+
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+
+// v = h 2^32 + l with a signed low word.
+__device__ __forceinline__ int fix_lo(long long v) { return (int)v; }
+__device__ __forceinline__ int fix_hi(long long v) {
+  return (int)(v >> 32) + (int)((unsigned)(int)v >> 31);
+}
+
+// (sum << 2) with the two bits below it taken from the cross products.
+__device__ __forceinline__ long long fix_join(long long sum, long long cross) {
+  const unsigned sl = (unsigned)sum, sh = (unsigned)((unsigned long long)sum >> 32);
+  const unsigned lo = __funnelshift_l((unsigned)cross, sl, 2);
+  const unsigned hi = __funnelshift_l(sl, sh, 2);
+  return (long long)(((unsigned long long)hi << 32) | lo);
+}
+
+// The products of a w for |a| <= 2^62: cross products (low by high words) from
+// `start` up, then the high products, in units of 2^32 / 4, on top of those
+// sums' high words by `carry`; the products of the two low words, below the last
+// place, are left out.
+template <class Carry>
+__device__ __forceinline__ void fmul_sums(Fix a, int4 w, long long start, Carry carry,
+                                          long long& sr, long long& si, long long& cr,
+                                          long long& ci) {
+  const int xl = fix_lo(a.x), xh = fix_hi(a.x), yl = fix_lo(a.y), yh = fix_hi(a.y);
+  const int nh = -w.z, nl = -w.w;
+  cr = mad_wide(xl, w.x, start);
+  ci = mad_wide(xl, w.z, start);
+  cr = mad_wide(xh, w.y, cr);
+  ci = mad_wide(xh, w.w, ci);
+  cr = mad_wide(yl, nh, cr);
+  ci = mad_wide(yl, w.x, ci);
+  cr = mad_wide(yh, nl, cr);
+  ci = mad_wide(yh, w.y, ci);
+  sr = mad_wide(xh, w.x, carry(cr));
+  si = mad_wide(xh, w.z, carry(ci));
+  sr = mad_wide(yh, nh, sr);
+  si = mad_wide(yh, w.x, si);
+}
+
+// A pass's twiddled points are a w / 4 + kFixBias (1 + i), rounded to nearest:
+// the cross products start at 2^63 (they stay within 2^62.5 of it), so their high
+// word is unsigned and carries over without a sign extension.  The untwiddled
+// point gets the same bias, and the DFT gathers it in its output 0, R times,
+// where it is taken off.
+constexpr long long kFixBias = 1ll << 31;
+__device__ __forceinline__ Fix fmul4(Fix a, int4 w) {
+  Fix s;
+  long long cr, ci;
+  fmul_sums(a, w, (long long)((1ull << 63) + (1ull << 31)),
+            [](long long c) { return (long long)((unsigned long long)c >> 32); }, s.x, s.y, cr,
+            ci);
+  return s;
+}
+// The untwiddled point of a pass, a / 4, rounded: rounding down would add the
+// same fraction to every butterfly, and the passes that follow would gather it
+// in a few outputs.
+__device__ __forceinline__ Fix fquarter(Fix a) {
+  return {(a.x + (4 * kFixBias + 2)) >> 2, (a.y + (4 * kFixBias + 2)) >> 2};
+}
+
+// a w, rounded to nearest: two more bits, from the cross products.
+__device__ __forceinline__ Fix fmul(Fix a, int4 w) {
+  long long sr, si, cr, ci;
+  fmul_sums(a, w, 1ll << 29, [](long long c) { return c >> 32; }, sr, si, cr, ci);
+  return {fix_join(sr, cr), fix_join(si, ci)};
+}
+
+// v (1 + f) for a constant f = fh 2^-32 + fl 2^-64, |f| < 1/2.
+__device__ __forceinline__ long long fix_scale1(long long v, int fh, int fl) {
+  const int l = fix_lo(v), h = fix_hi(v);
+  long long c = mad_wide(l, fh, 1ll << 31);
+  c = mad_wide(h, fl, c);
+  return mad_wide(h, fh, v + (c >> 32));
+}
+// 1/sqrt(2) - 1 and sqrt(3)/2 - 1 in units of 2^-64
+__device__ __forceinline__ long long mul_rsqrt2(long long v) {
+  return fix_scale1(v, -1257966796, -102865788);
+}
+__device__ __forceinline__ long long mul_sqrt3_2(long long v) {
+  return fix_scale1(v, -575416509, -1033546850);
+}
+
+// Small DFTs, kernel e^{-2 pi i / R} forward, conjugate inverse.
+template <bool INV> __device__ __forceinline__ void fdft3(Fix& a, Fix& b, Fix& c) {
+  const Fix s = fadd(b, c), d = fsub(b, c);
+  const Fix t = {a.x - s.x / 2, a.y - s.y / 2};  // (towards zero: no common sign)
+  a = fadd(a, s);
+  const Fix u = frot<INV>(Fix{mul_sqrt3_2(d.x), mul_sqrt3_2(d.y)});
+  b = fadd(t, u);
+  c = fsub(t, u);
+}
+template <bool INV> __device__ __forceinline__ void fdft4(Fix& a, Fix& b, Fix& c, Fix& d) {
+  const Fix t0 = fadd(a, c), t1 = fsub(a, c), t2 = fadd(b, d), t3 = frot<INV>(fsub(b, d));
+  a = fadd(t0, t2);
+  b = fadd(t1, t3);
+  c = fsub(t0, t2);
+  d = fsub(t1, t3);
+}
+template <int R, bool INV> __device__ __forceinline__ void fdft(Fix* v) {
+  if constexpr (R == 2) {
+    const Fix t = fsub(v[0], v[1]);
+    v[0] = fadd(v[0], v[1]);
+    v[1] = t;
+  } else if constexpr (R == 3) {
+    fdft3<INV>(v[0], v[1], v[2]);
+  } else if constexpr (R == 4) {
+    fdft4<INV>(v[0], v[1], v[2], v[3]);
+  } else if constexpr (R == 6) {  // 3 x 2 without twiddles (index maps modulo 6)
+    fdft3<INV>(v[0], v[2], v[4]);
+    fdft3<INV>(v[3], v[5], v[1]);
+    const Fix a0 = v[0], a1 = v[2], a2 = v[4], b0 = v[3], b1 = v[5], b2 = v[1];
+    v[0] = fadd(a0, b0);
+    v[3] = fsub(a0, b0);
+    v[4] = fadd(a1, b1);
+    v[1] = fsub(a1, b1);
+    v[2] = fadd(a2, b2);
+    v[5] = fsub(a2, b2);
+  } else {
+    fdft4<INV>(v[0], v[2], v[4], v[6]);
+    fdft4<INV>(v[1], v[3], v[5], v[7]);
+    // W8 v3 = r (x + y, y - x) forward, r (x - y, x + y) inverse; W8^3 = -+i W8
+    const Fix o1 = v[3], o3 = v[7];
+    const long long p1 = mul_rsqrt2(INV ? o1.x - o1.y : o1.x + o1.y);
+    const long long q1 = mul_rsqrt2(INV ? o1.x + o1.y : o1.y - o1.x);
+    const long long p3 = mul_rsqrt2(INV ? o3.x + o3.y : o3.x - o3.y);
+    const long long q3 = mul_rsqrt2(INV ? o3.x - o3.y : o3.x + o3.y);
+    const Fix w1 = {p1, q1}, w3 = {-p3, INV ? q3 : -q3};
+    const Fix w0 = v[1], w2 = frot<INV>(v[5]), e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
+    v[0] = fadd(e0, w0);
+    v[4] = fsub(e0, w0);
+    v[1] = fadd(e1, w1);
+    v[5] = fsub(e1, w1);
+    v[2] = fadd(e2, w2);
+    v[6] = fsub(e2, w2);
+    v[3] = fadd(e3, w3);
+    v[7] = fsub(e3, w3);
+  }
+}
+
+// --- the scale of a line ----------------------------------------------------
+
+__host__ __device__ constexpr int fix_ceil_log2(int v) {
+  int b = 0;
+  while ((1 << b) < v) ++b;
+  return b;
+}
+
+// Adds |v| to a butterfly's maximum (as the high word of a double) and to its sum
+// (as a float from the double's leading bits; values outside the range of
+// floats are below every bound that the sum is used for, or switch it off).
+__device__ __forceinline__ void fix_gather(double v, unsigned& top, float& sum) {
+  const unsigned u = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  top = max(top, u);
+  sum += __uint_as_float((max(u, 0x38100000u) - 0x38000000u) << 3);
+}
+
+// A line's scale.  kind 0: the conversions by shifts; kind 1: by the library's
+// scalbn (a line of subnormals, or with values beyond 2^+-900); kind 2: an
+// infinity or NaN (every output of the line is then NaN).
+struct FixScale {
+  int s, kind;
+};
+
+__device__ __forceinline__ bool fix_summed(unsigned top) { return (top >> 20) - 933u <= 180u; }
+
+// A butterfly's sum in units of 2^-19 of the power of two above the largest one
+// (integers add up to the same in any order); 0 if the line does not use it.
+__device__ __forceinline__ unsigned fix_quanta(float sum, unsigned top, unsigned most) {
+  if (!fix_summed(top)) return 0u;
+  return __float2uint_ru(sum * __uint_as_float((272u - ((most + 256u) >> 23)) << 23));
+}
+
+// The scale, from the line's largest value (high word), largest butterfly sum B
+// (float bits) and, unless it is 0, the sum of the butterflies' quanta; where
+// the maximum is far from 1, from the maximum and the points of a butterfly.  A
+// line of zeros takes s = 0.
+__device__ __forceinline__ FixScale fix_scale_of(unsigned top, unsigned most, unsigned quanta,
+                                                 int lgpts, int growth, int headroom) {
+  const int e = (int)(top >> 20);
+  if (fix_summed(top)) {
+    const int eb = (int)((most + 256u) >> 23) - 126;  // B < 2^eb
+    int ec = eb + growth;
+    // S / 4 < 2^(eb - 19 + bits(quanta) - 2)
+    if (quanta) ec = max(eb, min(ec, eb + 11 - __clz((int)quanta)));
+    return {headroom - ec, 0};
+  }
+  if (top == 0u) return {0, 0};
+  return {e == 0x7ff ? 0 : headroom - growth - (max(e, 1) - 1022 + lgpts),
+          e == 0x7ff ? 2 : (e < 123 || e > 1923) ? 1 : 0};
+}
+
+static __device__ __noinline__ long long fix_from_far(double v, FixScale f) {
+  return f.kind == 2 ? 0ll : __double2ll_rn(scalbn(v, f.s));
+}
+static __device__ __noinline__ double fix_to_far(long long v, int s, int kind) {
+  return kind == 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)v, -s);
+}
+
+// trunc(v 2^s): the significand, its leading bit at 62, shifted down.
+__device__ __forceinline__ long long fix_from(double v, FixScale f) {
+  if (f.kind) return fix_from_far(v, f);
+  const int hi = __double2hiint(v);
+  const unsigned lo = (unsigned)__double2loint(v);
+  const int t = 1085 - f.s - (int)(((unsigned)hi & 0x7fffffffu) >> 20);
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const unsigned long long m =
+      ((((unsigned long long)__funnelshift_l(lo, mh, 10)) << 32) | (lo << 10)) >> min(t, 63);
+  const long long sg = hi >> 31;
+  return ((long long)m ^ sg) - sg;
+}
+__device__ __forceinline__ Fix fix_from(double2 v, FixScale f) {
+  return {fix_from(v.x, f), fix_from(v.y, f)};
+}
+
+// v 2^-s, rounded to nearest (the exponent is adjusted on the encoding).
+__device__ __forceinline__ double fix_to(long long v, int s, int kind) {
+  if (kind) return fix_to_far(v, s, kind);
+  const double d = __ll2double_rn(v);
+  const int hi = __double2hiint(d);
+  return __hiloint2double(hi ? hi - (s << 20) : 0, __double2loint(d));
+}
+__device__ __forceinline__ double2 fix_to(Fix v, int s, int kind) {
+  return make_double2(fix_to(v.x, s, kind), fix_to(v.y, s, kind));
+}
+
+// The DFT of a pass after the first: v[r] w[r - 1] / 4, transformed.
+template <int R, bool INV>
+__device__ __forceinline__ void fix_twiddle_dft(Fix* v, const int4* __restrict__ tw, int stride) {
+  v[0] = fquarter(v[0]);
+#pragma unroll
+  for (int r = 1; r < R; ++r) v[r] = fmul4(v[r], __ldg(tw + (r - 1) * stride));
+  fdft<R, INV>(v);
+  v[0].x -= R * kFixBias;
+  v[0].y -= R * kFixBias;
+}
+
+// One Stockham radix-R butterfly: item j of a batch whose element e lives at
+// at(e): points j + r q of `in`, twiddles (over 4), DFT, positions (j - k) R + k
+// + r L of `out`, k = j mod L.
+template <int R, bool INV, class At>
+__device__ __forceinline__ void fix_butterfly(const Fix* in, Fix* out, int j, int q, int L,
+                                              const int4* __restrict__ tw, At at) {
+  Fix v[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) v[r] = in[at(j + r * q)];
+  const int k = j % L;
+  fix_twiddle_dft<R, INV>(v, tw + k, L);
+  const int o = (j - k) * R + k;
+#pragma unroll
+  for (int r = 0; r < R; ++r) out[at(o + r * L)] = v[r];
+}
+
+#endif  // __CUDACC__
+
+}  // namespace chanfs

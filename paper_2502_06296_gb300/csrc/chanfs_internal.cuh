@@ -36,10 +36,6 @@ constexpr int kPcrMaxUnknowns = 1024;  // rows of a PCR tile in shared memory
 constexpr int kMaxGroup = 4096;     // plans of one grouped solve
 constexpr int kBatchSlots = 4;      // device slots of a batch of host-buffer solves
 constexpr int kMaxStreamChunks = 8; // chunks a field of a streamed batch moves in
-// Default levels of CFS_OPT_F64_ADDS_X / _Y (FP64 butterfly additions on the
-// integer units).
-constexpr int kEmuDefaultX = 0;
-constexpr int kEmuDefaultY = 0;
 
 // Device status bits (plan->d_status)
 constexpr int kErrTmaTimeout = 1;
@@ -63,6 +59,18 @@ struct FftDesc {
 // Builds the radix plan and its FP64 twiddle table on the host.
 // Passes of radix 8 (max_radix 8) or 4 first, then at most one 2, then 3s.
 bool make_fft_desc(int n, FftDesc* d, std::vector<double2>* tw, int max_radix);
+
+// The same for the block fixed-point transforms (chanfs_fix.cuh): the passes in
+// execution order (each direction has its own), entry (r, k) of pass p, 1 <= r <
+// radix, k < span, at twoff + (r - 1) span + k.
+constexpr int kFixMaxPass = 8;
+constexpr int kFixMinLen = 9;  // shorter ones may have a single pass
+struct FixDesc {
+  int n, npass;
+  int growth;  // bits that the values may grow by after the first pass
+  int sums;    // whether the scale uses the sum over the line
+  int radix[kFixMaxPass], span[kFixMaxPass], twoff[kFixMaxPass];
+};
 
 // ----------------------------------------------------------------------------
 // Helmholtz coefficient set for Algorithm 2 (one (c, loc, nparts) entry).
@@ -135,6 +143,11 @@ struct cfs_plan {
   double2* d_twx;    // fx twiddles
   double2* d_twy;    // fy twiddles
   double2* d_post;   // 0.5 * W_nx^k, k = 0..M/2 (real-FFT post-processing)
+  // block fixed-point FP64 transforms (lengths >= kFixMinLen): passes, and in one
+  // allocation the twiddles, W_nx^k for k < M (and conjugates) and, for walls in
+  // y, exp(-i pi k / 2 Ny) (and conjugates)
+  chanfs::FixDesc xfwd, xinv, yfwd, yinv;
+  int4 *d_fix, *d_xfwd, *d_xinv, *d_xpost, *d_xpost_inv, *d_yfwd, *d_yinv, *d_ywall, *d_ywall_inv;
   // y-tile geometry
   int tk;            // complex columns per y tile
   int by, nbox;      // rows per TMA box, boxes per tile
@@ -151,8 +164,8 @@ struct cfs_plan {
   int helm_thomas;   // FP64 Helmholtz solves by Thomas sweeps instead of Algorithm 2
   int helm_thomas32; // FP32 inner Helmholtz solves of refinement by Thomas sweeps
   int fft_radix;     // largest radix of the x and y FFT passes (8 or 4)
-  int emu_x, emu_y;  // FP64 x / y transforms: levels 0..4 of butterfly additions
-                     // on the integer units (CFS_OPT_F64_ADDS_X / _Y)
+  int emu_x, emu_y;  // CFS_OPT_F64_ADDS_X / _Y as set (no effect: the FP64 transforms
+                     // run on the integer units as a whole)
   double* d_dzf;     // cell widths (weights of the Neumann mean)
   // Neumann (0,0) column: wn = w/sum(w), gn = g/sum(w) with g = T'^{-T} w,
   // hs = sc * T'^{-1} (0,1,..,1), T' the pinned operator; 3*nz doubles
@@ -223,6 +236,10 @@ namespace chanfs {
 cudaError_t launch_rfft_x(const cfs_plan* P, const double* in, double* out, bool inverse,
                           double scale, cudaStream_t st, long long nlines = -1);
 cudaError_t launch_fft_y(const cfs_plan* P, double* data, bool inverse, cudaStream_t st);
+// The block fixed-point transforms behind them (lengths >= kFixMinLen).
+cudaError_t launch_fix_x(const cfs_plan* P, const double* in, double* out, bool inverse, double mul,
+                         cudaStream_t st, long long nlines);
+cudaError_t launch_fix_y(const cfs_plan* P, double* data, bool inverse, cudaStream_t st);
 cudaError_t launch_thomas(const cfs_plan* P, double* data, cudaStream_t st);
 cudaError_t launch_rfft_x32(const cfs_plan* P, const float* in, float* out, bool inverse,
                             cudaStream_t st);

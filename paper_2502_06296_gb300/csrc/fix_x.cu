@@ -1,0 +1,583 @@
+// fix_x.cu -- the FP64 real FFT along x in block fixed point (chanfs_fix.cuh),
+// packed output (App. A of the paper).
+//
+// A line of nx = 2M reals is M complex numbers; a thread takes one butterfly
+// of the first pass straight from global memory into registers and one pair of
+// mirrored butterflies of the last pass straight back, so that the line visits
+// shared memory only between passes.  The last forward pass (the first inverse
+// one) holds the butterflies i and Q - i together: their outputs (inputs) k
+// and M - k are the pairs that the real transform untangles,
+//   2 X_k = E - i W^k O,  2 X_{M-k} = conj(E + i W^k O),
+//   E = Z_k + conj Z_{M-k},  O = Z_k - conj Z_{M-k},  W = exp(-2 pi i / nx).
+// Item i = 0 holds the butterflies 0 and Q/2, whose pairs lie within each.
+// What bounds it: the integer ALU pipe (about 57 of its instructions per real
+// point: 21 in additions, 17 in the conversion from double, the rest in the
+// products' halves; 68 % busy in ncu at 24 warps per SM), against 13.75
+// instructions per point on an FP64 pipe 32 times narrower: 2.03 / 1.99 ms forward
+// / inverse in FP64 at 512 x 384 x 384 on GB300, 0.34 / 0.35 ms here (3.6 TB/s).
+// Common lengths are compiled with every radix, span and offset a constant;
+// with a power of two of items per line, at most 32, a warp owns its lines and
+// never waits for another.
+#include "chanfs_fix.cuh"
+
+namespace chanfs {
+
+// Pairs of item i: entry r is (p[r], q[r]) = (Z_k, Z_{M-k}), k = pair_index.
+template <int R>
+__device__ __forceinline__ void pair_take(bool zero, const Fix* a, const Fix* b, Fix* p, Fix* q) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    p[r] = a[r];
+    q[r] = b[R - 1 - r];
+  }
+  if (zero) {
+    if constexpr (R == 6) {
+      p[0] = q[0] = a[3];
+      q[1] = a[5];
+      q[2] = a[4];
+      p[3] = b[0];
+      q[3] = b[5];
+      p[4] = b[1];
+      q[4] = b[4];
+      p[5] = b[2];
+      q[5] = b[3];
+    } else if constexpr (R == 4) {
+      p[0] = q[0] = a[2];
+      q[1] = a[3];
+      p[2] = b[0];
+      q[2] = b[3];
+      p[3] = b[1];
+      q[3] = b[2];
+    } else if constexpr (R == 3) {
+      p[0] = q[0] = b[1];
+      q[1] = a[2];
+      p[2] = b[0];
+      q[2] = b[2];
+    } else {
+      p[0] = q[0] = a[1];
+      p[1] = b[0];
+      q[1] = b[1];
+    }
+  }
+}
+// The inverse of pair_take (a[0] of item 0 is set by the caller).
+template <int R>
+__device__ __forceinline__ void pair_give(bool zero, const Fix* p, const Fix* q, Fix* a, Fix* b) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    a[r] = p[r];
+    b[R - 1 - r] = q[r];
+  }
+  if (zero) {
+    if constexpr (R == 6) {
+      a[1] = p[1];
+      a[2] = p[2];
+      a[3] = p[0];
+      a[4] = q[2];
+      a[5] = q[1];
+      b[0] = p[3];
+      b[1] = p[4];
+      b[2] = p[5];
+      b[3] = q[5];
+      b[4] = q[4];
+      b[5] = q[3];
+    } else if constexpr (R == 4) {
+      a[1] = p[1];
+      a[2] = p[0];
+      a[3] = q[1];
+      b[0] = p[2];
+      b[1] = p[3];
+      b[2] = q[3];
+      b[3] = q[2];
+    } else if constexpr (R == 3) {
+      a[1] = p[1];
+      a[2] = q[1];
+      b[0] = p[2];
+      b[1] = p[0];
+      b[2] = q[2];
+    } else {
+      a[1] = p[0];
+      b[0] = p[1];
+      b[1] = q[1];
+    }
+  }
+}
+template <int R> __device__ __forceinline__ int pair_index(bool zero, int i, int r, int Q) {
+  if (!zero) return i + r * Q;
+  if constexpr (R == 6) return r == 0 ? 3 * Q : r <= 2 ? r * Q : Q / 2 + (r - 3) * Q;
+  if constexpr (R == 4) return r == 0 ? 2 * Q : r == 1 ? Q : r == 2 ? Q / 2 : Q / 2 + Q;
+  if constexpr (R == 3) return r == 0 ? Q + Q / 2 : r == 1 ? Q : Q / 2;
+  return r == 0 ? Q : Q / 2;
+}
+// Whether entry r of item 0 belongs to the butterfly Q/2 (absent if Q is odd).
+template <int R> __device__ __forceinline__ bool pair_second(int r) {
+  return R == 6 ? r >= 3 : R == 4 ? r >= 2 : R == 3 ? r != 1 : r == 1;
+}
+
+// What a group of G threads (a warp, or the CTA) works on.
+struct XGroup {
+  int lane, G;         // this thread among them
+  int nl;              // its lines
+  long long line0;     // the first one
+  long long nlines;    // lines of the field
+  int n, ps, headroom, growth;
+  int drop;            // 2^-drop: the passes' divisions by 4 (and the factor 2 of 2 X or 2 Z)
+  Fix *A, *B;          // two buffers of nl padded lines
+  unsigned *top, *most, *quanta;
+  FixScale* scale;
+};
+
+template <bool WARP> __device__ __forceinline__ void group_sync() {
+  if constexpr (WARP) __syncwarp();
+  else __syncthreads();
+}
+
+// The maxima over the T items of each line (item lane of the group in line lane
+// / T) of the values' magnitudes and of the butterflies' sums, and the sum of
+// their quanta: the same on every thread of a line.
+template <bool WARP, int T>
+__device__ __forceinline__ bool warp_lead(const XGroup& g) {  // a warp's items share a line
+  return T ? T % 32 == 0 : g.nl == 1;
+}
+template <bool WARP, int T>
+__device__ __forceinline__ void line_max(const XGroup& g, int l, bool on, unsigned& top,
+                                         unsigned& most) {
+  if constexpr (WARP && T == 32) {
+    top = __reduce_max_sync(~0u, top);
+    most = __reduce_max_sync(~0u, most);
+  } else if constexpr (WARP) {
+#pragma unroll
+    for (int o = 1; o < T; o *= 2) {
+      top = max(top, __shfl_xor_sync(~0u, top, o));
+      most = max(most, __shfl_xor_sync(~0u, most, o));
+    }
+  } else {
+    if (warp_lead<WARP, T>(g)) {
+      top = __reduce_max_sync(~0u, top);
+      most = __reduce_max_sync(~0u, most);
+      on = on && (g.lane & 31) == 0;
+    }
+    if (on) {
+      atomicMax(g.top + l, top);
+      atomicMax(g.most + l, most);
+    }
+    __syncthreads();
+    top = g.top[l];
+    most = g.most[l];
+  }
+}
+template <bool WARP, int T>
+__device__ __forceinline__ unsigned line_sum(const XGroup& g, int l, bool on, unsigned v) {
+  if constexpr (WARP && T == 32) {
+    return __reduce_add_sync(~0u, v);
+  } else if constexpr (WARP) {
+#pragma unroll
+    for (int o = 1; o < T; o *= 2) v += __shfl_xor_sync(~0u, v, o);
+    return v;
+  } else {
+    if (warp_lead<WARP, T>(g)) {
+      v = __reduce_add_sync(~0u, v);
+      on = on && (g.lane & 31) == 0;
+    }
+    if (on) atomicAdd(g.quanta + l, v);
+    __syncthreads();
+    return g.quanta[l];
+  }
+}
+
+// Item it of the first pass: forward, butterfly j of line l (R points j + r Q);
+// inverse, the pairs of item i (2 R points, and the point 0 of item 0).
+template <int R, bool INV, int NRAW>
+__device__ __forceinline__ void load_item(const double2* line, int n, int Q, int i, double2* raw,
+                                          unsigned& top, float& sum) {
+  if constexpr (!INV) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) raw[r] = line[i + r * Q];
+  } else {
+    const bool z = i == 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const bool have = !z || (Q & 1) == 0 || !pair_second<R>(r);
+      const int k = pair_index<R>(z, i, r, Q);
+      raw[2 * r] = have ? line[k] : make_double2(0.0, 0.0);
+      raw[2 * r + 1] = have ? line[n - k] : make_double2(0.0, 0.0);
+    }
+    raw[2 * R] = z ? line[0] : make_double2(0.0, 0.0);
+  }
+#pragma unroll
+  for (int r = 0; r < NRAW; ++r) {
+    fix_gather(raw[r].x, top, sum);
+    fix_gather(raw[r].y, top, sum);
+  }
+}
+
+// The first pass's arithmetic on a loaded item, written to buffer A.
+template <int R, bool INV>
+__device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, int Q, int i,
+                                           const double2* raw, FixScale f,
+                                           const int4* __restrict__ post) {
+  if constexpr (!INV) {
+    Fix v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = fix_from(raw[r], f);
+    fdft<R, false>(v);
+#pragma unroll
+    for (int r = 0; r < R; ++r) line[fix_pad(i * R + r)] = v[r];
+  } else {
+    const bool z = i == 0;
+    Fix a[R], b[R], p[R], q[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {  // 2 Z_k = E + i conj(W^k) T, T = X_k - conj X_{M-k}
+      const Fix xk = fix_from(raw[2 * r], f), xm = fix_from(raw[2 * r + 1], f);
+      const Fix e = {xk.x + xm.x, xk.y - xm.y};
+      const Fix u = fmul(Fix{xk.x - xm.x, xk.y + xm.y},
+                         __ldg(post + pair_index<R>(z, i, r, Q)));
+      p[r] = {e.x - u.y, e.y + u.x};
+      q[r] = {e.x + u.y, u.x - e.y};
+    }
+    pair_give<R>(z, p, q, a, b);
+    if (z) {
+      const Fix x0 = fix_from(raw[2 * R], f);  // (X_0, X_M)
+      a[0] = {x0.x + x0.y, x0.x - x0.y};
+    }
+    fdft<R, true>(a);
+    fdft<R, true>(b);
+    const int jb = z ? Q / 2 : Q - i;
+#pragma unroll
+    for (int r = 0; r < R; ++r) line[fix_pad(i * R + r)] = a[r];
+    if (!z || (Q & 1) == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) line[fix_pad(jb * R + r)] = b[r];
+    }
+  }
+}
+
+// The first pass of the group's lines.  ONE: at most one item per thread, kept
+// in registers from the scan of its magnitudes on; else every item is read
+// again for each step (its lines are in L1 or L2 by then).
+// (sums: whether the scale uses the sum over the line.  Inverse: the two
+// butterflies of an item are each bounded by twice its sum, one factor 2 of which
+// is in the headroom.)
+template <int R, bool INV, bool WARP, int T, bool ONE>
+__device__ __forceinline__ void first_pass(const XGroup& g, const double2* in, bool sums,
+                                           const int4* __restrict__ post) {
+  constexpr int NRAW = INV ? 2 * R + 1 : R;
+  const int Q = g.n / R;
+  const int per = T ? T : (INV ? (Q + 1) / 2 : Q);
+  const int items = g.nl * per;
+  const long long left = g.nlines - g.line0;
+  if constexpr (ONE) {
+    const int l = min(g.lane / per, g.nl - 1), i = g.lane - l * per;
+    const bool on = g.lane < items && l < left;
+    double2 raw[NRAW];
+    unsigned top = 0u;
+    float sum = 0.0f;
+    if (on) load_item<R, INV, NRAW>(in + (g.line0 + l) * g.n, g.n, Q, i, raw, top, sum);
+    if constexpr (!WARP) __syncthreads();  // the reduction's cells are cleared
+    unsigned most = __float_as_uint(sum), quanta = 0u;
+    line_max<WARP, T>(g, l, on, top, most);
+    if (sums)
+      quanta = line_sum<WARP, T>(g, l, on, on ? (INV ? 2u : 1u) * fix_quanta(sum, top, most) : 0u);
+    if (on) {
+      const FixScale f =
+          fix_scale_of(top, most, quanta, fix_ceil_log2(4 * R), g.growth, g.headroom);
+      if (i == 0) g.scale[l] = f;
+      first_item<R, INV>(g, g.A + l * g.ps, g.n, Q, i, raw, f, post);
+    }
+  } else {  // one line per CTA
+    double2 raw[NRAW];
+    __syncthreads();
+    for (int step = sums ? 0 : 1; step < 3; ++step) {
+      for (int base = 0; base < items; base += g.G) {
+        const int i = base + g.lane;
+        const bool on = i < items;
+        unsigned top = 0u;
+        float sum = 0.0f;
+        if (on) load_item<R, INV, NRAW>(in + g.line0 * g.n, g.n, Q, i, raw, top, sum);
+        if (step == (sums ? 0 : 1)) {
+          top = __reduce_max_sync(~0u, top);
+          const unsigned most = __reduce_max_sync(~0u, __float_as_uint(sum));
+          if ((g.lane & 31) == 0) {
+            atomicMax(g.top, top);
+            atomicMax(g.most, most);
+          }
+        } else if (step == 1) {
+          const unsigned q = __reduce_add_sync(
+              ~0u, on ? (INV ? 2u : 1u) * fix_quanta(sum, g.top[0], g.most[0]) : 0u);
+          if ((g.lane & 31) == 0) atomicAdd(g.quanta, q);
+        } else if (on) {
+          const FixScale f = fix_scale_of(g.top[0], g.most[0], g.quanta[0], fix_ceil_log2(4 * R),
+                                          g.growth, g.headroom);
+          if (i == 0) g.scale[0] = f;
+          first_item<R, INV>(g, g.A, g.n, Q, i, raw, f, post);
+        }
+      }
+      if (step < 2) __syncthreads();
+    }
+  }
+}
+
+// A middle pass over the group's lines, from one buffer to the other.
+template <int R, bool INV>
+__device__ __forceinline__ void middle_pass(const XGroup& g, const Fix* in, Fix* out, int L,
+                                            const int4* __restrict__ tw) {
+  const int Q = g.n / R, items = g.nl * Q;
+  for (int it = g.lane; it < items; it += g.G) {
+    const int l = it / Q, j = it - l * Q;
+    fix_butterfly<R, INV>(in + l * g.ps, out + l * g.ps, j, Q, L, tw,
+                          [](int e) { return fix_pad(e); });
+  }
+}
+
+// The last forward pass with the untangling: pairs to global memory.
+template <int R>
+__device__ __forceinline__ void last_forward(const XGroup& g, const Fix* in, double2* out,
+                                             const int4* __restrict__ tw,
+                                             const int4* __restrict__ post) {
+  const int n = g.n, Q = n / R, per = (Q + 1) / 2, items = g.nl * per;
+  const bool odd = Q & 1;
+  for (int it = g.lane; it < items; it += g.G) {
+    const int l = it / per, i = it - l * per;
+    if (g.line0 + l >= g.nlines) continue;
+    const bool z = i == 0;
+    const int jb = z ? Q / 2 : Q - i;
+    const Fix* x = in + l * g.ps;
+    Fix a[R], b[R], p[R], q[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      a[r] = x[fix_pad(i + r * Q)];
+      b[r] = x[fix_pad(jb + r * Q)];
+    }
+    fix_twiddle_dft<R, false>(a, tw + i, Q);
+    fix_twiddle_dft<R, false>(b, tw + jb, Q);
+    const FixScale f = g.scale[l];
+    const int sh = f.s - g.drop;
+    double2* o = out + (g.line0 + l) * n;
+    if (z) o[0] = fix_to(Fix{a[0].x + a[0].y, a[0].x - a[0].y}, sh - 1, f.kind);  // (X_0, X_M)
+    pair_take<R>(z, a, b, p, q);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (z && odd && pair_second<R>(r)) continue;
+      const int k = pair_index<R>(z, i, r, Q);
+      const Fix e = {p[r].x + q[r].x, p[r].y - q[r].y};
+      const Fix u = fmul(Fix{p[r].x - q[r].x, p[r].y + q[r].y}, __ldg(post + k));
+      o[k] = fix_to(Fix{e.x + u.y, e.y - u.x}, sh, f.kind);
+      if (n - k != k) o[n - k] = fix_to(Fix{e.x - u.y, -e.y - u.x}, sh, f.kind);
+    }
+  }
+}
+
+static __device__ __noinline__ double2 scaled_by(double2 z, double mul) {
+  return make_double2(z.x * mul, z.y * mul);
+}
+
+// The last inverse pass: plain butterflies to global memory.
+// (The factor `mul`, where a caller wants one, goes on last: its FP64 products
+// are kept out of the plain code, where they would be most of the FP64 work.)
+template <int R>
+__device__ __forceinline__ void last_inverse(const XGroup& g, const Fix* in, double2* out,
+                                             const int4* __restrict__ tw, double mul, int scaled) {
+  const int n = g.n, Q = n / R, items = g.nl * Q;
+  for (int it = g.lane; it < items; it += g.G) {
+    const int l = it / Q, j = it - l * Q;
+    if (g.line0 + l >= g.nlines) continue;
+    const Fix* x = in + l * g.ps;
+    Fix v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = x[fix_pad(j + r * Q)];
+    fix_twiddle_dft<R, true>(v, tw + j, Q);
+    const FixScale f = g.scale[l];
+    const int sh = f.s - g.drop;
+    double2* o = out + (g.line0 + l) * n;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      double2 z = fix_to(v[r], sh, f.kind);
+      if (scaled) z = scaled_by(z, mul);
+      o[j + r * Q] = z;
+    }
+  }
+}
+
+// Items per line of the first pass.
+template <bool INV> __host__ __device__ constexpr int x_items(int n) {
+  const int R = fix_rad<true, INV>(n, 0), Q = n / R;
+  return INV ? (Q + 1) / 2 : Q;
+}
+__host__ __device__ constexpr bool warp_lines(int items) {
+  return items <= 32 && (items & (items - 1)) == 0;
+}
+
+template <int N, bool INV, int P>
+__device__ __forceinline__ void fixed_middle(const XGroup& g, Fix* a, Fix* b, const int4* tw,
+                                             Fix** end) {
+  constexpr int NP = fix_npass<true>(N);
+  constexpr bool WARP = warp_lines(x_items<INV>(N));
+  if constexpr (P + 1 < NP) {
+    middle_pass<fix_rad<true, INV>(N, P), INV>(g, a, b, fix_span<true, INV>(N, P),
+                                               tw + fix_twoff<true, INV>(N, P));
+    group_sync<WARP>();
+    fixed_middle<N, INV, P + 1>(g, b, a, tw, end);
+  } else {
+    *end = a;
+  }
+}
+
+// N > 0: the compile-time length; N = 0: any length, from d.
+template <int N, bool INV, bool ONE>
+__global__ void __launch_bounds__(256, 2)
+    fix_x_kernel(const double2* in, double2* out, long long nlines, FixDesc d,
+                 const int4* __restrict__ tw, const int4* __restrict__ post, int lb, double mul,
+                 int scaled) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int T = N ? x_items<INV>(N ? N : 8) : 0;
+  constexpr bool WARP = N > 0 && warp_lines(T);
+  const int n = N ? N : d.n;
+  const int ps = n + (n >> 3);
+  XGroup g;
+  g.n = n;
+  g.ps = ps;
+  // forward: 2 X is up to 4 times a value of the last pass; inverse: a butterfly
+  // of 2 Z is up to twice its item's sum, and nothing follows the last pass
+  g.headroom = INV ? 61 : 60;
+  g.growth = N ? fix_growth<true, INV>(N ? N : 9) : d.growth;
+  g.nlines = nlines;
+  const int grp = WARP ? (int)(threadIdx.x >> 5) : 0;
+  g.nl = WARP ? 32 / (T ? T : 32) : lb;
+  g.lane = WARP ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  g.G = WARP ? 32 : (int)blockDim.x;
+  g.line0 = (long long)blockIdx.x * lb + grp * g.nl;
+  Fix* buf = reinterpret_cast<Fix*>(smem_raw);
+  g.A = buf + grp * g.nl * ps;
+  const int npass = N ? fix_npass<true>(N ? N : 8) : d.npass;
+  g.drop = 2 * (npass - 1) - 1;
+  g.B = g.A + (npass > 2 ? lb * ps : 0);
+  int* cells = reinterpret_cast<int*>(buf + (npass > 2 ? 2 : 1) * lb * ps);
+  g.scale = reinterpret_cast<FixScale*>(cells) + grp * g.nl;
+  g.top = reinterpret_cast<unsigned*>(cells + 2 * lb);
+  g.most = g.top + lb;
+  g.quanta = g.most + lb;
+  if constexpr (!WARP)
+    for (int e = threadIdx.x; e < 3 * lb; e += blockDim.x) g.top[e] = 0u;
+  if constexpr (N > 0) {
+    first_pass<fix_rad<true, INV>(N, 0), INV, WARP, T, true>(g, in, fix_uses_sum<true, INV>(N),
+                                                              post);
+    group_sync<WARP>();
+    Fix* end;
+    fixed_middle<N, INV, 1>(g, g.A, g.B, tw, &end);
+    constexpr int PL = fix_npass<true>(N) - 1;
+    if constexpr (INV)
+      last_inverse<fix_rad<true, true>(N, PL)>(g, end, out, tw + fix_twoff<true, true>(N, PL),
+                                               mul, scaled);
+    else
+      last_forward<fix_rad<true, false>(N, PL)>(g, end, out, tw + fix_twoff<true, false>(N, PL),
+                                                post);
+  } else {
+    switch (d.radix[0]) {
+      case 8:
+        if constexpr (!INV) first_pass<8, INV, false, 0, ONE>(g, in, d.sums, post);
+        break;
+      case 6: first_pass<6, INV, false, 0, ONE>(g, in, d.sums, post); break;
+      case 4: first_pass<4, INV, false, 0, ONE>(g, in, d.sums, post); break;
+      case 3: first_pass<3, INV, false, 0, ONE>(g, in, d.sums, post); break;
+      default: first_pass<2, INV, false, 0, ONE>(g, in, d.sums, post); break;
+    }
+    __syncthreads();
+    Fix *a = g.A, *b = g.B;
+    for (int p = 1; p + 1 < npass; ++p) {
+      const int L = d.span[p];
+      const int4* t = tw + d.twoff[p];
+      switch (d.radix[p]) {
+        case 8: middle_pass<8, INV>(g, a, b, L, t); break;
+        case 6: middle_pass<6, INV>(g, a, b, L, t); break;
+        case 4: middle_pass<4, INV>(g, a, b, L, t); break;
+        case 3: middle_pass<3, INV>(g, a, b, L, t); break;
+        default: middle_pass<2, INV>(g, a, b, L, t); break;
+      }
+      __syncthreads();
+      Fix* s = a;
+      a = b;
+      b = s;
+    }
+    const int4* t = tw + d.twoff[npass - 1];
+    switch (d.radix[npass - 1]) {
+      case 8:
+        if constexpr (INV) last_inverse<8>(g, a, out, t, mul, scaled);
+        break;
+      case 6:
+        if constexpr (INV) last_inverse<6>(g, a, out, t, mul, scaled);
+        else last_forward<6>(g, a, out, t, post);
+        break;
+      case 4:
+        if constexpr (INV) last_inverse<4>(g, a, out, t, mul, scaled);
+        else last_forward<4>(g, a, out, t, post);
+        break;
+      case 3:
+        if constexpr (INV) last_inverse<3>(g, a, out, t, mul, scaled);
+        else last_forward<3>(g, a, out, t, post);
+        break;
+      default:
+        if constexpr (INV) last_inverse<2>(g, a, out, t, mul, scaled);
+        else last_forward<2>(g, a, out, t, post);
+        break;
+    }
+  }
+}
+
+template <int N, bool INV, bool ONE>
+static cudaError_t go(const cfs_plan* P, const double* in, double* out, double mul, long long nl,
+                      int threads, int lb, cudaStream_t st) {
+  const FixDesc& d = INV ? P->xinv : P->xfwd;
+  const int n = P->M;
+  const size_t smem = (size_t)(d.npass > 2 ? 2 : 1) * lb * (n + (n >> 3)) * sizeof(Fix) +
+                      (size_t)lb * 5 * sizeof(int);
+  auto k = fix_x_kernel<N, INV, ONE>;
+  allow_max_smem(k);
+  k<<<(unsigned)((nl + lb - 1) / lb), threads, smem, st>>>(
+      reinterpret_cast<const double2*>(in), reinterpret_cast<double2*>(out), nl, d,
+      INV ? P->d_xinv : P->d_xfwd, INV ? P->d_xpost_inv : P->d_xpost, lb, mul, mul != 1.0);
+  return cudaGetLastError();
+}
+
+template <int N, bool INV>
+static cudaError_t go_fixed(const cfs_plan* P, const double* in, double* out, double mul,
+                            long long nl, cudaStream_t st) {
+  constexpr int T = x_items<INV>(N);
+  if constexpr (warp_lines(T)) {
+    return go<N, INV, true>(P, in, out, mul, nl, 128, 4 * (32 / T), st);
+  } else {
+    constexpr int lb = T >= 192 ? 1 : 192 / T;
+    return go<N, INV, true>(P, in, out, mul, nl, (lb * T + 31) / 32 * 32, lb, st);
+  }
+}
+
+template <bool INV>
+static cudaError_t dispatch(const cfs_plan* P, const double* in, double* out, double mul,
+                            long long nl, cudaStream_t st) {
+  switch (P->M) {
+    case 32: return go_fixed<32, INV>(P, in, out, mul, nl, st);
+    case 64: return go_fixed<64, INV>(P, in, out, mul, nl, st);
+    case 96: return go_fixed<96, INV>(P, in, out, mul, nl, st);
+    case 128: return go_fixed<128, INV>(P, in, out, mul, nl, st);
+    case 192: return go_fixed<192, INV>(P, in, out, mul, nl, st);
+    case 256: return go_fixed<256, INV>(P, in, out, mul, nl, st);
+    case 384: return go_fixed<384, INV>(P, in, out, mul, nl, st);
+    case 512: return go_fixed<512, INV>(P, in, out, mul, nl, st);
+    default: break;
+  }
+  const int T = x_items<INV>(P->M);
+  if (T <= 256) {
+    const int lb = T >= 192 ? 1 : 192 / T;
+    return go<0, INV, true>(P, in, out, mul, nl, (lb * T + 31) / 32 * 32, lb, st);
+  }
+  return go<0, INV, false>(P, in, out, mul, nl, 256, 1, st);
+}
+
+cudaError_t launch_fix_x(const cfs_plan* P, const double* in, double* out, bool inverse, double mul,
+                         cudaStream_t st, long long nlines) {
+  if (nlines < 0) nlines = (long long)P->ny * P->nz;
+  if (nlines == 0) return cudaSuccess;
+  return inverse ? dispatch<true>(P, in, out, mul, nlines, st)
+                 : dispatch<false>(P, in, out, mul, nlines, st);
+}
+
+}  // namespace chanfs

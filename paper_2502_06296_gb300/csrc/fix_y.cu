@@ -1,0 +1,418 @@
+// fix_y.cu -- the FP64 complex FFT along y in block fixed point
+// (chanfs_fix.cuh), and the cosine / sine transforms of walls in y on top of it.
+//
+// A CTA takes tk neighbouring complex columns of one z plane (rows of 16 tk
+// contiguous bytes; consecutive threads on consecutive columns), every column
+// with its own scale.  The first pass reads its butterflies from global memory
+// into registers, the last one writes them back, so a tile visits shared
+// memory only between passes.  512 x 384 x 384 on GB300: 1.70 ms in FP64 on TMA
+// tiles (bound by the FP64 pipe), 0.46 ms here (2.6 TB/s), bound by the integer
+// ALU pipe and by the barriers between the passes of a tile.
+#include "chanfs_fix.cuh"
+
+namespace chanfs {
+
+struct YTile {
+  double2* col;    // column 0 of the tile, row 0 of the plane
+  int M;           // columns of the field (row stride)
+  int valid;       // columns of this tile inside it
+  int tk, sh;      // columns of the tile (a power of two), its logarithm
+  int n, headroom, growth, lgpts;
+  int drop;        // 2^-drop: the passes' divisions by 4
+  bool first;      // the tile holds the packed column kx = 0
+  Fix *A, *B;
+  unsigned *top, *most, *quanta;
+};
+
+__device__ __forceinline__ FixScale scale_of(const YTile& t, int c) {
+  return fix_scale_of(t.top[c], t.most[c], t.quanta[c], t.lgpts, t.growth, t.headroom);
+}
+
+// Rows of a wall transform: element t of the FFT is row wall_row(t).
+__device__ __forceinline__ int wall_row(int t, int n) {
+  return t < (n + 1) / 2 ? 2 * t : 2 * (n - 1 - t) + 1;
+}
+
+enum { kPeriodic = 0, kCos = 1, kSin = 2 };
+
+// Element e of column c of the first pass's input.
+template <bool INV, bool WALL>
+__device__ __forceinline__ double2 load_elem(const YTile& t, int e, int c, int ytype) {
+  const double2* p = t.col + c;
+  if constexpr (WALL && !INV) {
+    const int j = wall_row(e, t.n);
+    double2 v = p[(size_t)j * t.M];
+    if (ytype == kSin && (j & 1)) v = make_double2(-v.x, -v.y);
+    return v;
+  } else if constexpr (WALL) {
+    return p[(size_t)(ytype == kSin ? t.n - 1 - e : e) * t.M];  // X_e
+  } else {
+    return p[(size_t)e * t.M];
+  }
+}
+
+// The packed column kx = 0 is stored untangled (slot ky holds F(0, ky), slot Ny -
+// ky holds F(Nx/2, ky)): Z_ky = F0 + i FM, Z_{Ny-ky} = conj F0 + i conj FM.
+__device__ __forceinline__ double2 load_packed(const YTile& t, int e) {
+  const int n = t.n;
+  const double2 v = t.col[(size_t)e * t.M];
+  if (e == 0 || 2 * e == n) return v;
+  const double2 w = t.col[(size_t)(n - e) * t.M];
+  return 2 * e < n ? make_double2(v.x - w.y, v.y + w.x) : make_double2(w.x + v.y, v.x - w.y);
+}
+
+template <int R, bool INV, bool WALL>
+__device__ __forceinline__ void load_points(const YTile& t, int j, int c, int ytype, double2* raw,
+                                            unsigned& top, float& sum) {
+  const int Q = t.n / R;
+  if (INV && !WALL && t.first && c == 0) {
+    for (int r = 0; r < R; ++r) raw[r] = load_packed(t, j + r * Q);
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) raw[r] = load_elem<INV, WALL>(t, j + r * Q, c, ytype);
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    fix_gather(raw[r].x, top, sum);
+    fix_gather(raw[r].y, top, sum);
+  }
+}
+
+// V_e of the inverse wall transform from its column's X: conj(w_e) (X_e - i
+// X_{N-e}), w_e = exp(-i pi e / 2N); V_0 = X_0.  (Points past the middle: w_m
+// (X_e + ... ) with m = N - e, the same formula.)
+__device__ __forceinline__ Fix wall_unmix(Fix xe, Fix xn, int4 wconj) {
+  return fmul(Fix{xe.x + xn.y, xe.y - xn.x}, wconj);
+}
+
+template <int R, bool INV, bool WALL>
+__device__ __forceinline__ void first_points(const YTile& t, int j, int c, int ytype,
+                                             const double2* raw, FixScale f,
+                                             const int4* __restrict__ wy) {
+  const int Q = t.n / R;
+  Fix v[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    v[r] = fix_from(raw[r], f);
+    if constexpr (INV && WALL) {
+      const int e = j + r * Q;
+      if (e > 0) {
+        const Fix xn = fix_from(load_elem<INV, WALL>(t, t.n - e, c, ytype), f);
+        v[r] = wall_unmix(v[r], xn, __ldg(wy + e));
+      }
+    }
+  }
+  fdft<R, INV>(v);
+#pragma unroll
+  for (int r = 0; r < R; ++r) t.A[fix_pad(((j * R + r) << t.sh) + c)] = v[r];
+}
+
+// The first pass of a tile (see fix_x.cu: ONE keeps a thread's one item in
+// registers; otherwise each step reads it again).
+template <int R, bool INV, bool WALL, bool ONE>
+__device__ __forceinline__ void first_pass(const YTile& t, int ytype, bool sums,
+                                           const int4* __restrict__ wy) {
+  const int items = (t.n / R) << t.sh;
+  if constexpr (ONE) {
+    const int it = threadIdx.x, c = it & (t.tk - 1), j = it >> t.sh;
+    const bool on = it < items && c < t.valid;
+    double2 raw[R];
+    unsigned top = 0u;
+    float sum = 0.0f;
+    if (on) load_points<R, INV, WALL>(t, j, c, ytype, raw, top, sum);
+    __syncthreads();  // the reduction's cells are cleared
+    unsigned most = __float_as_uint(sum);
+    const bool lead = (threadIdx.x & 31) < t.tk;
+    for (int o = t.tk; o < 32; o *= 2) {
+      top = max(top, __shfl_xor_sync(~0u, top, o));
+      most = max(most, __shfl_xor_sync(~0u, most, o));
+    }
+    if (lead) {
+      atomicMax(t.top + c, top);
+      atomicMax(t.most + c, most);
+    }
+    __syncthreads();
+    if (sums) {
+      unsigned q = on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
+      for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
+      if (lead) atomicAdd(t.quanta + c, q);
+      __syncthreads();
+    }
+    if (on) first_points<R, INV, WALL>(t, j, c, ytype, raw, scale_of(t, c), wy);
+  } else {
+    __syncthreads();
+    for (int step = sums ? 0 : 1; step < 3; ++step) {
+      for (int base = 0; base < items; base += blockDim.x) {
+        const int it = base + threadIdx.x, c = it & (t.tk - 1), j = it >> t.sh;
+        const bool on = it < items && c < t.valid, lead = (threadIdx.x & 31) < t.tk;
+        double2 raw[R];
+        unsigned top = 0u;
+        float sum = 0.0f;
+        if (on) load_points<R, INV, WALL>(t, j, c, ytype, raw, top, sum);
+        if (step == (sums ? 0 : 1)) {
+          unsigned most = __float_as_uint(sum);
+          for (int o = t.tk; o < 32; o *= 2) {
+            top = max(top, __shfl_xor_sync(~0u, top, o));
+            most = max(most, __shfl_xor_sync(~0u, most, o));
+          }
+          if (lead) {
+            atomicMax(t.top + c, top);
+            atomicMax(t.most + c, most);
+          }
+        } else if (step == 1) {
+          unsigned q = on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
+          for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
+          if (lead) atomicAdd(t.quanta + c, q);
+        } else if (on) {
+          first_points<R, INV, WALL>(t, j, c, ytype, raw, scale_of(t, c), wy);
+        }
+      }
+      if (step < 2) __syncthreads();
+    }
+  }
+}
+
+template <int R, bool INV>
+__device__ __forceinline__ void middle_pass(const YTile& t, const Fix* in, Fix* out, int L,
+                                            const int4* __restrict__ tw) {
+  const int Q = t.n / R, items = Q << t.sh;
+  for (int it = threadIdx.x; it < items; it += blockDim.x) {
+    const int c = it & (t.tk - 1), j = it >> t.sh;
+    const int sh = t.sh;
+    fix_butterfly<R, INV>(in, out, j, Q, L, tw, [=](int e) { return fix_pad((e << sh) + c); });
+  }
+}
+
+// The last pass: plain columns to global memory.  A forward wall transform
+// leaves every column in shared memory for the mixing pass, the tile of the
+// packed column leaves that one.
+template <int R, bool INV, bool WALL>
+__device__ __forceinline__ void last_pass(const YTile& t, const Fix* in, Fix* keep, int ytype,
+                                          const int4* __restrict__ tw) {
+  const int n = t.n, Q = n / R, items = Q << t.sh;
+  for (int it = threadIdx.x; it < items; it += blockDim.x) {
+    const int c = it & (t.tk - 1), j = it >> t.sh;
+    if (c >= t.valid) continue;
+    Fix v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = in[fix_pad(((j + r * Q) << t.sh) + c)];
+    fix_twiddle_dft<R, INV>(v, tw + j, Q);
+    if (!INV && (WALL || (t.first && c == 0))) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) keep[fix_pad(((j + r * Q) << t.sh) + c)] = v[r];
+    } else {
+      const FixScale f = scale_of(t, c);
+      double2* o = t.col + c;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int e = j + r * Q;
+        double2 z = fix_to(v[r], f.s - t.drop, f.kind);
+        int row = e;
+        if constexpr (WALL) {
+          row = wall_row(e, n);
+          if (ytype == kSin && (row & 1)) z = make_double2(-z.x, -z.y);
+        }
+        o[(size_t)row * t.M] = z;
+      }
+    }
+  }
+}
+
+// The forward wall transform from V: with A = w_k V_k, B = conj(w_k) V_{N-k},
+// 2 X_k = A + B and 2 X_{N-k} = i (A - B); X_0 = V_0.
+__device__ __forceinline__ void wall_mix(const YTile& t, const Fix* in, int ytype,
+                                         const int4* __restrict__ wy) {
+  const int n = t.n, items = (n / 2 + 1) << t.sh;
+  for (int it = threadIdx.x; it < items; it += blockDim.x) {
+    const int c = it & (t.tk - 1), k = it >> t.sh;
+    if (c >= t.valid) continue;
+    const FixScale f = scale_of(t, c);
+    double2* o = t.col + c;
+    const auto slot = [&](int e) { return (size_t)(ytype == kSin ? n - 1 - e : e) * t.M; };
+    const Fix vk = in[fix_pad((k << t.sh) + c)];
+    if (k == 0) {
+      o[slot(0)] = fix_to(vk, f.s - t.drop, f.kind);
+      continue;
+    }
+    const int4 w = __ldg(wy + k);
+    const Fix a = fmul(vk, w);
+    const Fix b = fmul(in[fix_pad(((n - k) << t.sh) + c)], make_int4(w.x, w.y, -w.z, -w.w));
+    o[slot(k)] = fix_to(fadd(a, b), f.s - t.drop + 1, f.kind);
+    if (n - k != k) o[slot(n - k)] = fix_to(Fix{b.y - a.y, a.x - b.x}, f.s - t.drop + 1, f.kind);
+  }
+}
+
+// The packed column kx = 0 of the forward transform: slot ky (0 < 2 ky < Ny)
+// takes F(0, ky) = (Z_ky + conj Z_{Ny-ky}) / 2, slot Ny - ky takes F(Nx/2, ky)
+// = -i (Z_ky - conj Z_{Ny-ky}) / 2; the self-conjugate slots keep the pair.
+__device__ __forceinline__ void untangle_column(const YTile& t, const Fix* in) {
+  const int n = t.n;
+  const FixScale f = scale_of(t, 0);
+  for (int k = threadIdx.x; 2 * k <= n; k += blockDim.x) {
+    const Fix z = in[fix_pad(k << t.sh)];
+    if (k == 0 || 2 * k == n) {
+      t.col[(size_t)k * t.M] = fix_to(z, f.s - t.drop, f.kind);
+      continue;
+    }
+    const Fix m = in[fix_pad((n - k) << t.sh)];
+    t.col[(size_t)k * t.M] = fix_to(Fix{z.x + m.x, z.y - m.y}, f.s - t.drop + 1, f.kind);
+    t.col[(size_t)(n - k) * t.M] = fix_to(Fix{z.y + m.y, m.x - z.x}, f.s - t.drop + 1, f.kind);
+  }
+}
+
+template <int N, bool INV, int P>
+__device__ __forceinline__ void fixed_middle(const YTile& t, Fix* a, Fix* b, const int4* tw,
+                                             Fix** end) {
+  if constexpr (P + 1 < fix_npass<false>(N)) {
+    middle_pass<fix_rad<false, INV>(N, P), INV>(t, a, b, fix_span<false, INV>(N, P),
+                                                tw + fix_twoff<false, INV>(N, P));
+    __syncthreads();
+    fixed_middle<N, INV, P + 1>(t, b, a, tw, end);
+  } else {
+    *end = a;
+  }
+}
+
+// Columns per tile (a power of two, as its logarithm): 8, rows of 128 bytes,
+// while the first pass's items (`items` per column) fit 256 threads, else 4 or 2.
+__host__ __device__ constexpr int y_shift(int items) {
+  int sh = 3;
+  while (sh > 1 && (items << sh) > 256) --sh;
+  return sh;
+}
+constexpr int y_threads(int n) {
+  const int items = n / fix_radix<false>(n, 0);
+  return ((items << y_shift(items)) + 31) / 32 * 32;
+}
+
+// N > 0: the compile-time length (periodic y); N = 0: any length, from d.  The
+// fixed lengths ask for 24 warps per SM (80 registers).
+template <int N, bool INV, bool WALL, bool ONE>
+__global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : ONE ? 256 : 512,
+                                  N ? 768 / y_threads(N ? N : 9) : ONE ? 2 : 1)
+    fix_y_kernel(double2* data, int M, FixDesc d, const int4* __restrict__ tw,
+                 const int4* __restrict__ wy, int shift, int ytype) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n = N ? N : d.n;
+  const int npass = N ? fix_npass<false>(N ? N : 8) : d.npass;
+  const int sh = N ? y_shift((N ? N : 9) / fix_radix<false>(N ? N : 9, 0)) : shift;
+  YTile t;
+  t.n = n;
+  t.M = M;
+  t.sh = sh;
+  t.tk = 1 << sh;
+  const int x0 = blockIdx.x << sh;
+  t.valid = min(t.tk, M - x0);
+  t.first = x0 == 0;
+  t.col = data + (size_t)blockIdx.y * n * M + x0;
+  // (an inverse wall transform's V_e is up to |X_e| + |X_{N-e}|)
+  t.headroom = INV && WALL ? 60 : 61;
+  t.growth = N ? fix_growth<false, INV>(N ? N : 9) : d.growth;
+  t.lgpts = fix_ceil_log2(4 * (N ? fix_rad<false, INV>(N ? N : 9, 0) : d.radix[0]));
+  t.drop = 2 * (npass - 1);
+  const int pts = n << sh, buf = pts + (pts >> 3);
+  t.A = reinterpret_cast<Fix*>(smem_raw);
+  t.B = t.A + buf;
+  t.top = reinterpret_cast<unsigned*>(t.B + buf);
+  t.most = t.top + t.tk;
+  t.quanta = t.most + t.tk;
+  for (int e = threadIdx.x; e < 3 * t.tk; e += blockDim.x) t.top[e] = 0u;
+  Fix *a = t.A, *b = t.B;
+  if constexpr (N > 0) {
+    first_pass<fix_rad<false, INV>(N, 0), INV, false, true>(t, ytype, fix_uses_sum<false, INV>(N),
+                                                             wy);
+    __syncthreads();
+    fixed_middle<N, INV, 1>(t, t.A, t.B, tw, &a);
+    b = a == t.A ? t.B : t.A;
+    constexpr int PL = fix_npass<false>(N) - 1;
+    last_pass<fix_rad<false, INV>(N, PL), INV, false>(t, a, b, ytype,
+                                                      tw + fix_twoff<false, INV>(N, PL));
+  } else {
+    switch (d.radix[0]) {
+      case 8: first_pass<8, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
+      case 6: first_pass<6, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
+      case 4: first_pass<4, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
+      case 3: first_pass<3, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
+      default: first_pass<2, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
+    }
+    __syncthreads();
+    for (int p = 1; p + 1 < npass; ++p) {
+      const int L = d.span[p];
+      const int4* w = tw + d.twoff[p];
+      switch (d.radix[p]) {
+        case 8: middle_pass<8, INV>(t, a, b, L, w); break;
+        case 6: middle_pass<6, INV>(t, a, b, L, w); break;
+        case 4: middle_pass<4, INV>(t, a, b, L, w); break;
+        case 3: middle_pass<3, INV>(t, a, b, L, w); break;
+        default: middle_pass<2, INV>(t, a, b, L, w); break;
+      }
+      __syncthreads();
+      Fix* s = a;
+      a = b;
+      b = s;
+    }
+    const int4* w = tw + d.twoff[npass - 1];
+    switch (d.radix[npass - 1]) {
+      case 8: last_pass<8, INV, WALL>(t, a, b, ytype, w); break;
+      case 6: last_pass<6, INV, WALL>(t, a, b, ytype, w); break;
+      case 4: last_pass<4, INV, WALL>(t, a, b, ytype, w); break;
+      case 3: last_pass<3, INV, WALL>(t, a, b, ytype, w); break;
+      default: last_pass<2, INV, WALL>(t, a, b, ytype, w); break;
+    }
+  }
+  if constexpr (!INV) {
+    if (WALL || t.first) {
+      __syncthreads();
+      if constexpr (WALL) wall_mix(t, b, ytype, wy);
+      else untangle_column(t, b);
+    }
+  }
+}
+
+static size_t y_smem(int n, int sh) {
+  const size_t pts = (size_t)n << sh;
+  return 2 * (pts + (pts >> 3)) * sizeof(Fix) + ((size_t)3 << sh) * sizeof(unsigned);
+}
+
+template <int N, bool INV, bool WALL, bool ONE>
+static cudaError_t go(const cfs_plan* P, double* data, int sh, int threads, cudaStream_t st) {
+  auto k = fix_y_kernel<N, INV, WALL, ONE>;
+  allow_max_smem(k);
+  const dim3 grid((P->M + (1 << sh) - 1) >> sh, P->nz);
+  k<<<grid, threads, y_smem(P->ny, sh), st>>>(
+      reinterpret_cast<double2*>(data), P->M, INV ? P->yinv : P->yfwd, INV ? P->d_yinv : P->d_yfwd,
+      INV ? P->d_ywall_inv : P->d_ywall, sh, P->ybc);
+  return cudaGetLastError();
+}
+
+template <bool INV, bool WALL>
+static cudaError_t dispatch(const cfs_plan* P, double* data, cudaStream_t st) {
+  const int n = P->ny;
+  const int T = n / (INV ? P->yinv : P->yfwd).radix[0];  // items per column
+  int sh = y_shift(T);
+  while (sh > 0 && y_smem(n, sh) > kMaxDynSmem) --sh;
+  const int threads = ((T << sh) + 31) / 32 * 32;
+  if (threads > 256) return go<0, INV, WALL, false>(P, data, sh, 512, st);
+  if constexpr (!WALL) {
+    switch (n) {
+      case 64: return go<64, INV, false, true>(P, data, sh, threads, st);
+      case 96: return go<96, INV, false, true>(P, data, sh, threads, st);
+      case 128: return go<128, INV, false, true>(P, data, sh, threads, st);
+      case 192: return go<192, INV, false, true>(P, data, sh, threads, st);
+      case 256: return go<256, INV, false, true>(P, data, sh, threads, st);
+      case 384: return go<384, INV, false, true>(P, data, sh, threads, st);
+      case 512: return go<512, INV, false, true>(P, data, sh, threads, st);
+      case 768: return go<768, INV, false, true>(P, data, sh, threads, st);
+      default: break;
+    }
+  }
+  return go<0, INV, WALL, true>(P, data, sh, threads, st);
+}
+
+cudaError_t launch_fix_y(const cfs_plan* P, double* data, bool inverse, cudaStream_t st) {
+  if (P->ybc == CFS_Y_PERIODIC)
+    return inverse ? dispatch<true, false>(P, data, st) : dispatch<false, false>(P, data, st);
+  return inverse ? dispatch<true, true>(P, data, st) : dispatch<false, true>(P, data, st);
+}
+
+}  // namespace chanfs

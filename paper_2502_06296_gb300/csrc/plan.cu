@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "chanfs_alg2.cuh"
+#include "chanfs_fix.cuh"
 #include "chanfs_internal.cuh"
 
 using namespace chanfs;
@@ -53,6 +54,69 @@ bool make_fft_desc(int n, FftDesc* d, std::vector<double2>* tw, int max_radix) {
   d->ntw = (int)tw->size();
   if (tw->empty()) tw->push_back(make_double2(1.0, 0.0));  // keep a valid pointer
   return true;
+}
+
+// exp(-+2 pi i e / n) in units of 2^-62, the low words signed.  The values of
+// an eighth of the circle are computed once, in long double; the others are
+// their reflections.
+class FixRoots {
+ public:
+  explicit FixRoots(int n) : n_(n) {
+    const long double half_pi = 1.57079632679489661923132169163975144L;
+    for (int r = 0; 2 * r <= n; r += 4) add(half_pi * (long double)r / (long double)n);
+    if (n % 4) {  // the remainders of 4 e / n run over more than multiples of 4
+      cs_.clear();
+      for (int r = 0; 2 * r <= n; ++r) add(half_pi * (long double)r / (long double)n);
+    }
+  }
+  int4 at(long long e, bool conj) const {
+    e %= n_;
+    const long long q = 4 * e / n_, rest = 4 * e - q * n_;  // quarter turns, rest / n of the next
+    const bool swap = 2 * rest > n_;
+    const long long i = swap ? n_ - rest : rest;
+    const longlong2 cs = cs_[n_ % 4 ? i : i / 4];
+    const long long u = swap ? cs.y : cs.x, v = swap ? cs.x : cs.y;
+    const long long re = q == 0 ? u : q == 1 ? -v : q == 2 ? -u : v;
+    const long long im = q == 0 ? v : q == 1 ? u : q == 2 ? -v : -u;  // e^{+i angle}
+    int4 w;
+    split(re, &w.x, &w.y);
+    split(conj ? im : -im, &w.z, &w.w);
+    return w;
+  }
+
+ private:
+  void add(long double a) {
+    cs_.push_back(make_longlong2(llroundl(cosl(a) * 4611686018427387904.0L),
+                                 llroundl(sinl(a) * 4611686018427387904.0L)));
+  }
+  static void split(long long x, int* hi, int* lo) {
+    long long l = (long long)(int)(x & 0xffffffffll);
+    if (l == -2147483648ll) l = -2147483647ll;  // its negative is used too
+    *hi = (int)((x - l) >> 32);
+    *lo = (int)l;
+  }
+  long long n_;
+  std::vector<longlong2> cs_;
+};
+
+// Passes of a block fixed-point transform, and its twiddles appended to tw.
+// (roots: of a multiple of n)
+template <bool PAIR, bool INV>
+static void make_fix_desc(int n, FixDesc* d, std::vector<int4>* tw, const FixRoots& roots,
+                          int total) {
+  memset(d, 0, sizeof(*d));
+  d->n = n;
+  d->npass = fix_npass<PAIR>(n);
+  d->growth = fix_growth<PAIR, INV>(n);
+  d->sums = fix_uses_sum<PAIR, INV>(n);
+  for (int p = 0; p < d->npass; ++p) {
+    const int R = d->radix[p] = fix_rad<PAIR, INV>(n, p);
+    const int L = d->span[p] = fix_span<PAIR, INV>(n, p);
+    d->twoff[p] = fix_twoff<PAIR, INV>(n, p);
+    for (int r = 1; r < R; ++r)
+      for (int k = 0; k < L; ++k)
+        tw->push_back(roots.at((long long)r * k * (total / (L * R)), INV));
+  }
 }
 
 }  // namespace chanfs
@@ -166,6 +230,7 @@ static void plan_free(cfs_plan* P) {
   cudaFree(P->d_twx);
   cudaFree(P->d_twy);
   cudaFree(P->d_post);
+  cudaFree(P->d_fix);
   cudaFree(P->d_dzf);
   cudaFree(P->d_sing);
   cudaFree(P->d_stage);
@@ -278,8 +343,6 @@ extern "C" int cfs_plan_create_walls(cfs_plan_t* out, int nx, int ny, int nz, do
 
   std::vector<double2> twx, twy;
   P->fft_radix = 8;
-  P->emu_x = kEmuDefaultX;
-  P->emu_y = kEmuDefaultY;
   if (!make_fft_desc(P->M, &P->fx, &twx, 8) || !make_fft_desc(ny, &P->fy, &twy, 8)) {
     plan_free(P);
     return CFS_EUNSUPPORTED;
@@ -306,6 +369,32 @@ extern "C" int cfs_plan_create_walls(cfs_plan_t* out, int nx, int ny, int nz, do
   std::vector<double2> wy;
   if (ybc != CFS_Y_PERIODIC)
     for (int k = 0; k < ny; ++k) wy.push_back(chanfs::root(k, 4 * ny));
+  // the block fixed-point transforms' tables, one upload
+  std::vector<int4> fix;
+  size_t fix_at[8] = {};
+  if (P->M >= kFixMinLen) {
+    const FixRoots roots(nx);
+    fix_at[0] = fix.size();
+    make_fix_desc<true, false>(P->M, &P->xfwd, &fix, roots, nx);
+    fix_at[1] = fix.size();
+    make_fix_desc<true, true>(P->M, &P->xinv, &fix, roots, nx);
+    for (int inv = 0; inv < 2; ++inv) {
+      fix_at[2 + inv] = fix.size();
+      for (int k = 0; k < P->M; ++k) fix.push_back(roots.at(k, inv));
+    }
+  }
+  if (ny >= kFixMinLen) {
+    const int total = ybc == CFS_Y_PERIODIC ? ny : 4 * ny;
+    const FixRoots roots(total);
+    fix_at[4] = fix.size();
+    make_fix_desc<false, false>(ny, &P->yfwd, &fix, roots, total);
+    fix_at[5] = fix.size();
+    make_fix_desc<false, true>(ny, &P->yinv, &fix, roots, total);
+    for (int inv = 0; inv < 2 && ybc != CFS_Y_PERIODIC; ++inv) {
+      fix_at[6 + inv] = fix.size();
+      for (int k = 0; k < ny; ++k) fix.push_back(roots.at(k, inv));
+    }
+  }
   P->lamx_h = lamx;
   P->lamy_h = lamy;
   std::vector<double> A, B, C;
@@ -366,6 +455,23 @@ extern "C" int cfs_plan_create_walls(cfs_plan_t* out, int nx, int ny, int nz, do
   if (!rc) rc = dev_upload(&P->d_twx, twx.data(), twx.size(), &P->device_bytes);
   if (!rc) rc = dev_upload(&P->d_twy, twy.data(), twy.size(), &P->device_bytes);
   if (!rc) rc = dev_upload(&P->d_post, post.data(), post.size(), &P->device_bytes);
+  if (!rc && !fix.empty()) {
+    rc = dev_upload(&P->d_fix, fix.data(), fix.size(), &P->device_bytes);
+    if (P->M >= kFixMinLen) {
+      P->d_xfwd = P->d_fix + fix_at[0];
+      P->d_xinv = P->d_fix + fix_at[1];
+      P->d_xpost = P->d_fix + fix_at[2];
+      P->d_xpost_inv = P->d_fix + fix_at[3];
+    }
+    if (ny >= kFixMinLen) {
+      P->d_yfwd = P->d_fix + fix_at[4];
+      P->d_yinv = P->d_fix + fix_at[5];
+      if (ybc != CFS_Y_PERIODIC) {
+        P->d_ywall = P->d_fix + fix_at[6];
+        P->d_ywall_inv = P->d_fix + fix_at[7];
+      }
+    }
+  }
   if (!rc) rc = dev_upload(&P->d_dzf, P->dzf.data(), (size_t)nz, &P->device_bytes);
   if (!rc) rc = dev_upload(&P->d_sing, sing.data(), sing.size(), &P->device_bytes);
   if (!rc && !wy.empty()) rc = dev_upload(&P->d_wy, wy.data(), wy.size(), &P->device_bytes);

@@ -120,8 +120,13 @@ extern "C" int cfs_plan_autotune(cfs_plan_t P, void* stream) {
   const size_t cs = fp32 ? sizeof(float2) : sizeof(double2);
   Choice best{};
 
+  // FP64 transforms in block fixed point (fix_x.cu, fix_y.cu) have one shape per
+  // length: nothing to time there
+  const bool shaped_x = fp32 || P->M < kFixMinLen, shaped_y = fp32 || P->ny < kFixMinLen;
+
   // radix plan of the x and y transforms (default tiles), all four passes
-  {
+  best.radix = P->fft_radix;
+  if (shaped_x || shaped_y) {
     float tbest = 1e30f;
     best.radix = 8;
     for (int r : {8, 4}) {
@@ -146,7 +151,8 @@ extern "C" int cfs_plan_autotune(cfs_plan_t P, void* stream) {
     if (plan_set_radix(P, best.radix) != CFS_OK) return CFS_ECUDA;
   }
   // x-lines per CTA: forward and inverse x transform
-  {
+  best.x_lines = std::min(64, x_lines_per_cta(P, cs));
+  if (shaped_x) {
     float tbest = 1e30f;
     const long long nlines = (long long)P->ny * P->nz;
     for (int lines : {1, 2, 4, 8, 16, 32, 64}) {
@@ -179,6 +185,10 @@ extern "C" int cfs_plan_autotune(cfs_plan_t P, void* stream) {
     best.y_tile = tk0;
     for (int cand : {1, 2, 4, 8, 16, 32}) {
       if (!y_tile_ok(P, cand, fp32)) continue;
+      if (!shaped_y) {  // the option must still name a tile that fits
+        if (!y_tile_ok(P, best.y_tile, fp32)) best.y_tile = cand;
+        continue;
+      }
       tk = cand;
       const float t = best_ms(st, [&]() {
         cudaError_t e = fp32 ? launch_fft_y32(P, s32, false, st) : launch_fft_y(P, s64, false, st);
