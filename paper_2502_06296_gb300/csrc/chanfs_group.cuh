@@ -65,7 +65,6 @@ struct ThomasArgs {  // z sweeps of Eq. 12 (thomas.cu)
   double sing_cg;        // g^T 1' / sum(w)
   double sing_sc;        // the factor scale of the (0,0) column
   int M, ny, nz, nky;
-  int nblk_x;            // blocks along kx per ky
   int neumann;
   int kx64, ky64;        // FP32 spectra: columns kx < kx64, |ky| < ky64 in FP64
   int ywall;             // y walls: every slot ky is its own column (no +-ky pairs)

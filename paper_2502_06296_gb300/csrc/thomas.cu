@@ -10,8 +10,8 @@
 //   backward x_k = g_k - (C_k/piv_k) x_{k+1}
 // i.e. 3 FP64 instructions per real unknown, no division at run time.
 //
-// One thread per column of the spectrum; consecutive threads take consecutive
-// kx so that every z-plane access is coalesced.  Column kx = 0 arrives
+// A thread sweeps one to four real columns of the spectrum; consecutive threads take
+// consecutive kx so that every z-plane access is coalesced.  Column kx = 0 arrives
 // untangled by the y transform (App. A's packing applied again along y), so
 // every slot is one column of Eq. 12; the two self-conjugate slots hold two
 // real columns with different eigenvalues in their real and imaginary parts.
@@ -28,290 +28,194 @@ namespace chanfs {
 
 
 constexpr int kThomasBlock = 64;
-// Rows each thread keeps in flight ahead of its sweep (by arithmetic type):
-// an FP64 sweep is bound by the FP64 pipe and needs few; an FP32 sweep is
-// bound by memory latency.  (Deeper prefetch spills at the register budget
-// of 14 blocks of 64 threads per SM.)
-template <class CA> struct prefetch_rows { static constexpr int value = 3; };
-template <> struct prefetch_rows<float2> { static constexpr int value = 6; };
-// The same for a thread that sweeps two columns (sweep_pair): two rows per
-// step.  DEEP (FP64 plans of moderate size): the launch fits in one wave at
-// 6 (DEEP = 6) or 8 (DEEP = 4) blocks per SM, so each thread may keep a
-// queue of DEEP rows; the sweep is bound by memory latency at the few warps
-// per SM such a launch has (the channel's FP64 spectrum: 772 blocks, 6 rows
-// measured 5 % faster than 4).
-template <class CA, int DEEP> struct pair_prefetch_rows {
-  static constexpr int value = DEEP ? DEEP : 2;
-};
-template <int DEEP> struct pair_prefetch_rows<float2, DEEP> { static constexpr int value = 3; };
 
 template <class C> struct cplx_traits;
-template <> struct cplx_traits<double2> {
-  using T = double;
-  __device__ static double2 mk(double x, double y) { return make_double2(x, y); }
-};
-template <> struct cplx_traits<float2> {
-  using T = float;
-  __device__ static float2 mk(float x, float y) { return make_float2(x, y); }
-};
-template <class CA, class CS> __device__ __forceinline__ CA cvt(CS v) {
-  return cplx_traits<CA>::mk((typename cplx_traits<CA>::T)v.x, (typename cplx_traits<CA>::T)v.y);
-}
+template <> struct cplx_traits<double2> { using T = double; };
+template <> struct cplx_traits<float2> { using T = float; };
 
-// One column sweep: storage type CS (the spectrum), arithmetic type CA with
-// its factor tables F (pairs) and B (scalars).  Pointers step by a row stride
-// and each thread keeps the next prefetch_rows<CA> rows in flight while the recurrence
-// consumes the current one (the sweep is sequential in k, and there are only
-// a few warps per SM, so this in-thread prefetch is what hides the memory
-// latency).  Real and imaginary parts use factor sets x and y, which differ
-// only for the two self-conjugate slots of kx = 0 (a real F(0,ky) and a real
-// F(Nx/2,ky) packed together; see fft_y.cu).
-//
-// Neumann (0, 0) column (real part of slot (0, 0)): singular.  Its system is
+// The NV real right-hand sides of one row that a thread sweeps: one real
+// component, one complex column, or the complex columns of the slots ky and
+// Ny - ky (which share their factors: the eigenvalue depends on |ky|).
+template <class S, int NV> struct ZRow;
+template <class S> struct ZRow<S, 1> {
+  S v[1];
+  __device__ __forceinline__ void load(const S* s, const S*) { v[0] = *s; }
+  __device__ __forceinline__ void store(S* s, S*) const { *s = v[0]; }
+};
+template <class S> struct ZRow<S, 2> {
+  S v[2];
+  __device__ __forceinline__ void load(const S* s, const S*);
+  __device__ __forceinline__ void store(S* s, S*) const;
+};
+template <> __device__ __forceinline__ void ZRow<double, 2>::load(const double* s, const double*) {
+  const double2 a = *reinterpret_cast<const double2*>(s);
+  v[0] = a.x;
+  v[1] = a.y;
+}
+template <> __device__ __forceinline__ void ZRow<double, 2>::store(double* s, double*) const {
+  *reinterpret_cast<double2*>(s) = make_double2(v[0], v[1]);
+}
+template <> __device__ __forceinline__ void ZRow<float, 2>::load(const float* s, const float*) {
+  const float2 a = *reinterpret_cast<const float2*>(s);
+  v[0] = a.x;
+  v[1] = a.y;
+}
+template <> __device__ __forceinline__ void ZRow<float, 2>::store(float* s, float*) const {
+  *reinterpret_cast<float2*>(s) = make_float2(v[0], v[1]);
+}
+template <class S> struct ZRow<S, 4> {
+  S v[4];
+  __device__ __forceinline__ void load(const S* s, const S* t) {
+    ZRow<S, 2> a, b;
+    a.load(s, nullptr);
+    b.load(t, nullptr);
+    v[0] = a.v[0];
+    v[1] = a.v[1];
+    v[2] = b.v[0];
+    v[3] = b.v[1];
+  }
+  __device__ __forceinline__ void store(S* s, S* t) const {
+    ZRow<S, 2> a, b;
+    a.v[0] = v[0];
+    a.v[1] = v[1];
+    b.v[0] = v[2];
+    b.v[1] = v[3];
+    a.store(s, nullptr);
+    b.store(t, nullptr);
+  }
+};
+
+// The Neumann (0, 0) column (real part of slot (0, 0)): singular.  Its system is
 // pinned (row 0: F_0 = 0) and, by linearity, both projections are folded
 // into the same two sweeps:
 //   mu = sum_k wn_k E_k                   (dz-weighted mean of the rhs)
 //   x  = T'^{-1} E' - mu h - nu,  E' = (0, E_1, ..)
 //   nu = (g^T E' - mu g^T 1') / sum w     (dz-weighted mean of the solution)
 // with h = T'^{-1} (0, 1, .., 1) and g = T'^{-T} w precomputed by the plan.
-//
-// ONE: the real and imaginary parts share factor set x (every column but
-// kx = 0); fy0 and by0 are then not read.
-template <class CS, class CA, bool ONE, int PF, class F2, class F1>
-__device__ __forceinline__ void sweep_column(const ThomasArgs& a, CS* const s0, const F2* const fx0,
-                                             const F2* const fy0, const F1* const bx0,
-                                             const F1* const by0, const bool sing) {
-  using T = typename cplx_traits<CA>::T;
-  const int nz = a.nz;
-  const long long rs = (long long)a.ny * a.M;         // spectrum row stride
-  const long long rt = (long long)a.nky * (a.M + 1);  // factor row stride
+struct SingColumn {
+  const double* hs;  // per row; null: an ordinary column
+  double mu, nu;
+  bool mine;         // this thread's column is the singular one
+};
 
-  // forward: g_k = (s/piv_k) f_k - (A_k/piv_k) g_{k-1}, in place
-  CS qu[PF];
-  F2 qx[PF], qy[ONE ? 1 : PF];
+// The sweeps of one thread: NV right-hand sides of type S (storage; row stride
+// rs) with one factor set (row stride rt) in type T,
+//   forward  g_k = (s/piv_k) f_k - (A_k/piv_k) g_{k-1}, in place
+//   backward x_k = g_k - (C_k/piv_k) x_{k+1}, from the top wall down.
+// The sweep is sequential in k, so the thread itself keeps memory busy: rows
+// come in groups of G, the next group's loads issued together before the
+// current group is swept.  (A queue refilled row by row waits on its newest
+// load at every row, whatever its depth, because the hardware tracks loads in
+// flight by a handful of counters and not one by one: on GB300 a lone warp took
+// 2300 clocks per row that way, of which FP64 issue is 900.)
+template <class S, class T, int NV, int G, bool SING, class F2, class F1>
+__device__ __forceinline__ void sweep(S* const s0, S* const t0, const long long rs,
+                                      const F2* const f0, const F1* const b0, const long long rt,
+                                      const int nz, const SingColumn& sing) {
+  {
+    struct Group {
+      ZRow<S, NV> u[G];
+      F2 f[G];
+    } A, B;
+    const S *ps = s0, *pt = t0;
+    const F2* pf = f0;
+    const auto load = [&](Group& q, int k) {
 #pragma unroll
-  for (int i = 0; i < PF; ++i) {
-    if (i < nz) {
-      qu[i] = s0[i * rs];
-      qx[i] = fx0[i * rt];
-      if (!ONE) qy[i] = fy0[i * rt];
+      for (int i = 0; i < G; ++i) {
+        if (k + i < nz) {
+          q.u[i].load(ps, pt);
+          q.f[i] = *pf;
+        }
+        ps += rs;
+        pt += rs;
+        pf += rt;
+      }
+    };
+    T g[NV] = {};
+    S *ws = s0, *wt = t0;
+    const auto run = [&](const Group& q, int k) {
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        if (k + i < nz) {
+          ZRow<S, NV> o;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            g[v] = fma(-q.f[i].y, g[v], q.f[i].x * (T)q.u[i].v[v]);
+            o.v[v] = (S)g[v];
+          }
+          o.store(ws, wt);
+        }
+        ws += rs;
+        wt += rs;
+      }
+    };
+    load(A, 0);
+    if (SING && sing.mine) A.u[0].v[0] = S(0);  // the pinned row
+    for (int k = 0; k < nz; k += 2 * G) {
+      load(B, k + G);
+      run(A, k);
+      load(A, k + 2 * G);
+      run(B, k + G);
     }
   }
-  const CS* pu = s0 + PF * rs;  // next rows to prefetch
-  const F2* px = fx0 + PF * rt;
-  const F2* py = ONE ? px : fy0 + PF * rt;
-  CS* ps = s0;                         // row being written
-  CA g = cplx_traits<CA>::mk(T(0), T(0));
-  double mu = 0.0, gam = 0.0;
-  for (int k = 0; k < nz; k += PF) {
+  {
+    struct Group {
+      ZRow<S, NV> u[G];
+      F1 b[G];
+      double h[SING ? G : 1];
+    } A, B;
+    const long long top = (long long)(nz - 1) * rs;
+    const S *ps = s0 + top, *pt = t0 + top;
+    const F1* pb = b0 + (long long)(nz - 1) * rt;
+    const auto load = [&](Group& q, int r) {
 #pragma unroll
-    for (int i = 0; i < PF; ++i) {
-      if (k + i >= nz) break;
-      CA u = cvt<CA>(qu[i]);
-      const F2 fx = qx[i], fy = ONE ? fx : qy[i];
-      if (k + i + PF < nz) {
-        qu[i] = *pu;
-        qx[i] = *px;
-        if (!ONE) qy[i] = *py;
+      for (int i = 0; i < G; ++i) {
+        if (r + i < nz) {
+          q.u[i].load(ps, pt);
+          q.b[i] = *pb;
+          if constexpr (SING) q.h[i] = sing.hs[nz - 1 - r - i];
+        }
+        ps -= rs;
+        pt -= rs;
+        pb -= rt;
       }
-      pu += rs;
-      px += rt;
-      if (!ONE) py += rt;
-      if (sing) {
-        mu = fma(a.sing[k + i], (double)u.x, mu);
-        if (k + i > 0) gam = fma(a.sing[nz + k + i], (double)u.x, gam);
-        else u.x = T(0);  // pinned row
-      }
-      g = cplx_traits<CA>::mk(fma(-fx.y, g.x, fx.x * u.x), fma(-fy.y, g.y, fy.x * u.y));
-      *ps = cvt<CS>(g);
-      ps += rs;
-    }
-  }
-  const double nu = sing ? a.sing_sc * (gam - mu * a.sing_cg) : 0.0;
-
-  // backward: x_k = g_k - (C_k/piv_k) x_{k+1}, from the top wall down
-  CS qg[PF];
-  F1 qbx[PF], qby[ONE ? 1 : PF];
-  CS* const s1 = s0 + (long long)(nz - 1) * rs;
-  const F1* const bx1 = bx0 + (long long)(nz - 1) * rt;
-  const F1* const by1 = ONE ? bx1 : by0 + (long long)(nz - 1) * rt;
+    };
+    T x[NV] = {};
+    S *ws = s0 + top, *wt = t0 + top;
+    const auto run = [&](const Group& q, int r) {
 #pragma unroll
-  for (int i = 0; i < PF; ++i) {
-    if (i < nz) {
-      qg[i] = s1[-i * rs];
-      qbx[i] = bx1[-i * rt];
-      if (!ONE) qby[i] = by1[-i * rt];
-    }
-  }
-  const CS* pg = s1 - PF * rs;
-  const F1* pbx = bx1 - PF * rt;
-  const F1* pby = by1 - PF * rt;
-  ps = s1;
-  CA x = cplx_traits<CA>::mk(T(0), T(0));
-  for (int r = 0; r < nz; r += PF) {
+      for (int i = 0; i < G; ++i) {
+        if (r + i < nz) {
+          ZRow<S, NV> o;
 #pragma unroll
-    for (int i = 0; i < PF; ++i) {
-      if (r + i >= nz) break;
-      const CA gg = cvt<CA>(qg[i]);
-      const F1 bx = qbx[i], by = ONE ? bx : qby[i];
-      if (r + i + PF < nz) {
-        qg[i] = *pg;
-        qbx[i] = *pbx;
-        if (!ONE) qby[i] = *pby;
+          for (int v = 0; v < NV; ++v) {
+            x[v] = fma(-q.b[i], x[v], (T)q.u[i].v[v]);
+            o.v[v] = (S)x[v];
+          }
+          if constexpr (SING)
+            if (sing.mine) o.v[0] = (S)(fma(-sing.mu, q.h[i], (double)x[0]) - sing.nu);
+          o.store(ws, wt);
+        }
+        ws -= rs;
+        wt -= rs;
       }
-      pg -= rs;
-      pbx -= rt;
-      if (!ONE) pby -= rt;
-      x = cplx_traits<CA>::mk(fma(-bx, x.x, gg.x), fma(-by, x.y, gg.y));
-      CA out = x;
-      if (sing) out.x = (T)(fma(-mu, a.sing[2 * nz + (nz - 1 - r - i)], (double)out.x) - nu);
-      *ps = cvt<CS>(out);
-      ps -= rs;
+    };
+    load(A, 0);
+    for (int r = 0; r < nz; r += 2 * G) {
+      load(B, r + G);
+      run(A, r);
+      load(A, r + 2 * G);
+      run(B, r + G);
     }
   }
 }
 
-// One thread per spectrum column (kx = j in [0, M), slot ky in [0, Ny)),
-// consecutive threads on consecutive kx (every z-plane access of a warp is
-// one contiguous run).  With an FP32 spectrum (the inner solve of iterative
-// refinement) the near-singular columns of small |kx|, |ky| -- the singular
-// Neumann (0,0) one included -- are still solved in FP64 arithmetic with the
-// FP64 factors, the rest in FP32.
-//
-// The columns split into two launches: the main kernel takes every column
-// with kx >= 1 in the spectrum's own precision, whose real and imaginary
-// parts share one factor set (fewer loads and registers, deeper prefetch);
-// the special kernel takes column kx = 0 of every slot (two real columns, or
-// the singular one) and, for FP32 spectra, the FP64 columns.
-
-// Column (ky, j) in full generality; PF rows of prefetch.
-template <class CS, int PF = 1>
-__device__ __forceinline__ void thomas_column(const ThomasArgs& a, int ky, int j) {
-  // factor sets of the real (x) and imaginary (y) parts
-  int kx_x = j, kx_y = j, kp_x, kp_y;
-  if (a.ywall) {  // every slot its own column; column 0 holds the real pair F(0) + i F(M)
-    kp_x = kp_y = ky;
-    if (j == 0) kx_y = a.M;
-  } else if (j > 0) {
-    kp_x = kp_y = min(ky, a.ny - ky);
-  } else if (2 * ky == 0 || 2 * ky == a.ny) {  // real pair F(0,ky) + i F(M,ky)
-    kp_x = kp_y = ky;
-    kx_y = a.M;
-  } else if (2 * ky < a.ny) {  // F(0, ky)
-    kp_x = kp_y = ky;
-  } else {  // F(M, Ny - ky)
-    kx_x = kx_y = a.M;
-    kp_x = kp_y = a.ny - ky;
-  }
-  const bool sing = a.neumann && j == 0 && ky == 0;
-  CS* const s0 = reinterpret_cast<CS*>(a.S) + (long long)ky * a.M + j;
-  const long long ox = (long long)kp_x * (a.M + 1) + kx_x;
-  const long long oy = (long long)kp_y * (a.M + 1) + kx_y;
-  const bool fp64 = sizeof(CS) == sizeof(double2) || sing ||
-                    (kx_x < a.kx64 && kp_x < a.ky64 && kx_y < a.kx64 && kp_y < a.ky64);
-  // (one row of prefetch: these few columns run beside the main ones, whose
-  // register budget the kernel keeps)
-  if (fp64)
-    sweep_column<CS, double2, false, PF>(a, s0, a.fwd + ox, a.fwd + oy, a.bwd + ox, a.bwd + oy,
-                                        sing);
-  else
-    sweep_column<CS, float2, false, PF>(a, s0, a.fwd32 + ox, a.fwd32 + oy, a.bwd32 + ox,
-                                       a.bwd32 + oy, false);
-}
-
-// Columns (ky, j) and (Ny - ky, j) of a periodic-y spectrum share one factor
-// set (the eigenvalue depends on |ky|): one thread sweeps both, so that the
-// factors are read once for two columns and the two recurrences are
-// independent work for the same thread (the sweeps are bound by memory
-// latency).  ONE factor set (kx >= 1); both columns advance row by row.
-template <class CS, class CA, int PF, class F2, class F1>
-__device__ __forceinline__ void sweep_pair(const ThomasArgs& a, CS* const s0, CS* const t0,
-                                           const F2* const fx0, const F1* const bx0) {
-  using T = typename cplx_traits<CA>::T;
-  const int nz = a.nz;
-  const long long rs = (long long)a.ny * a.M;         // spectrum row stride
-  const long long rt = (long long)a.nky * (a.M + 1);  // factor row stride
-
-  // forward: g_k = (s/piv_k) f_k - (A_k/piv_k) g_{k-1}, in place, both columns
-  CS qu[PF], qv[PF];
-  F2 qx[PF];
-#pragma unroll
-  for (int i = 0; i < PF; ++i) {
-    if (i < nz) {
-      qu[i] = s0[i * rs];
-      qv[i] = t0[i * rs];
-      qx[i] = fx0[i * rt];
-    }
-  }
-  long long off = PF * rs;  // next row to prefetch (spectrum)
-  const F2* px = fx0 + PF * rt;
-  long long w = 0;          // row being written
-  CA g = cplx_traits<CA>::mk(T(0), T(0)), h = g;
-  for (int k = 0; k < nz; k += PF) {
-#pragma unroll
-    for (int i = 0; i < PF; ++i) {
-      if (k + i >= nz) break;
-      const CA u = cvt<CA>(qu[i]), v = cvt<CA>(qv[i]);
-      const F2 fx = qx[i];
-      if (k + i + PF < nz) {
-        qu[i] = s0[off];
-        qv[i] = t0[off];
-        qx[i] = *px;
-      }
-      off += rs;
-      px += rt;
-      g = cplx_traits<CA>::mk(fma(-fx.y, g.x, fx.x * u.x), fma(-fx.y, g.y, fx.x * u.y));
-      h = cplx_traits<CA>::mk(fma(-fx.y, h.x, fx.x * v.x), fma(-fx.y, h.y, fx.x * v.y));
-      s0[w] = cvt<CS>(g);
-      t0[w] = cvt<CS>(h);
-      w += rs;
-    }
-  }
-
-  // backward: x_k = g_k - (C_k/piv_k) x_{k+1}, from the top wall down
-  CS qg[PF], qh[PF];
-  F1 qb[PF];
-  const long long top = (long long)(nz - 1) * rs;
-  const F1* const bx1 = bx0 + (long long)(nz - 1) * rt;
-#pragma unroll
-  for (int i = 0; i < PF; ++i) {
-    if (i < nz) {
-      qg[i] = s0[top - i * rs];
-      qh[i] = t0[top - i * rs];
-      qb[i] = bx1[-i * rt];
-    }
-  }
-  off = top - PF * rs;
-  const F1* pb = bx1 - PF * rt;
-  w = top;
-  CA x = cplx_traits<CA>::mk(T(0), T(0)), y = x;
-  for (int r = 0; r < nz; r += PF) {
-#pragma unroll
-    for (int i = 0; i < PF; ++i) {
-      if (r + i >= nz) break;
-      const CA gg = cvt<CA>(qg[i]), hh = cvt<CA>(qh[i]);
-      const F1 b = qb[i];
-      if (r + i + PF < nz) {
-        qg[i] = s0[off];
-        qh[i] = t0[off];
-        qb[i] = *pb;
-      }
-      off -= rs;
-      pb -= rt;
-      x = cplx_traits<CA>::mk(fma(-b, x.x, gg.x), fma(-b, x.y, gg.y));
-      y = cplx_traits<CA>::mk(fma(-b, y.x, hh.x), fma(-b, y.y, hh.y));
-      s0[w] = cvt<CS>(x);
-      t0[w] = cvt<CS>(y);
-      w -= rs;
-    }
-  }
-}
-
-// Rows of main blocks: periodic y pairs the slots ky and Ny - ky (kp = 0 ..
-// Ny/2); y walls have every slot its own column.
-__host__ __device__ inline int main_rows(const ThomasArgs& a) {
-  return a.ywall ? a.ny : a.ny / 2 + 1;
-}
+// The columns split into two kinds of blocks: main blocks take every column
+// with kx >= 1 in the spectrum's own precision (real and imaginary parts share
+// one factor set); special blocks take column kx = 0 of every slot (two real
+// columns with their own factors, or the singular one) and, for FP32 spectra,
+// the near-singular columns of small |kx|, |ky|, which are solved in FP64
+// arithmetic with the FP64 factors: one real component per thread.
 
 // Whether column (ky, j >= 1) of an FP32 spectrum is solved in FP64.
 __device__ __forceinline__ bool fp64_column(const ThomasArgs& a, int ky, int j) {
@@ -319,36 +223,7 @@ __device__ __forceinline__ bool fp64_column(const ThomasArgs& a, int ky, int j) 
   return j < a.kx64 && kp < a.ky64;
 }
 
-template <class CS, int DEEP>
-__device__ __forceinline__ void thomas_body(const ThomasArgs& a, int blk) {
-  const int ky = blk / a.nblk_x;  // (the pair index kp for periodic y)
-  const int j = (blk % a.nblk_x) * kThomasBlock + threadIdx.x;
-  if (j == 0 || j >= a.M) return;
-  if (sizeof(CS) == sizeof(float2) && fp64_column(a, ky, j)) return;
-  if (!a.ywall && ky > 0 && 2 * ky != a.ny) {  // slots ky and Ny - ky together
-    CS* const s0 = reinterpret_cast<CS*>(a.S) + (long long)ky * a.M + j;
-    CS* const t0 = reinterpret_cast<CS*>(a.S) + (long long)(a.ny - ky) * a.M + j;
-    const long long o = (long long)ky * (a.M + 1) + j;
-    if constexpr (sizeof(CS) == sizeof(double2))
-      sweep_pair<CS, double2, pair_prefetch_rows<double2, DEEP>::value>(a, s0, t0, a.fwd + o,
-                                                                  a.bwd + o);
-    else
-      sweep_pair<CS, float2, pair_prefetch_rows<float2, DEEP>::value>(a, s0, t0, a.fwd32 + o,
-                                                                a.bwd32 + o);
-    return;
-  }
-  const int kp = a.ywall ? ky : min(ky, a.ny - ky);
-  CS* const s0 = reinterpret_cast<CS*>(a.S) + (long long)ky * a.M + j;
-  const long long o = (long long)kp * (a.M + 1) + j;
-  if constexpr (sizeof(CS) == sizeof(double2))
-    sweep_column<CS, double2, true, prefetch_rows<double2>::value>(a, s0, a.fwd + o, a.fwd + o,
-                                                                   a.bwd + o, a.bwd + o, false);
-  else
-    sweep_column<CS, float2, true, prefetch_rows<float2>::value>(
-        a, s0, a.fwd32 + o, a.fwd32 + o, a.bwd32 + o, a.bwd32 + o, false);
-}
-
-// Columns per slot of the special kernel: kx = 0, and for FP32 spectra the
+// Columns per slot of the special blocks: kx = 0, and for FP32 spectra the
 // FP64 columns kx < kx64.
 template <class CS>
 __host__ __device__ inline int special_width(const ThomasArgs& a) {
@@ -356,51 +231,147 @@ __host__ __device__ inline int special_width(const ThomasArgs& a) {
   const int w = a.kx64 > 1 ? a.kx64 : 1;
   return w < a.M ? w : a.M;
 }
-
-template <class CS, int PF = 1>
-__device__ __forceinline__ void thomas_special_body(const ThomasArgs& a, int blk) {
-  const int kxs = special_width<CS>(a);
-  const int t = blk * kThomasBlock + threadIdx.x;
-  const int j = t % kxs, ky = t / kxs;
-  if (ky >= a.ny) return;
-  if (j > 0 && !fp64_column(a, ky, j)) return;  // the main kernel's column
-  thomas_column<CS, PF>(a, ky, j);
+template <class CS>
+__host__ __device__ inline int special_blocks(const ThomasArgs& a) {
+  return (2 * a.ny * special_width<CS>(a) + kThomasBlock - 1) / kThomasBlock;
 }
 
 template <class CS>
-__host__ __device__ inline int special_blocks(const ThomasArgs& a) {
-  return (a.ny * special_width<CS>(a) + kThomasBlock - 1) / kThomasBlock;
+__device__ __forceinline__ void thomas_special_body(const ThomasArgs& a, int blk) {
+  using S = typename cplx_traits<CS>::T;
+  const int kxs = special_width<CS>(a);
+  const int t = blk * kThomasBlock + threadIdx.x;
+  const int comp = t & 1, j = (t >> 1) % kxs, ky = (t >> 1) / kxs;
+  const long long rs = 2LL * a.ny * a.M;              // spectrum row stride (reals)
+  const long long rt = (long long)a.nky * (a.M + 1);  // factor row stride
+  SingColumn sing = {nullptr, 0.0, 0.0, false};
+  if (a.neumann && blk == 0 && threadIdx.x < 32) {  // the warp of the singular column
+    const S* e = reinterpret_cast<const S*>(a.S);
+    double mu = 0.0, gam = 0.0;
+    for (int k = threadIdx.x; k < a.nz; k += 32) {
+      const double v = (double)e[k * rs];
+      mu = fma(a.sing[k], v, mu);
+      if (k > 0) gam = fma(a.sing[a.nz + k], v, gam);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mu += __shfl_xor_sync(~0u, mu, o);
+      gam += __shfl_xor_sync(~0u, gam, o);
+    }
+    sing = {a.sing + 2 * a.nz, mu, a.sing_sc * (gam - mu * a.sing_cg), threadIdx.x == 0};
+  }
+  if (ky >= a.ny) return;
+  if (j > 0 && !fp64_column(a, ky, j)) return;  // a main block's column
+  int kx = j, kp;
+  if (a.ywall) {  // every slot its own column; column 0 holds the real pair F(0) + i F(M)
+    kp = ky;
+    if (j == 0 && comp) kx = a.M;
+  } else if (j > 0) {
+    kp = min(ky, a.ny - ky);
+  } else if (ky == 0 || 2 * ky == a.ny) {  // real pair F(0,ky) + i F(M,ky)
+    kp = ky;
+    if (comp) kx = a.M;
+  } else if (2 * ky < a.ny) {  // F(0, ky)
+    kp = ky;
+  } else {  // F(M, Ny - ky)
+    kx = a.M;
+    kp = a.ny - ky;
+  }
+  S* const s = reinterpret_cast<S*>(a.S) + 2 * ((long long)ky * a.M + j) + comp;
+  const long long o = (long long)kp * (a.M + 1) + kx;
+  constexpr int G = 4;
+  if (sing.hs)
+    sweep<S, double, 1, G, true>(s, s, rs, a.fwd + o, a.bwd + o, rt, a.nz, sing);
+  else if (sizeof(S) == 8 || (kx < a.kx64 && kp < a.ky64))
+    sweep<S, double, 1, G, false>(s, s, rs, a.fwd + o, a.bwd + o, rt, a.nz, sing);
+  else if constexpr (sizeof(S) == 4)
+    sweep<S, float, 1, G, false>(s, s, rs, a.fwd32 + o, a.bwd32 + o, rt, a.nz, sing);
 }
 
-// One launch: the special columns' blocks first (their sweeps are the
-// longest-latency ones and overlap the main columns), then the main blocks.
-template <class CS, int DEEP>
+// Rows of main blocks: threads that take both slots ky and Ny - ky (periodic y)
+// run over kp = 0 .. Ny/2; the others over every slot.
+template <int NV> __host__ __device__ inline int main_rows(const ThomasArgs& a) {
+  return NV < 4 || a.ywall ? a.ny : a.ny / 2 + 1;
+}
+// Main blocks per row: kThomasBlock threads of NV right-hand sides each (two
+// threads per column with NV = 1).
+template <int NV> __host__ __device__ inline int main_width(const ThomasArgs& a) {
+  const int cols = NV == 1 ? kThomasBlock / 2 : kThomasBlock;
+  return (a.M + cols - 1) / cols;
+}
+
+template <class S, int NV, int G>
+__device__ __forceinline__ void main_sweep(const ThomasArgs& a, int ky, int ky2, int j, int comp) {
+  const long long rs = 2LL * a.ny * a.M, rt = (long long)a.nky * (a.M + 1);
+  const int kp = a.ywall ? ky : min(ky, a.ny - ky);
+  S* const s = reinterpret_cast<S*>(a.S) + 2 * ((long long)ky * a.M + j) + comp;
+  S* const t = reinterpret_cast<S*>(a.S) + 2 * ((long long)ky2 * a.M + j) + comp;
+  const long long o = (long long)kp * (a.M + 1) + j;
+  const SingColumn none = {nullptr, 0.0, 0.0, false};
+  if constexpr (sizeof(S) == 8)
+    sweep<S, S, NV, G, false>(s, t, rs, a.fwd + o, a.bwd + o, rt, a.nz, none);
+  else
+    sweep<S, S, NV, G, false>(s, t, rs, a.fwd32 + o, a.bwd32 + o, rt, a.nz, none);
+}
+
+template <class CS, int NV, int G>
+__device__ __forceinline__ void thomas_body(const ThomasArgs& a, int blk) {
+  using S = typename cplx_traits<CS>::T;
+  const int w = main_width<NV>(a);
+  const int ky = blk / w;  // (the pair index kp for both slots at once)
+  const int t = (blk % w) * kThomasBlock + threadIdx.x;
+  const int j = NV == 1 ? t >> 1 : t, comp = NV == 1 ? t & 1 : 0;
+  if (j == 0 || j >= a.M) return;
+  if (sizeof(CS) == sizeof(float2) && fp64_column(a, ky, j)) return;
+  if constexpr (NV == 4) {
+    if (!a.ywall && ky > 0 && 2 * ky != a.ny) main_sweep<S, 4, G>(a, ky, a.ny - ky, j, 0);
+    else main_sweep<S, 2, 4>(a, ky, ky, j, 0);
+  } else {
+    main_sweep<S, NV, G>(a, ky, ky, j, comp);
+  }
+}
+
+// One launch: the special columns' blocks first, then the main blocks.
+template <class CS, int NV, int G>
 __device__ __forceinline__ void thomas_launch_body(const ThomasArgs& a, int blk) {
   const int nsp = special_blocks<CS>(a);
   if (blk < nsp) thomas_special_body<CS>(a, blk);
-  else thomas_body<CS, DEEP>(a, blk - nsp);
+  else thomas_body<CS, NV, G>(a, blk - nsp);
 }
 
-// Resident blocks the register budget is sized for: 14 per SM, or 8 / 6
-// with deeper prefetch queues (DEEP 4 / 6) for launches that fit in one wave
-// of those.
-template <class CS, int DEEP>
-__global__ void __launch_bounds__(kThomasBlock, DEEP == 6 ? 6 : (DEEP == 4 ? 8 : 14))
-    thomas_kernel(ThomasArgs a) {
-  thomas_launch_body<CS, DEEP>(a, blockIdx.x);
+template <class CS, int NV, int G, int MINB>
+__global__ void __launch_bounds__(kThomasBlock, MINB) thomas_kernel(ThomasArgs a) {
+  thomas_launch_body<CS, NV, G>(a, blockIdx.x);
 }
 
 // One launch for several boxes (FP32 inner solves of grouped refinement).
-__global__ void __launch_bounds__(kThomasBlock, 14) thomas_group_kernel(const ThomasArgs* boxes,
+__global__ void __launch_bounds__(kThomasBlock, 10) thomas_group_kernel(const ThomasArgs* boxes,
                                                                         GroupMap g) {
   int b, blk;
   if (!group_block(g, &b, &blk)) return;
-  thomas_launch_body<float2, 0>(boxes[b], blk);
+  thomas_launch_body<float2, 4, 3>(boxes[b], blk);
 }
 
+template <class CS, int NV, int G, int MINB>
+static cudaError_t go_streaming(const ThomasArgs& a, cudaStream_t st) {
+  const long long blocks = special_blocks<CS>(a) + (long long)main_width<NV>(a) * main_rows<NV>(a);
+  thomas_kernel<CS, NV, G, MINB><<<(unsigned)blocks, kThomasBlock, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+// FP64: the right-hand sides per thread.  A warp's FP64 instructions occupy its
+// SM quarter's pipe for 64 clocks each, so a launch needs about two warps per
+// quarter to spread evenly and no more: both slots of a pair (NV = 4, the factors
+// read once for both) where that still gives two, else one column, else one
+// real component, which also shortens the serial sweep of a small box.  us on
+// GB300, NV = 4 / 2 / 1: 512 x 384 x 384 515 / 670 / 541, 384 x 256 x 192 171 / 134 / 154,
+// 256 x 192 x 192 140 / 89 / 85, 128 x 96 x 128 91 / 54 / 48 (FP64 floor, 3 instructions
+// per real unknown at 528 G/s: 429, 107, 54, 9).  FP32 sweeps, with little work per
+// row, take NV = 4, and a tighter register budget from 5 blocks per SM up (a refined
+// 512 x 384 x 384 solve 4.06 -> 3.81 ms; 128 x 96 x 128, where it spills in the longer
+// FP64 columns, 0.425 -> 0.45).
 template <class CS>
 static cudaError_t launch_streaming(const ThomasArgs& a, cudaStream_t st) {
-  const long long blocks = special_blocks<CS>(a) + (long long)a.nblk_x * main_rows(a);
   static std::atomic<int> sms{0};  // SMs of the device (the same on every GB300 of a process)
   int nsm = sms.load(std::memory_order_relaxed);
   if (nsm == 0) {
@@ -410,17 +381,16 @@ static cudaError_t launch_streaming(const ThomasArgs& a, cudaStream_t st) {
     sms.store(nsm, std::memory_order_relaxed);
   }
   if constexpr (sizeof(CS) == sizeof(double2)) {
-    if (blocks <= 6LL * nsm) {
-      thomas_kernel<CS, 6><<<(unsigned)blocks, kThomasBlock, 0, st>>>(a);
-      return cudaGetLastError();
-    }
-    if (blocks <= 8LL * nsm) {
-      thomas_kernel<CS, 4><<<(unsigned)blocks, kThomasBlock, 0, st>>>(a);
-      return cudaGetLastError();
-    }
+    const long long enough = 2LL * 32 * 4 * nsm;  // threads: two warps per SM quarter
+    if (!a.ywall && (long long)a.M * (a.ny / 2 + 1) >= enough)
+      return go_streaming<CS, 4, 3, 8>(a, st);
+    if ((long long)a.M * a.ny >= enough) return go_streaming<CS, 2, 4, 8>(a, st);
+    return go_streaming<CS, 1, 4, 8>(a, st);
+  } else {
+    if ((long long)main_width<4>(a) * main_rows<4>(a) >= 5LL * nsm)
+      return go_streaming<CS, 4, 3, 12>(a, st);
+    return go_streaming<CS, 4, 3, 10>(a, st);
   }
-  thomas_kernel<CS, 0><<<(unsigned)blocks, kThomasBlock, 0, st>>>(a);
-  return cudaGetLastError();
 }
 
 // ----------------------------------------------------------------------------
@@ -629,9 +599,7 @@ __device__ __forceinline__ void zpart_body(const ZPartArgs& z, int tile) {
 template <int MM>
 __device__ __forceinline__ void zpart_block(const ZPartArgs& z, int blk) {
   if (blk < z.nsp) {
-    // (a deeper prefetch than in the streaming kernel: here the main columns
-    // finish sooner, and these serial sweeps would be the launch's tail)
-    if (threadIdx.x < kThomasBlock) thomas_special_body<float2, 4>(z.t, blk);
+    if (threadIdx.x < kThomasBlock) thomas_special_body<float2>(z.t, blk);
     return;
   }
   zpart_body<MM>(z, blk - z.nsp);
@@ -674,7 +642,7 @@ static int zpart_args(const cfs_plan* P, float* data, ZPartArgs* z) {
   z->C = C;
   z->ntx = (P->M + C - 1) / C;
   z->nsp = special_blocks<float2>(z->t);
-  return z->nsp + main_rows(z->t) * z->ntx;  // slot pairs (ky, Ny - ky), or slots (y walls)
+  return z->nsp + main_rows<4>(z->t) * z->ntx;  // slot pairs (ky, Ny - ky), or slots (y walls)
 }
 
 static size_t zpart_smem(const ZPartArgs& z) {
@@ -945,7 +913,6 @@ static ThomasArgs thomas_args(const cfs_plan* P, void* data) {
   a.ny = P->ny;
   a.nz = P->nz;
   a.nky = P->nky;
-  a.nblk_x = (P->M + kThomasBlock - 1) / kThomasBlock;
   a.neumann = P->has_null;
   a.kx64 = P->kx64;
   a.ky64 = P->ky64;
@@ -1133,7 +1100,7 @@ cudaError_t launch_thomas_factor(cfs_plan* P, const double* dA, const double* dB
 
 size_t thomas_group_box(const cfs_plan* P, ThomasArgs* box, int* blocks) {
   *box = thomas_args(P, P->d_r32);
-  *blocks = special_blocks<float2>(*box) + box->nblk_x * main_rows(*box);
+  *blocks = special_blocks<float2>(*box) + main_width<4>(*box) * main_rows<4>(*box);
   return 0;
 }
 
