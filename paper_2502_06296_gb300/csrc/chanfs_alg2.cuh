@@ -181,6 +181,40 @@ __host__ __device__ inline void alg2_reduced_factor(int J, const double* sub, co
   }
 }
 
+// The same system factored from both ends (J even): rows 0 .. h-1 downwards as
+// above, rows J-1 .. h upwards, h = J/2, so that two lanes per column solve it in
+// half the steps:
+//   y_j = b_j - rl_j y_{j-1} (j < h), y_j = b_j - rl_j y_{j+1} (j >= h),
+//   x_j = rip_j y_j - ripc_j z,  z = x_{j+1} (j < h-1), x_{j-1} (j > h),
+// and in the middle the two rows left, coupled to each other alone, solved
+// outright: x_{h-1} with z = y_h, x_h with z = y_{h-1}.  T: the type of the
+// elimination (the plans factor in long double and round the factors once).
+template <class T>
+__host__ __device__ inline void alg2_reduced_twisted(int J, const double* sub, const double* diag,
+                                                     const double* sup, double* rl, double* rip,
+                                                     double* ripc) {
+  const int h = J / 2;
+  T u = diag[0], v = diag[J - 1];
+  rl[0] = rl[J - 1] = 0.0;
+  for (int j = 0; j < h - 1; ++j) {  // rows j and t = J-1-j, pivots u and v
+    const int t = J - 1 - j;
+    rip[j] = (double)(T(1) / u);
+    ripc[j] = (double)(sup[j] / u);
+    rip[t] = (double)(T(1) / v);
+    ripc[t] = (double)(sub[t] / v);
+    const T fu = sub[j + 1] / u, fv = sup[t - 1] / v;
+    rl[j + 1] = (double)fu;
+    rl[t - 1] = (double)fv;
+    u = diag[j + 1] - fu * sup[j];
+    v = diag[t - 1] - fv * sub[t];
+  }
+  const T det = u * v - T(sup[h - 1]) * sub[h];
+  rip[h - 1] = (double)(v / det);
+  ripc[h - 1] = (double)(sup[h - 1] / det);
+  rip[h] = (double)(u / det);
+  ripc[h] = (double)(sub[h] / det);
+}
+
 // The reduced system solved in parallel instead (Step 3 again): parallel
 // cyclic reduction.  At level l (stride s = 2^l) row j takes away s-away rows
 // j - s and j + s with the multipliers k1_j = sub_j / diag_{j-s} and

@@ -76,9 +76,9 @@ struct FixDesc {
 // Helmholtz coefficient set for Algorithm 2 (one (c, loc, nparts) entry).
 // Device arrays (n = rows): alpha[i] = A_i / b_{i-1}, beta[i] = C_i / b_{i+1},
 // ib[i] = 1/b_i, ap[i] = a_i/b_i, cp[i] = c_i/b_i (partition-local recurrences
-// of Algorithm 2, indexed by global row), and the LU factors of the reduced
-// 2*nparts system: rl[j] (sub-diagonal multipliers), rip[j] (inverse pivots),
-// ripc[j] (super-diagonal times inverse pivot).
+// of Algorithm 2, indexed by global row), and the factors of the reduced
+// 2*nparts system from both ends (alg2_reduced_twisted): rl[j] (multipliers),
+// rip[j] (inverse pivots), ripc[j] (the other off-diagonal times inverse pivot).
 // ----------------------------------------------------------------------------
 struct HelmCoef {
   double c;

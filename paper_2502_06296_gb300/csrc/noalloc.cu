@@ -7,7 +7,7 @@
 // other stream in flight), and applications that reserve the device's memory
 // up front for their own pool or budget have none left to give.  This entry
 // point needs no plan and allocates nothing.  A one-block kernel computes the
-// coefficients (Step 1 of Algorithm 2 for every partition, then the LU of the
+// coefficients (Step 1 of Algorithm 2 for every partition, then the factors of the
 // reduced system: 5n + 6p doubles for n unknowns and p partitions) on the GPU
 // in FP64 from the cell widths, which travel in its kernel parameters, into a
 // fixed file-scope device array; the Algorithm 2 kernel of cfs_helmholtz_solve
@@ -56,7 +56,7 @@ struct NoallocGrid {
 };
 
 // Step 1 of Algorithm 2 (Sec. 2.2.4) for the np partitions of I - c L_z,
-// thread q taking partition q, then the LU of the reduced 2np system by
+// thread q taking partition q, then the factors of the reduced 2np system by
 // thread 0: the layout pcr_kernel reads, alpha | beta | ib | ap | cp (n each)
 // at rows, then rl | rip | ripc (2np each) at red.
 __global__ void __launch_bounds__(kNoAllocParts)
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kNoAllocParts)
   __syncthreads();
   if (q == 0) {
     const int J = 2 * np;
-    alg2_reduced_factor(J, ra, rb, rc, red, red + J, red + 2 * J);
+    alg2_reduced_twisted<double>(J, ra, rb, rc, red, red + J, red + 2 * J);
   }
 }
 

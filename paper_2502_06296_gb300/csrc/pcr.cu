@@ -11,8 +11,8 @@
 //   Step 2: forward  d_i -= alpha_i d_{i-1}  (i = 2..m-1),
 //           backward d_i -= beta_i  d_{i+1}  (i = m-3..0),
 //   Step 3: the 2p boundary unknowns of each column go to a small array;
-//           16 lanes of warp 0 solve the reduced tridiagonal systems with the
-//           LU factors prepared on the host,
+//           warp 0 solves the reduced tridiagonal systems from both ends with
+//           the factors prepared on the host,
 //   Step 4: d_i = ib_i d_i - ap_i x_0 - cp_i x_{m-1}.
 // Only the right-hand side changes at run time (the point of Algorithm 2):
 // 5 FP64 instructions per unknown, no division.  The coefficients, identical
@@ -27,11 +27,14 @@ namespace chanfs {
 
 constexpr int kPcrCols = kPcrTileColumns;  // columns per tile (one half-warp)
 
+// Threads of a CTA: a half-warp per partition, a whole warp for Step 3.
+static int pcr_threads(int nparts) { return nparts < 2 ? 2 * kPcrCols : nparts * kPcrCols; }
+
 
 // Steps 2-4 of Algorithm 2 on a tile T [rows][16] in shared memory, in place:
 // the thread of column threadIdx.x % 16 and partition q (rows s .. s+m-1;
 // `part` false for threads beyond the partitions) reduces its right-hand
-// side (Step 2), 16 lanes solve the reduced systems (Step 3), and every
+// side (Step 2), one warp solves the reduced systems (Step 3), and every
 // partition is reconstructed (Step 4).  s_x holds the 2p boundary values of
 // each column, [2p][16].
 template <class R>
@@ -59,25 +62,32 @@ __device__ __forceinline__ void pcr_step2(R* T, R* s_x, const R* s_rows, int n, 
   }
 }
 
-// Step 3 by the LU factors of the reduced system, one lane per column.
+// Step 3 by the factors of the reduced system from both ends
+// (alg2_reduced_twisted): lane c of the first warp sweeps rows 0 .. J/2-1 of column
+// c, lane 16 + c rows J-1 .. J/2.  An FP64 instruction holds its SM quarter's pipe
+// for 64 clocks however many of the warp's lanes take part, and the CTA waits for
+// this step: one lane per column took twice the instructions.
 template <class R>
-__device__ __forceinline__ void pcr_step3_lu(R* s_x, const R* s_red, int J) {
+__device__ __forceinline__ void pcr_step3(R* s_x, const R* s_red, int J) {
+  if (threadIdx.x >= 32) return;
   const R* rl = s_red;
   const R* rip = s_red + J;
   const R* ripc = s_red + 2 * J;
-  const int c = threadIdx.x % kPcrCols;
-  if (threadIdx.x < kPcrCols) {
-    R y = s_x[c];
-    for (int jj = 1; jj < J; ++jj) {
-      y = fma(-rl[jj], y, s_x[jj * kPcrCols + c]);
-      s_x[jj * kPcrCols + c] = y;
-    }
-    R x = rip[J - 1] * y;
-    s_x[(J - 1) * kPcrCols + c] = x;
-    for (int jj = J - 2; jj >= 0; --jj) {
-      x = fma(-ripc[jj], x, rip[jj] * s_x[jj * kPcrCols + c]);
-      s_x[jj * kPcrCols + c] = x;
-    }
+  const int c = threadIdx.x % kPcrCols, h = J / 2;
+  const int step = threadIdx.x < kPcrCols ? 1 : -1;  // towards the middle
+  int j = step > 0 ? 0 : J - 1;
+  R y = s_x[j * kPcrCols + c];
+  for (int i = 1; i < h; ++i) {
+    j += step;
+    y = fma(-rl[j], y, s_x[j * kPcrCols + c]);
+    s_x[j * kPcrCols + c] = y;
+  }
+  R x = fma(-ripc[j], __shfl_xor_sync(~0u, y, kPcrCols), rip[j] * y);
+  s_x[j * kPcrCols + c] = x;
+  for (int i = 1; i < h; ++i) {
+    j -= step;
+    x = fma(-ripc[j], x, rip[j] * s_x[j * kPcrCols + c]);
+    s_x[j * kPcrCols + c] = x;
   }
 }
 
@@ -107,7 +117,7 @@ __device__ __forceinline__ void pcr_steps(R* T, R* s_x, const R* s_rows, const R
                                           int J, int q, bool part, int s, int m) {
   pcr_step2<R>(T, s_x, s_rows, n, q, part, s, m);
   __syncthreads();
-  pcr_step3_lu<R>(s_x, s_red, J);
+  pcr_step3<R>(s_x, s_red, J);
   __syncthreads();
   pcr_step4<R>(T, s_x, s_rows, n, q, part, s, m);
 }
@@ -507,7 +517,7 @@ static cudaError_t launch_pcr_t(const cfs_plan* P, const HelmCoef& h, const R* r
       !pcr_map<R>(&out_map, u, a.ncols, h.n, a.by, plane))
     return cudaErrorInvalidValue;
   const size_t smem = pcr_smem_t<R>(h.n, h.nparts);
-  const int threads = kPcrCols * h.nparts;
+  const int threads = pcr_threads(h.nparts);
   auto kern = pcr_kernel<R>;
   allow_max_smem(kern);
   int dev = 0, nsm = 0, per_sm = 0;
@@ -565,7 +575,7 @@ static size_t pcr_group_box_t(const cfs_plan* P, const HelmCoef& h, const R* row
   box->blocks = (int)((ntiles + kPcrGroupTiles - 1) / kPcrGroupTiles);
   box->status = P->d_status;
   *blocks = box->blocks;
-  *threads = kPcrCols * h.nparts;
+  *threads = pcr_threads(h.nparts);
   return pcr_smem_t<R>(h.n, h.nparts);
 }
 
@@ -751,7 +761,7 @@ cudaError_t launch_pcr_raw(long long ncols, int nz, int n, int nparts, int loc, 
       !pcr_map<double>(&out_map, u, ncols, n, a.by))
     return cudaErrorInvalidValue;
   const size_t smem = pcr_smem_t<double>(n, nparts);
-  const int threads = kPcrCols * nparts;
+  const int threads = pcr_threads(nparts);
   auto kern = pcr_kernel<double>;
   cudaError_t e = allow_max_smem(kern);
   if (e != cudaSuccess) return e;

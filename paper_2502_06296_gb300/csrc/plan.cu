@@ -747,10 +747,10 @@ static int helm_prepare(cfs_plan* P, double c, int loc, int nparts, HelmCoef** r
     rb[2 * q + 1] = last[1];
     rc[2 * q + 1] = last[2];
   }
-  // LU of the reduced system (Step 3; no pivoting: diagonally dominant)
+  // the reduced system's factors (Step 3; no pivoting: diagonally dominant)
   std::vector<double> red(3 * (size_t)J);
-  alg2_reduced_factor(J, ra.data(), rb.data(), rc.data(), red.data(), red.data() + J,
-                      red.data() + 2 * J);
+  alg2_reduced_twisted<long double>(J, ra.data(), rb.data(), rc.data(), red.data(), red.data() + J,
+                                    red.data() + 2 * J);
   // Thomas factors of the same system: fs = 1/piv, fa = A'/piv, fc = C'/piv
   std::vector<double> th(3 * (size_t)n);
   {
