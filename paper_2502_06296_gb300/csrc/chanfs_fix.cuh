@@ -107,6 +107,17 @@ template <bool PAIR, bool INV> __host__ __device__ constexpr bool fix_uses_sum(i
   return fix_growth<PAIR, INV>(n) + 2 * (fix_npass<PAIR>(n) - 1) >= 7;
 }
 
+// The lengths with kernels of their own (every radix, span and offset a constant:
+// about half the time of the general ones): 2^a 3^b, b <= 3, from 16 to 2048.
+#define CHANFS_FIX_LENGTHS                                                                  \
+  CHANFS_FIX_LEN(16) CHANFS_FIX_LEN(18) CHANFS_FIX_LEN(24) CHANFS_FIX_LEN(32)               \
+  CHANFS_FIX_LEN(36) CHANFS_FIX_LEN(48) CHANFS_FIX_LEN(54) CHANFS_FIX_LEN(64)               \
+  CHANFS_FIX_LEN(72) CHANFS_FIX_LEN(96) CHANFS_FIX_LEN(108) CHANFS_FIX_LEN(128)             \
+  CHANFS_FIX_LEN(144) CHANFS_FIX_LEN(192) CHANFS_FIX_LEN(216) CHANFS_FIX_LEN(256)           \
+  CHANFS_FIX_LEN(288) CHANFS_FIX_LEN(384) CHANFS_FIX_LEN(432) CHANFS_FIX_LEN(512)           \
+  CHANFS_FIX_LEN(576) CHANFS_FIX_LEN(768) CHANFS_FIX_LEN(864) CHANFS_FIX_LEN(1024)          \
+  CHANFS_FIX_LEN(1152) CHANFS_FIX_LEN(1536) CHANFS_FIX_LEN(1728) CHANFS_FIX_LEN(2048)
+
 // Shared-memory place of element e: one 16-byte element of padding per 8, so
 // that the 8 lanes of a 128-byte access phase fall on different banks also in
 // the first pass's stride-R writes.

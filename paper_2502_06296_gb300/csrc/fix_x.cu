@@ -15,7 +15,7 @@
 // products' halves; 68 % busy in ncu at 24 warps per SM), against 13.75
 // instructions per point on an FP64 pipe 32 times narrower: 2.03 / 1.99 ms forward
 // / inverse in FP64 at 512 x 384 x 384 on GB300, 0.34 / 0.35 ms here (3.6 TB/s).
-// Common lengths are compiled with every radix, span and offset a constant;
+// Lengths with up to three factors 3 are compiled with every radix, span and offset a constant;
 // with a power of two of items per line, at most 32, a warp owns its lines and
 // never waits for another.
 #include "chanfs_fix.cuh"
@@ -252,13 +252,12 @@ __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, in
   }
 }
 
-// The first pass of the group's lines.  ONE: at most one item per thread, kept
-// in registers from the scan of its magnitudes on; else every item is read
-// again for each step (its lines are in L1 or L2 by then).
+// The first pass of the group's lines: at most one item per thread, kept in
+// registers from the scan of its magnitudes on.
 // (sums: whether the scale uses the sum over the line.  Inverse: the two
 // butterflies of an item are each bounded by twice its sum, one factor 2 of which
 // is in the headroom.)
-template <int R, bool INV, bool WARP, int T, bool ONE>
+template <int R, bool INV, bool WARP, int T>
 __device__ __forceinline__ void first_pass(const XGroup& g, const double2* in, bool sums,
                                            const int4* __restrict__ post) {
   constexpr int NRAW = INV ? 2 * R + 1 : R;
@@ -266,54 +265,21 @@ __device__ __forceinline__ void first_pass(const XGroup& g, const double2* in, b
   const int per = T ? T : (INV ? (Q + 1) / 2 : Q);
   const int items = g.nl * per;
   const long long left = g.nlines - g.line0;
-  if constexpr (ONE) {
-    const int l = min(g.lane / per, g.nl - 1), i = g.lane - l * per;
-    const bool on = g.lane < items && l < left;
-    double2 raw[NRAW];
-    unsigned top = 0u;
-    float sum = 0.0f;
-    if (on) load_item<R, INV, NRAW>(in + (g.line0 + l) * g.n, g.n, Q, i, raw, top, sum);
-    if constexpr (!WARP) __syncthreads();  // the reduction's cells are cleared
-    unsigned most = __float_as_uint(sum), quanta = 0u;
-    line_max<WARP, T>(g, l, on, top, most);
-    if (sums)
-      quanta = line_sum<WARP, T>(g, l, on, on ? (INV ? 2u : 1u) * fix_quanta(sum, top, most) : 0u);
-    if (on) {
-      const FixScale f =
-          fix_scale_of(top, most, quanta, fix_ceil_log2(4 * R), g.growth, g.headroom);
-      if (i == 0) g.scale[l] = f;
-      first_item<R, INV>(g, g.A + l * g.ps, g.n, Q, i, raw, f, post);
-    }
-  } else {  // one line per CTA
-    double2 raw[NRAW];
-    __syncthreads();
-    for (int step = sums ? 0 : 1; step < 3; ++step) {
-      for (int base = 0; base < items; base += g.G) {
-        const int i = base + g.lane;
-        const bool on = i < items;
-        unsigned top = 0u;
-        float sum = 0.0f;
-        if (on) load_item<R, INV, NRAW>(in + g.line0 * g.n, g.n, Q, i, raw, top, sum);
-        if (step == (sums ? 0 : 1)) {
-          top = __reduce_max_sync(~0u, top);
-          const unsigned most = __reduce_max_sync(~0u, __float_as_uint(sum));
-          if ((g.lane & 31) == 0) {
-            atomicMax(g.top, top);
-            atomicMax(g.most, most);
-          }
-        } else if (step == 1) {
-          const unsigned q = __reduce_add_sync(
-              ~0u, on ? (INV ? 2u : 1u) * fix_quanta(sum, g.top[0], g.most[0]) : 0u);
-          if ((g.lane & 31) == 0) atomicAdd(g.quanta, q);
-        } else if (on) {
-          const FixScale f = fix_scale_of(g.top[0], g.most[0], g.quanta[0], fix_ceil_log2(4 * R),
-                                          g.growth, g.headroom);
-          if (i == 0) g.scale[0] = f;
-          first_item<R, INV>(g, g.A, g.n, Q, i, raw, f, post);
-        }
-      }
-      if (step < 2) __syncthreads();
-    }
+  const int l = min(g.lane / per, g.nl - 1), i = g.lane - l * per;
+  const bool on = g.lane < items && l < left;
+  double2 raw[NRAW];
+  unsigned top = 0u, quanta = 0u;
+  float sum = 0.0f;
+  if (on) load_item<R, INV, NRAW>(in + (g.line0 + l) * g.n, g.n, Q, i, raw, top, sum);
+  if constexpr (!WARP) __syncthreads();  // the reduction's cells are cleared
+  unsigned most = __float_as_uint(sum);
+  line_max<WARP, T>(g, l, on, top, most);
+  if (sums)
+    quanta = line_sum<WARP, T>(g, l, on, on ? (INV ? 2u : 1u) * fix_quanta(sum, top, most) : 0u);
+  if (on) {
+    const FixScale f = fix_scale_of(top, most, quanta, fix_ceil_log2(4 * R), g.growth, g.headroom);
+    if (i == 0) g.scale[l] = f;
+    first_item<R, INV>(g, g.A + l * g.ps, g.n, Q, i, raw, f, post);
   }
 }
 
@@ -422,9 +388,10 @@ __device__ __forceinline__ void fixed_middle(const XGroup& g, Fix* a, Fix* b, co
   }
 }
 
-// N > 0: the compile-time length; N = 0: any length, from d.
-template <int N, bool INV, bool ONE>
-__global__ void __launch_bounds__(256, 2)
+// N > 0: the compile-time length; N = 0: any length, from d (at most 384 items
+// of the first pass per line).
+template <int N, bool INV>
+__global__ void __launch_bounds__(N ? 256 : 384, N ? 3 : 2)
     fix_x_kernel(const double2* in, double2* out, long long nlines, FixDesc d,
                  const int4* __restrict__ tw, const int4* __restrict__ post, int lb, double mul,
                  int scaled) {
@@ -459,7 +426,7 @@ __global__ void __launch_bounds__(256, 2)
   if constexpr (!WARP)
     for (int e = threadIdx.x; e < 3 * lb; e += blockDim.x) g.top[e] = 0u;
   if constexpr (N > 0) {
-    first_pass<fix_rad<true, INV>(N, 0), INV, WARP, T, true>(g, in, fix_uses_sum<true, INV>(N),
+    first_pass<fix_rad<true, INV>(N, 0), INV, WARP, T>(g, in, fix_uses_sum<true, INV>(N),
                                                               post);
     group_sync<WARP>();
     Fix* end;
@@ -474,12 +441,12 @@ __global__ void __launch_bounds__(256, 2)
   } else {
     switch (d.radix[0]) {
       case 8:
-        if constexpr (!INV) first_pass<8, INV, false, 0, ONE>(g, in, d.sums, post);
+        if constexpr (!INV) first_pass<8, INV, false, 0>(g, in, d.sums, post);
         break;
-      case 6: first_pass<6, INV, false, 0, ONE>(g, in, d.sums, post); break;
-      case 4: first_pass<4, INV, false, 0, ONE>(g, in, d.sums, post); break;
-      case 3: first_pass<3, INV, false, 0, ONE>(g, in, d.sums, post); break;
-      default: first_pass<2, INV, false, 0, ONE>(g, in, d.sums, post); break;
+      case 6: first_pass<6, INV, false, 0>(g, in, d.sums, post); break;
+      case 4: first_pass<4, INV, false, 0>(g, in, d.sums, post); break;
+      case 3: first_pass<3, INV, false, 0>(g, in, d.sums, post); break;
+      default: first_pass<2, INV, false, 0>(g, in, d.sums, post); break;
     }
     __syncthreads();
     Fix *a = g.A, *b = g.B;
@@ -523,14 +490,14 @@ __global__ void __launch_bounds__(256, 2)
   }
 }
 
-template <int N, bool INV, bool ONE>
+template <int N, bool INV>
 static cudaError_t go(const cfs_plan* P, const double* in, double* out, double mul, long long nl,
                       int threads, int lb, cudaStream_t st) {
   const FixDesc& d = INV ? P->xinv : P->xfwd;
   const int n = P->M;
   const size_t smem = (size_t)(d.npass > 2 ? 2 : 1) * lb * (n + (n >> 3)) * sizeof(Fix) +
                       (size_t)lb * 5 * sizeof(int);
-  auto k = fix_x_kernel<N, INV, ONE>;
+  auto k = fix_x_kernel<N, INV>;
   allow_max_smem(k);
   k<<<(unsigned)((nl + lb - 1) / lb), threads, smem, st>>>(
       reinterpret_cast<const double2*>(in), reinterpret_cast<double2*>(out), nl, d,
@@ -543,10 +510,10 @@ static cudaError_t go_fixed(const cfs_plan* P, const double* in, double* out, do
                             long long nl, cudaStream_t st) {
   constexpr int T = x_items<INV>(N);
   if constexpr (warp_lines(T)) {
-    return go<N, INV, true>(P, in, out, mul, nl, 128, 4 * (32 / T), st);
+    return go<N, INV>(P, in, out, mul, nl, 128, 4 * (32 / T), st);
   } else {
     constexpr int lb = T >= 192 ? 1 : 192 / T;
-    return go<N, INV, true>(P, in, out, mul, nl, (lb * T + 31) / 32 * 32, lb, st);
+    return go<N, INV>(P, in, out, mul, nl, (lb * T + 31) / 32 * 32, lb, st);
   }
 }
 
@@ -554,22 +521,15 @@ template <bool INV>
 static cudaError_t dispatch(const cfs_plan* P, const double* in, double* out, double mul,
                             long long nl, cudaStream_t st) {
   switch (P->M) {
-    case 32: return go_fixed<32, INV>(P, in, out, mul, nl, st);
-    case 64: return go_fixed<64, INV>(P, in, out, mul, nl, st);
-    case 96: return go_fixed<96, INV>(P, in, out, mul, nl, st);
-    case 128: return go_fixed<128, INV>(P, in, out, mul, nl, st);
-    case 192: return go_fixed<192, INV>(P, in, out, mul, nl, st);
-    case 256: return go_fixed<256, INV>(P, in, out, mul, nl, st);
-    case 384: return go_fixed<384, INV>(P, in, out, mul, nl, st);
-    case 512: return go_fixed<512, INV>(P, in, out, mul, nl, st);
+#define CHANFS_FIX_LEN(n) \
+  case n:                 \
+    return go_fixed<n, INV>(P, in, out, mul, nl, st);
+    CHANFS_FIX_LENGTHS
+#undef CHANFS_FIX_LEN
     default: break;
   }
-  const int T = x_items<INV>(P->M);
-  if (T <= 256) {
-    const int lb = T >= 192 ? 1 : 192 / T;
-    return go<0, INV, true>(P, in, out, mul, nl, (lb * T + 31) / 32 * 32, lb, st);
-  }
-  return go<0, INV, false>(P, in, out, mul, nl, 256, 1, st);
+  const int T = x_items<INV>(P->M), lb = T >= 192 ? 1 : 192 / T;
+  return go<0, INV>(P, in, out, mul, nl, (lb * T + 31) / 32 * 32, lb, st);
 }
 
 cudaError_t launch_fix_x(const cfs_plan* P, const double* in, double* out, bool inverse, double mul,

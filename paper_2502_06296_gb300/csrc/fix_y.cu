@@ -6,8 +6,9 @@
 // with its own scale.  The first pass reads its butterflies from global memory
 // into registers, the last one writes them back, so a tile visits shared
 // memory only between passes.  512 x 384 x 384 on GB300: 1.70 ms in FP64 on TMA
-// tiles (bound by the FP64 pipe), 0.46 ms here (2.6 TB/s), bound by the integer
-// ALU pipe and by the barriers between the passes of a tile.
+// tiles (bound by the FP64 pipe), 0.45 ms here (2.7 TB/s), bound by the integer
+// ALU pipe and by the barriers between the passes of a tile; 3456 x 3072 x 30 11 ms
+// and 3.7 ms (tiles of two columns, one CTA of 24 warps per SM).
 #include "chanfs_fix.cuh"
 
 namespace chanfs {
@@ -107,69 +108,37 @@ __device__ __forceinline__ void first_points(const YTile& t, int j, int c, int y
   for (int r = 0; r < R; ++r) t.A[fix_pad(((j * R + r) << t.sh) + c)] = v[r];
 }
 
-// The first pass of a tile (see fix_x.cu: ONE keeps a thread's one item in
-// registers; otherwise each step reads it again).
-template <int R, bool INV, bool WALL, bool ONE>
+// The first pass of a tile: at most one item per thread, kept in registers from
+// the scan of its magnitudes on.
+template <int R, bool INV, bool WALL>
 __device__ __forceinline__ void first_pass(const YTile& t, int ytype, bool sums,
                                            const int4* __restrict__ wy) {
   const int items = (t.n / R) << t.sh;
-  if constexpr (ONE) {
-    const int it = threadIdx.x, c = it & (t.tk - 1), j = it >> t.sh;
-    const bool on = it < items && c < t.valid;
-    double2 raw[R];
-    unsigned top = 0u;
-    float sum = 0.0f;
-    if (on) load_points<R, INV, WALL>(t, j, c, ytype, raw, top, sum);
-    __syncthreads();  // the reduction's cells are cleared
-    unsigned most = __float_as_uint(sum);
-    const bool lead = (threadIdx.x & 31) < t.tk;
-    for (int o = t.tk; o < 32; o *= 2) {
-      top = max(top, __shfl_xor_sync(~0u, top, o));
-      most = max(most, __shfl_xor_sync(~0u, most, o));
-    }
-    if (lead) {
-      atomicMax(t.top + c, top);
-      atomicMax(t.most + c, most);
-    }
-    __syncthreads();
-    if (sums) {
-      unsigned q = on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
-      for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
-      if (lead) atomicAdd(t.quanta + c, q);
-      __syncthreads();
-    }
-    if (on) first_points<R, INV, WALL>(t, j, c, ytype, raw, scale_of(t, c), wy);
-  } else {
-    __syncthreads();
-    for (int step = sums ? 0 : 1; step < 3; ++step) {
-      for (int base = 0; base < items; base += blockDim.x) {
-        const int it = base + threadIdx.x, c = it & (t.tk - 1), j = it >> t.sh;
-        const bool on = it < items && c < t.valid, lead = (threadIdx.x & 31) < t.tk;
-        double2 raw[R];
-        unsigned top = 0u;
-        float sum = 0.0f;
-        if (on) load_points<R, INV, WALL>(t, j, c, ytype, raw, top, sum);
-        if (step == (sums ? 0 : 1)) {
-          unsigned most = __float_as_uint(sum);
-          for (int o = t.tk; o < 32; o *= 2) {
-            top = max(top, __shfl_xor_sync(~0u, top, o));
-            most = max(most, __shfl_xor_sync(~0u, most, o));
-          }
-          if (lead) {
-            atomicMax(t.top + c, top);
-            atomicMax(t.most + c, most);
-          }
-        } else if (step == 1) {
-          unsigned q = on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
-          for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
-          if (lead) atomicAdd(t.quanta + c, q);
-        } else if (on) {
-          first_points<R, INV, WALL>(t, j, c, ytype, raw, scale_of(t, c), wy);
-        }
-      }
-      if (step < 2) __syncthreads();
-    }
+  const int it = threadIdx.x, c = it & (t.tk - 1), j = it >> t.sh;
+  const bool on = it < items && c < t.valid;
+  double2 raw[R];
+  unsigned top = 0u;
+  float sum = 0.0f;
+  if (on) load_points<R, INV, WALL>(t, j, c, ytype, raw, top, sum);
+  __syncthreads();  // the reduction's cells are cleared
+  unsigned most = __float_as_uint(sum);
+  const bool lead = (threadIdx.x & 31) < t.tk;
+  for (int o = t.tk; o < 32; o *= 2) {
+    top = max(top, __shfl_xor_sync(~0u, top, o));
+    most = max(most, __shfl_xor_sync(~0u, most, o));
   }
+  if (lead) {
+    atomicMax(t.top + c, top);
+    atomicMax(t.most + c, most);
+  }
+  __syncthreads();
+  if (sums) {
+    unsigned q = on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
+    for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
+    if (lead) atomicAdd(t.quanta + c, q);
+    __syncthreads();
+  }
+  if (on) first_points<R, INV, WALL>(t, j, c, ytype, raw, scale_of(t, c), wy);
 }
 
 template <int R, bool INV>
@@ -274,10 +243,12 @@ __device__ __forceinline__ void fixed_middle(const YTile& t, Fix* a, Fix* b, con
 }
 
 // Columns per tile (a power of two, as its logarithm): 8, rows of 128 bytes,
-// while the first pass's items (`items` per column) fit 256 threads, else 4 or 2.
+// while the first pass's items (`items` per column) fit 384 threads, else 4, and
+// fewer only past 768 threads (rows of 32 and 16 bytes cost more than the waiting
+// of one large CTA per SM).
 __host__ __device__ constexpr int y_shift(int items) {
   int sh = 3;
-  while (sh > 1 && (items << sh) > 256) --sh;
+  while (sh > 0 && (items << sh) > (sh == 3 ? 384 : 768)) --sh;
   return sh;
 }
 constexpr int y_threads(int n) {
@@ -285,11 +256,11 @@ constexpr int y_threads(int n) {
   return ((items << y_shift(items)) + 31) / 32 * 32;
 }
 
-// N > 0: the compile-time length (periodic y); N = 0: any length, from d.  The
-// fixed lengths ask for 24 warps per SM (80 registers).
-template <int N, bool INV, bool WALL, bool ONE>
-__global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : ONE ? 256 : 512,
-                                  N ? 768 / y_threads(N ? N : 9) : ONE ? 2 : 1)
+// N > 0: the compile-time length (periodic y); N = 0: any length, from d.  Both
+// ask for 24 warps per SM (80 registers).
+template <int N, bool INV, bool WALL>
+__global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : 768,
+                                  N ? 768 / y_threads(N ? N : 9) : 1)
     fix_y_kernel(double2* data, int M, FixDesc d, const int4* __restrict__ tw,
                  const int4* __restrict__ wy, int shift, int ytype) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -319,7 +290,7 @@ __global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : ONE ? 256 : 512,
   for (int e = threadIdx.x; e < 3 * t.tk; e += blockDim.x) t.top[e] = 0u;
   Fix *a = t.A, *b = t.B;
   if constexpr (N > 0) {
-    first_pass<fix_rad<false, INV>(N, 0), INV, false, true>(t, ytype, fix_uses_sum<false, INV>(N),
+    first_pass<fix_rad<false, INV>(N, 0), INV, false>(t, ytype, fix_uses_sum<false, INV>(N),
                                                              wy);
     __syncthreads();
     fixed_middle<N, INV, 1>(t, t.A, t.B, tw, &a);
@@ -329,11 +300,11 @@ __global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : ONE ? 256 : 512,
                                                       tw + fix_twoff<false, INV>(N, PL));
   } else {
     switch (d.radix[0]) {
-      case 8: first_pass<8, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
-      case 6: first_pass<6, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
-      case 4: first_pass<4, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
-      case 3: first_pass<3, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
-      default: first_pass<2, INV, WALL, ONE>(t, ytype, d.sums, wy); break;
+      case 8: first_pass<8, INV, WALL>(t, ytype, d.sums, wy); break;
+      case 6: first_pass<6, INV, WALL>(t, ytype, d.sums, wy); break;
+      case 4: first_pass<4, INV, WALL>(t, ytype, d.sums, wy); break;
+      case 3: first_pass<3, INV, WALL>(t, ytype, d.sums, wy); break;
+      default: first_pass<2, INV, WALL>(t, ytype, d.sums, wy); break;
     }
     __syncthreads();
     for (int p = 1; p + 1 < npass; ++p) {
@@ -374,9 +345,9 @@ static size_t y_smem(int n, int sh) {
   return 2 * (pts + (pts >> 3)) * sizeof(Fix) + ((size_t)3 << sh) * sizeof(unsigned);
 }
 
-template <int N, bool INV, bool WALL, bool ONE>
+template <int N, bool INV, bool WALL>
 static cudaError_t go(const cfs_plan* P, double* data, int sh, int threads, cudaStream_t st) {
-  auto k = fix_y_kernel<N, INV, WALL, ONE>;
+  auto k = fix_y_kernel<N, INV, WALL>;
   allow_max_smem(k);
   const dim3 grid((P->M + (1 << sh) - 1) >> sh, P->nz);
   k<<<grid, threads, y_smem(P->ny, sh), st>>>(
@@ -388,25 +359,21 @@ static cudaError_t go(const cfs_plan* P, double* data, int sh, int threads, cuda
 template <bool INV, bool WALL>
 static cudaError_t dispatch(const cfs_plan* P, double* data, cudaStream_t st) {
   const int n = P->ny;
-  const int T = n / (INV ? P->yinv : P->yfwd).radix[0];  // items per column
-  int sh = y_shift(T);
-  while (sh > 0 && y_smem(n, sh) > kMaxDynSmem) --sh;
+  const int T = n / (INV ? P->yinv : P->yfwd).radix[0];  // items per column, at most 729
+  const int sh = y_shift(T);
   const int threads = ((T << sh) + 31) / 32 * 32;
-  if (threads > 256) return go<0, INV, WALL, false>(P, data, sh, 512, st);
   if constexpr (!WALL) {
     switch (n) {
-      case 64: return go<64, INV, false, true>(P, data, sh, threads, st);
-      case 96: return go<96, INV, false, true>(P, data, sh, threads, st);
-      case 128: return go<128, INV, false, true>(P, data, sh, threads, st);
-      case 192: return go<192, INV, false, true>(P, data, sh, threads, st);
-      case 256: return go<256, INV, false, true>(P, data, sh, threads, st);
-      case 384: return go<384, INV, false, true>(P, data, sh, threads, st);
-      case 512: return go<512, INV, false, true>(P, data, sh, threads, st);
-      case 768: return go<768, INV, false, true>(P, data, sh, threads, st);
+#define CHANFS_FIX_LEN(n) \
+  case n:                 \
+    return go<n, INV, false>(P, data, sh, threads, st);
+      CHANFS_FIX_LENGTHS
+      CHANFS_FIX_LEN(2304) CHANFS_FIX_LEN(3072) CHANFS_FIX_LEN(3456) CHANFS_FIX_LEN(4096)
+#undef CHANFS_FIX_LEN
       default: break;
     }
   }
-  return go<0, INV, WALL, true>(P, data, sh, threads, st);
+  return go<0, INV, WALL>(P, data, sh, threads, st);
 }
 
 cudaError_t launch_fix_y(const cfs_plan* P, double* data, bool inverse, cudaStream_t st) {
