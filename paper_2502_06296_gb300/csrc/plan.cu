@@ -452,9 +452,11 @@ extern "C" int cfs_plan_create_walls(cfs_plan_t* out, int nx, int ny, int nz, do
   double *dA = nullptr, *dB = nullptr, *dC = nullptr, *dlx = nullptr, *dly = nullptr;
   size_t scratch = 0;
   const size_t nfac = (size_t)(P->M + 1) * P->nky * nz;
-  if (!rc) rc = dev_upload(&P->d_twx, twx.data(), twx.size(), &P->device_bytes);
-  if (!rc) rc = dev_upload(&P->d_twy, twy.data(), twy.size(), &P->device_bytes);
-  if (!rc) rc = dev_upload(&P->d_post, post.data(), post.size(), &P->device_bytes);
+  // the FP64 tables of lengths too short for the fixed-point transforms
+  const bool short_x = P->M < kFixMinLen, short_y = ny < kFixMinLen;
+  if (!rc && short_x) rc = dev_upload(&P->d_twx, twx.data(), twx.size(), &P->device_bytes);
+  if (!rc && short_y) rc = dev_upload(&P->d_twy, twy.data(), twy.size(), &P->device_bytes);
+  if (!rc && short_x) rc = dev_upload(&P->d_post, post.data(), post.size(), &P->device_bytes);
   if (!rc && !fix.empty()) {
     rc = dev_upload(&P->d_fix, fix.data(), fix.size(), &P->device_bytes);
     if (P->M >= kFixMinLen) {
@@ -474,7 +476,8 @@ extern "C" int cfs_plan_create_walls(cfs_plan_t* out, int nx, int ny, int nz, do
   }
   if (!rc) rc = dev_upload(&P->d_dzf, P->dzf.data(), (size_t)nz, &P->device_bytes);
   if (!rc) rc = dev_upload(&P->d_sing, sing.data(), sing.size(), &P->device_bytes);
-  if (!rc && !wy.empty()) rc = dev_upload(&P->d_wy, wy.data(), wy.size(), &P->device_bytes);
+  if (!rc && short_y && !wy.empty())
+    rc = dev_upload(&P->d_wy, wy.data(), wy.size(), &P->device_bytes);
   if (!rc) rc = dev_alloc_guarded(P, &P->d_fwd, nfac);
   if (!rc) rc = dev_alloc_guarded(P, &P->d_bwd, nfac);
   if (!rc) rc = dev_upload<int>(&P->d_status, nullptr, 1, &P->device_bytes);
@@ -993,8 +996,9 @@ int chanfs::plan_set_radix(cfs_plan* P, int max_radix) {
     for (size_t i = 0; i < v.size(); ++i) o[i] = make_float2((float)v[i].x, (float)v[i].y);
     return cudaMemcpy(dst, o.data(), sizeof(float2) * o.size(), cudaMemcpyHostToDevice);
   };
-  cudaError_t e = put64(P->d_twx, twx);
-  if (e == cudaSuccess) e = put64(P->d_twy, twy);
+  cudaError_t e = cudaSuccess;
+  if (P->d_twx) e = put64(P->d_twx, twx);
+  if (e == cudaSuccess && P->d_twy) e = put64(P->d_twy, twy);
   if (e == cudaSuccess && P->d_twx32) e = put32(P->d_twx32, twx);
   if (e == cudaSuccess && P->d_twy32) e = put32(P->d_twy32, twy);
   if (e != cudaSuccess) return CFS_ECUDA;
