@@ -122,6 +122,27 @@ inline __host__ __device__ int start_chunks(int nz) {
   return c < 1 ? 1 : (c > kMaxStartChunks ? kMaxStartChunks : c);
 }
 
+// The blocks of a refined Poisson residual (refine.cu): 128 columns each, and
+// the planes in chunks where the columns alone make fewer than 3648 blocks
+// (four times what the SMs hold at once, so that the last wave costs little),
+// of at least 16 planes (a chunk reads one plane more than it writes).  A
+// function of the box alone: a box sums its correction's mean in the same
+// order whether it is solved alone or in a group.
+struct ResGrid {
+  int cols, planes, chunks;  // column blocks, planes per chunk, chunks
+  __host__ __device__ int blocks() const { return cols * chunks; }
+};
+inline __host__ __device__ ResGrid res_grid(int nx, int ny, int nz) {
+  ResGrid g;
+  g.cols = (int)(((long long)nx * ny + 127) / 128);
+  const int want = (3648 + g.cols - 1) / g.cols;
+  g.planes = (nz + want - 1) / want;
+  if (g.planes < 16) g.planes = 16;
+  g.planes = (g.planes + 3) / 4 * 4;  // whole groups of planes
+  g.chunks = (nz + g.planes - 1) / g.planes;
+  return g;
+}
+
 }  // namespace chanfs
 
 // ----------------------------------------------------------------------------
@@ -334,10 +355,11 @@ inline cudaError_t allow_max_smem(K kernel) {
 __device__ __forceinline__ double f32_to_f64(float f) {
   const unsigned u = __float_as_uint(f);
   const unsigned a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)  // normal: bias 127 -> 1023 under the exponent field
+    return __hiloint2double((int)(((a >> 3) + (896u << 20)) | (u & 0x80000000u)), (int)(u << 29));
   unsigned hi = 0u, lo = 0u;
-  if (a >= 0x00800000u) {  // normal, infinity or NaN: bias 127 -> 1023
-    const unsigned e = a >> 23;
-    hi = (e == 0xffu ? 0x7ff00000u : (e + 896u) << 20) | ((a >> 3) & 0xfffffu);
+  if (a >= 0x7f800000u) {  // infinity or NaN
+    hi = 0x7ff00000u | ((a >> 3) & 0xfffffu);
     lo = a << 29;
   } else if (a != 0u) {  // subnormal a * 2^-149: the leading bit moves to bit 23
     const unsigned sh = (unsigned)__clz((int)a) - 8u;
@@ -348,17 +370,23 @@ __device__ __forceinline__ double f32_to_f64(float f) {
   return __hiloint2double((int)((u & 0x80000000u) | hi), (int)lo);
 }
 
+// A normal binary32 (or one that rounds up to infinity) from the absolute
+// high word (its exponent field in [897, 1150]) and the low word: the fields
+// move up by three bits as one, and the 29 dropped bits plus half a unit less
+// the tie's parity carry into them; *up is that carry.
+__device__ __forceinline__ unsigned f64_round_bits(unsigned ahi, unsigned lw, unsigned* up) {
+  const unsigned t = __funnelshift_l(lw, ahi - (896u << 20), 3);
+  *up = ((lw & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29;
+  return t + *up;
+}
+
 __device__ __forceinline__ float f64_to_f32(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const unsigned e = (hi >> 20) & 0x7ffu;
   unsigned bits;
-  if (e >= 897u && e <= 1150u) {  // a normal binary32 (or its rounding overflows)
-    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);  // the top 23 mantissa bits
-    const unsigned rest = lo & 0x1fffffffu;                  // the 29 dropped bits
-    bits = ((e - 896u) << 23) | m;
-    // a carry out of the mantissa raises the exponent (to infinity past the
-    // largest binary32)
-    bits += (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
+  if (e - 897u <= 253u) {  // a normal binary32 (or its rounding overflows)
+    unsigned up;
+    bits = f64_round_bits(hi & 0x7fffffffu, lo, &up);
   } else if (e > 1150u) {  // too large, infinity or NaN
     bits = (e == 0x7ffu && ((hi & 0xfffffu) | lo)) ? 0x7fc00000u : 0x7f800000u;
   } else if (e == 0u) {  // binary64 zero or subnormal: rounds to zero
@@ -388,6 +416,16 @@ __device__ __forceinline__ float f64_to_f32(double x) {
 __device__ __forceinline__ void f64_split(double x, float* hi, float* lo) {
   const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
   const unsigned e = (hw >> 20) & 0x7ffu;
+  if (e - 949u <= 201u) {  // the unit 2^(e - 1075) of d is a normal binary32 itself
+    unsigned up;
+    *hi = __uint_as_float(f64_round_bits(hw & 0x7fffffffu, lw, &up) | (hw & 0x80000000u));
+    const int d = (int)(lw & 0x1fffffffu) - (int)(up << 29);
+    const unsigned unit = ((hw & 0x7ff00000u) - (948u << 20)) << 3;
+    // the conversion rounds d to 24 bits, ties to even, the product is exact;
+    // + 0 turns the -0 of d = 0 into +0
+    *lo = __fmaf_rn(__int2float_rn(d), __uint_as_float(unit | (hw & 0x80000000u)), 0.0f);
+    return;
+  }
   *hi = f64_to_f32(x);
   unsigned lbits = 0u;
   if (e >= 897u && e <= 1150u) {

@@ -47,7 +47,7 @@ std::vector<int> offsets(const std::vector<int>& blocks, int* total) {
 // Descriptor tables of a bound group, at fixed offsets of one device buffer
 // (and of its pinned host staging copy) sized for the group's capacity.
 struct GroupTables {
-  size_t xf, xi, y, th, zp, res, sx, sy, sth, szp, sres, splane, sone, ssub, neu, bytes;
+  size_t xf, xi, y, th, zp, res, sx, sy, sth, szp, sres, spres, splane, sone, ssub, neu, bytes;
   explicit GroupTables(int cap) {
     size_t o = 0;
     auto take = [&](size_t n) {
@@ -66,6 +66,7 @@ struct GroupTables {
     sth = take(sizeof(int) * (cap + 1));
     szp = take(sizeof(int) * (cap + 1));
     sres = take(sizeof(int) * (cap + 1));
+    spres = take(sizeof(int) * (cap + 1));
     splane = take(sizeof(int) * (cap + 1));
     sone = take(sizeof(int) * (cap + 1));
     ssub = take(sizeof(int) * (cap + 1));
@@ -91,9 +92,10 @@ struct cfs_group {
   ZPartArgs* d_zp = nullptr;    // partitioned z solves
   ResBox* d_res = nullptr;
   int *d_sx = nullptr, *d_sy = nullptr, *d_sth = nullptr, *d_szp = nullptr, *d_sres = nullptr;
+  int* d_spres = nullptr;
   int *d_splane = nullptr, *d_sone = nullptr, *d_ssub = nullptr;
   int* d_neumann = nullptr;  // boxes whose operator has the constants as null space
-  int tx = 0, ty = 0, tth = 0, tzp = 0, tres = 0, tplane = 0, tone = 0, tsub = 0;
+  int tx = 0, ty = 0, tth = 0, tzp = 0, tres = 0, tpres = 0, tplane = 0, tone = 0, tsub = 0;
   size_t smem_x = 0, smem_y = 0, smem_zp = 0;
   // refinement state
   int* d_active = nullptr;  // boxes still iterating
@@ -313,6 +315,7 @@ static int group_alloc(cfs_group* G, int cap) {
   G->d_sth = reinterpret_cast<int*>(G->d_tab + t.sth);
   G->d_szp = reinterpret_cast<int*>(G->d_tab + t.szp);
   G->d_sres = reinterpret_cast<int*>(G->d_tab + t.sres);
+  G->d_spres = reinterpret_cast<int*>(G->d_tab + t.spres);
   G->d_splane = reinterpret_cast<int*>(G->d_tab + t.splane);
   G->d_sone = reinterpret_cast<int*>(G->d_tab + t.sone);
   G->d_ssub = reinterpret_cast<int*>(G->d_tab + t.ssub);
@@ -342,7 +345,7 @@ static int group_bind(cfs_group* G, int nplans, const cfs_plan_t* plans, cudaStr
   ZPartArgs* zp = reinterpret_cast<ZPartArgs*>(G->h_tab + t.zp);
   ResBox* res = reinterpret_cast<ResBox*>(G->h_tab + t.res);
   std::vector<int> bx(nplans), by(nplans), bth(nplans), bzp(nplans, 0), bres(nplans),
-      bplane(nplans), bone(nplans, 1), bsub(nplans);
+      bpres(nplans), bplane(nplans), bone(nplans, 1), bsub(nplans);
   G->plans.clear();
   G->neumann.clear();
   G->res.assign(nplans, ResBox{});
@@ -385,6 +388,7 @@ static int group_bind(cfs_group* G, int nplans, const cfs_plan_t* plans, cudaStr
     r.inv_wn = P->inv_wn;
     G->res[b] = r;
     bres[b] = (int)((nxy + 127) / 128);
+    bpres[b] = res_grid(P->nx, P->ny, P->nz).blocks();
     bplane[b] = P->nz * start_chunks(P->nz);
     bsub[b] = (int)group_sub_blocks(nxy * P->nz);
   }
@@ -396,6 +400,7 @@ static int group_bind(cfs_group* G, int nplans, const cfs_plan_t* plans, cudaStr
   put(t.sth, offsets(bth, &G->tth));
   put(t.szp, offsets(bzp, &G->tzp));
   put(t.sres, offsets(bres, &G->tres));
+  put(t.spres, offsets(bpres, &G->tpres));
   put(t.splane, offsets(bplane, &G->tplane));
   put(t.sone, offsets(bone, &G->tone));
   put(t.ssub, offsets(bsub, &G->tsub));
@@ -627,10 +632,10 @@ cudaError_t poisson_iteration(cfs_group* G, int kind, cudaGraphConditionalHandle
     });
   }
   if (e == cudaSuccess) {
-    g.start = G->d_sres;
+    g.start = G->d_spres;
     e = traced(G, st, [&] {
       return launch_group_refine_stage(kind == 0 ? GSTAGE_RESIDUAL : GSTAGE_UPDATE, G->d_res, g,
-                                       G->tres, G->d_io, 1, st);
+                                       G->tpres, G->d_io, 1, st);
     });
   }
   if (e == cudaSuccess) {  // the weighted sum of p, correction by correction (Neumann boxes)
@@ -716,7 +721,7 @@ extern "C" int cfs_group_poisson_solve(cfs_group_t G, const double* const* f, do
   }
   G->trace_n = 0;
   const std::vector<long long> sig = {0,       nb,      G->tx,     G->ty,
-                                      G->tth,  G->tzp,  G->tres,   G->tplane,
+                                      G->tth,  G->tzp,  G->tpres,  G->tplane,
                                       G->tone, G->tsub, (long long)G->smem_x,
                                       (long long)G->smem_y, (long long)G->smem_zp};
   const bool graphs = G->graphs && !G->trace;

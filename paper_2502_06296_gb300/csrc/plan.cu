@@ -553,7 +553,7 @@ extern "C" int cfs_plan_create_walls(cfs_plan_t* out, int nx, int ny, int nz, do
     if (!rc) rc = dev_upload(&P->d_zk, zk.data(), zk.size(), &P->device_bytes);
     P->inv_wn = 1.0 / (wsum * (double)nx * (double)ny);
     if (!rc)
-      rc = dev_alloc_guarded(P, &P->d_mpart, ((size_t)nx * ny + 127) / 128);
+      rc = dev_alloc_guarded(P, &P->d_mpart, (size_t)res_grid(nx, ny, nz).blocks());
     if (!rc) rc = dev_alloc_guarded(P, &P->d_r32b, (size_t)nx * ny * nz);
     if (!rc) rc = dev_alloc_guarded(P, &P->d_rlo, (size_t)nx * ny * nz);
     if (!rc) rc = dev_alloc_guarded(P, &P->d_w2, (size_t)nx * ny * nz);

@@ -14,11 +14,24 @@
 #include <math.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "chanfs_group.cuh"
 
 namespace chanfs {
 
 constexpr int kResBlock = 128;
+// The Poisson residuals: planes whose loads are issued together, and the blocks
+// per SM that the registers are held to.  The kernels were bound by the wait
+// for one plane's loads after another's and by issue slots; in groups, with
+// neighbours of one coefficient added first and conversions cut to a dozen
+// instructions, first residual and update take 2370 and 2030 us at
+// 1024 x 768 x 512 (3243 and 2290 plane by plane; 20 bytes a point, 1180 us at
+// 6.8 TB/s) and 69 and 55 us at 256 x 192 x 192 (134 and 150, before the planes
+// were split into chunks).  Groups of 2, 3 and 6 planes, with the registers
+// that they leave room for, are 3 to 13% slower at both.
+constexpr int kFirstPlanes = 4, kFirstMinBlocks = 5;
+constexpr int kUpdatePlanes = 4, kUpdateMinBlocks = 6;
 
 __device__ __forceinline__ void block_max_to(float v, unsigned int* out) {
   // non-negative floats order like their bit patterns
@@ -201,92 +214,138 @@ __host__ __device__ inline double start_norm(const unsigned int* words, double m
 // two 16-byte loads: zk[3k] = (A_k, C_k), zk[3k+1] = (B'_k, dz_k),
 // zk[3k+2] = (D_k, dz_k) (first residual, below), zk[3nz] = (1/dx^2, 1/dy^2),
 // each pair as (hi, lo).
-template <class I>
+// acc (+)= c * (h + l) for c = ch + cl, all four FP32.
+template <bool INIT>
+__device__ __forceinline__ void term_acc(DoubleFloat& acc, float ch, float cl, float h, float l) {
+  const float q = __fmul_rn(ch, h);
+  float e = __fmaf_rn(ch, h, -q);  // ch * h - q, exact
+  e = __fmaf_rn(ch, l, e);
+  e = __fmaf_rn(cl, h, e);
+  if (INIT) {
+    acc.s = q;
+    acc.e = e;
+  } else {
+    float s, t;
+    two_sum(acc.s, q, s, t);
+    acc.s = s;
+    acc.e = __fadd_rn(acc.e, __fadd_rn(t, e));
+  }
+}
+
+// acc += c * (a + b): two neighbours of one coefficient, their sum exact.
+__device__ __forceinline__ void pair_acc(DoubleFloat& acc, float ch, float cl, float a, float b) {
+  float h, l;
+  two_sum(a, b, h, l);
+  term_acc<false>(acc, ch, cl, h, l);
+}
+
+// The columns that a thread of the residual kernels reads in a plane, as byte
+// offsets of FP32 values (a plane has at most 4096^2 columns, so they fit 32
+// bits; the plane's own address is the same for the whole grid).
+struct ResCol {
+  unsigned c, ip, im, jp, jm;
+  bool np, nm;  // the y ghost of a Dirichlet wall: negated
+};
+static_assert(8ull * kMaxNx * kMaxNy < (1ull << 32), "32-bit offsets of FP64 values in a plane");
+
+__device__ __forceinline__ ResCol res_col(unsigned col, int nx, int ny, int ybc) {
+  const int i = (int)(col % (unsigned)nx), j = (int)(col / (unsigned)nx);
+  ResCol q;
+  q.c = 4u * col;
+  q.ip = 4u * ((i + 1 == nx) ? col - i : col + 1);
+  q.im = 4u * ((i == 0) ? col + nx - 1 : col - 1);
+  const bool top = (j + 1 == ny), bot = (j == 0);
+  q.np = (ybc == CFS_Y_DIRICHLET) && top;
+  q.nm = (ybc == CFS_Y_DIRICHLET) && bot;
+  const bool per = (ybc == CFS_Y_PERIODIC);
+  q.jp = 4u * (top ? (per ? col - (unsigned)j * nx : col) : col + nx);
+  q.jm = 4u * (bot ? (per ? col + (unsigned)(ny - 1) * nx : col) : col - nx);
+  return q;
+}
+
+__device__ __forceinline__ float ldf(const float* plane, unsigned off) {
+  return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(plane) + off);
+}
+__device__ __forceinline__ void stf(float* plane, unsigned off, float v) {
+  *reinterpret_cast<float*>(reinterpret_cast<char*>(plane) + off) = v;
+}
+
+// Planes [k, end) of a residual kernel's column, G at a time where the plane
+// after the group exists too, then the rest one by one.
+template <int G, class F>
+__device__ __forceinline__ void by_planes(int k, int end, int nz, F&& group) {
+  for (const int whole = min(end, nz - 1) - G; k <= whole; k += G)
+    group(std::integral_constant<int, G>{}, k);
+  for (; k < end; ++k) group(std::integral_constant<int, 1>{}, k);
+}
+
 __device__ __forceinline__ void poisson_update_body(const float* __restrict__ dlt,
                                                     float* __restrict__ rhi,
                                                     float* __restrict__ rlo,
                                                     const float4* __restrict__ zk,
                                                     unsigned int* rmax, int nx, int ny, int nz,
                                                     int ybc, double* mpart, long long blk) {
-  const I nxy = (I)nx * ny;
-  const I col = (I)(blk * blockDim.x + threadIdx.x);
+  const int nxy = nx * ny;
+  const ResGrid rg = res_grid(nx, ny, nz);
+  const int chunk = (int)blk / rg.cols;
+  const int kb = chunk * rg.planes, ke = min(kb + rg.planes, nz);
+  const unsigned col = (unsigned)((int)blk - chunk * rg.cols) * kResBlock + threadIdx.x;
   float vmax = 0.0f;
-  DoubleFloat macc{0.0f, 0.0f};  // sum_k dz_k delta_k of the column
-  if (col < nxy) {
-    const int i = (int)(col % nx), j = (int)(col / nx);
-    const I ip = (i + 1 == nx) ? col - i : col + 1;
-    const I im = (i == 0) ? col + nx - 1 : col - 1;
-    I jp, jm;
-    bool np_ = false, nm_ = false;
-    if (ybc == CFS_Y_PERIODIC) {
-      jp = (j + 1 == ny) ? col - (I)j * nx : col + nx;
-      jm = (j == 0) ? col + (I)(ny - 1) * nx : col - nx;
-    } else {
-      jp = (j + 1 == ny) ? col : col + nx;
-      jm = (j == 0) ? col : col - nx;
-      np_ = (ybc == CFS_Y_DIRICHLET) && (j + 1 == ny);
-      nm_ = (ybc == CFS_Y_DIRICHLET) && (j == 0);
-    }
+  DoubleFloat macc{0.0f, 0.0f};  // sum_k dz_k delta_k of the column's chunk
+  if (col < (unsigned)nxy) {
+    const ResCol q = res_col(col, nx, ny, ybc);
     const float4 axy = zk[3 * nz];
-    // the loads of plane k + 1 are issued one iteration ahead, so that they
-    // are in flight while plane k is combined
-    float dkm = 0.0f, dk = dlt[col];
-    float dkp = (nz > 1) ? dlt[nxy + col] : 0.0f;
-    float xp = dlt[ip], xm = dlt[im], yp = dlt[jp], ym = dlt[jm];
-    float2 rp = make_float2(rhi[col], rlo[col]);
-    for (int k = 0; k < nz; ++k) {
-      const I o = (I)k * nxy;
-      const bool more = k + 1 < nz;
-      const I on = more ? o + nxy : o;  // plane k + 1 (clamped)
-      const float dkp2 = (k + 2 < nz) ? dlt[on + nxy + col] : 0.0f;
-      const float xpn = dlt[on + ip], xmn = dlt[on + im], ypn = dlt[on + jp], ymn = dlt[on + jm];
-      const float2 rpn = make_float2(rhi[on + col], rlo[on + col]);
-      const float4 ac = zk[3 * k], bw = zk[3 * k + 1];
-      DoubleFloat acc;
-      df_acc<true>(acc, bw.x, bw.y, dk);
-      df_acc<false>(acc, axy.x, axy.y, xp);
-      df_acc<false>(acc, axy.x, axy.y, xm);
-      df_acc<false>(acc, axy.z, axy.w, np_ ? -yp : yp);
-      df_acc<false>(acc, axy.z, axy.w, nm_ ? -ym : ym);
-      df_acc<false>(acc, ac.x, ac.y, dkm);
-      df_acc<false>(acc, ac.z, ac.w, dkp);
-      // (hi, lo) - (s + e) in double-float: TwoSum of the leading parts, the
-      // rest added to the error term, renormalised by a second TwoSum
-      float sh, se, hi, lo;
-      two_sum(rp.x, -acc.s, sh, se);
-      se = __fadd_rn(se, __fsub_rn(rp.y, acc.e));
-      two_sum(sh, se, hi, lo);
-      rhi[o + col] = hi;  // also the next FP32 right-hand side
-      rlo[o + col] = lo;
-      vmax = fmaxf(vmax, fabsf(hi));
-      if (mpart) df_acc<false>(macc, bw.z, bw.w, dk);
-      dkm = dk;
-      dk = dkp;
-      dkp = dkp2;
-      xp = xpn;
-      xm = xmn;
-      yp = ypn;
-      ym = ymn;
-      rp = rpn;
-    }
+    const float* start = dlt + (size_t)kb * nxy;
+    float dkm = kb ? ldf(start - nxy, q.c) : 0.0f, dk = ldf(start, q.c);
+    by_planes<kUpdatePlanes>(kb, ke, nz, [&](auto ng, int k0) {
+      constexpr int G = decltype(ng)::value;
+      float d[G], xp[G], xm[G], yp[G], ym[G], rh[G], rl[G];
+#pragma unroll
+      for (int g = 0; g < G; ++g) {  // every load of the group before its first use
+        const size_t o = (size_t)(k0 + g) * nxy;
+        d[g] = (G > 1 || k0 + 1 < nz) ? ldf(dlt + o + nxy, q.c) : 0.0f;
+        rh[g] = ldf(rhi + o, q.c);
+        rl[g] = ldf(rlo + o, q.c);
+        xp[g] = ldf(dlt + o, q.ip);
+        xm[g] = ldf(dlt + o, q.im);
+        yp[g] = ldf(dlt + o, q.jp);
+        ym[g] = ldf(dlt + o, q.jm);
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int k = k0 + g;
+        const size_t o = (size_t)k * nxy;
+        const float4 ac = zk[3 * k], bw = zk[3 * k + 1];
+        DoubleFloat acc;
+        df_acc<true>(acc, bw.x, bw.y, dk);
+        pair_acc(acc, axy.x, axy.y, xp[g], xm[g]);
+        pair_acc(acc, axy.z, axy.w, q.np ? -yp[g] : yp[g], q.nm ? -ym[g] : ym[g]);
+        df_acc<false>(acc, ac.x, ac.y, dkm);
+        df_acc<false>(acc, ac.z, ac.w, d[g]);
+        // (hi, lo) - (s + e) in double-float: TwoSum of the leading parts, the
+        // rest added to the error term, renormalised by a second TwoSum
+        float sh, se, hi, lo;
+        two_sum(rh[g], -acc.s, sh, se);
+        se = __fadd_rn(se, __fsub_rn(rl[g], acc.e));
+        two_sum(sh, se, hi, lo);
+        stf(rhi + o, q.c, hi);  // also the next FP32 right-hand side
+        stf(rlo + o, q.c, lo);
+        vmax = fmaxf(vmax, fabsf(hi));
+        if (mpart) df_acc<false>(macc, bw.z, bw.w, dk);
+        dkm = dk;
+        dk = d[g];
+      }
+    });
   }
   if (mpart) block_sum_to(f32_to_f64(macc.s) + f32_to_f64(macc.e), mpart + blk);
   block_max_to(vmax, rmax);
 }
 
-// Index type of a residual kernel: 32-bit offsets where every index of the
-// field (and the look-ahead two planes on) fits, which saves the 64-bit
-// address arithmetic of the six loads and three stores per point.
-inline __host__ __device__ bool res_idx32(int nx, int ny, int nz) {
-  return (long long)nx * ny * (nz + 2) + kResBlock < (1LL << 31);
-}
-
-template <class I>
-__global__ void __launch_bounds__(kResBlock) poisson_update_kernel(
+__global__ void __launch_bounds__(kResBlock, kUpdateMinBlocks) poisson_update_kernel(
     const float* __restrict__ dlt, float* __restrict__ rhi, float* __restrict__ rlo,
     const float4* __restrict__ zk, unsigned int* rmax, int nx, int ny, int nz, int ybc,
     double* mpart) {
-  poisson_update_body<I>(dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x);
+  poisson_update_body(dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x);
 }
 
 // ----------------------------------------------------------------------------
@@ -311,108 +370,95 @@ __global__ void __launch_bounds__(kResBlock) poisson_update_kernel(
 // smooth (its grid-scale part is O(h^2 |f|)).  f - mean is one FP64
 // subtraction; its split into hi + lo runs on the integer units.
 // ----------------------------------------------------------------------------
-// acc (+)= c * (a - b), the difference exact (TwoSum), c = ch + cl.
-template <bool INIT>
-__device__ __forceinline__ void diff_acc(DoubleFloat& acc, float ch, float cl, float a, float b) {
-  float dh, dl;
-  two_sum(a, -b, dh, dl);
-  const float q = __fmul_rn(ch, dh);
-  float e = __fmaf_rn(ch, dh, -q);  // ch * dh - q, exact
-  e = __fmaf_rn(ch, dl, e);
-  e = __fmaf_rn(cl, dh, e);
-  if (INIT) {
-    acc.s = q;
-    acc.e = e;
-  } else {
-    float s, t;
-    two_sum(acc.s, q, s, t);
-    acc.s = s;
-    acc.e = __fadd_rn(acc.e, __fadd_rn(t, e));
-  }
+// acc += c * ((a - m) + (b - m)), given twice = -2 m.  a + b and its sum with
+// -2 m are taken exactly (TwoSum); only the sum of the two errors is rounded.
+// Where a, b and 2 m are close the second is exact, so that sum is a single
+// term and exact too; where they are not, the result is of their size and the
+// rounding is 2^-48 of it.
+__device__ __forceinline__ void second_diff_acc(DoubleFloat& acc, float ch, float cl, float a,
+                                                float b, float twice) {
+  float s, t, h, l;
+  two_sum(a, b, s, t);
+  two_sum(s, twice, h, l);
+  term_acc<false>(acc, ch, cl, h, __fadd_rn(l, t));
 }
 
 // zk as for the update.  r32 must not alias dlt (the neighbours of a column
 // are read from dlt).
-template <class I>
 __device__ __forceinline__ void poisson_first_body(
     const double* __restrict__ f, const double* __restrict__ mean, const float* __restrict__ dlt,
     float* __restrict__ rhi, float* __restrict__ rlo, const float4* __restrict__ zk,
     unsigned int* rmax, int nx, int ny, int nz, int ybc, double* mpart, long long blk,
     float* __restrict__ dcopy) {
-  const I nxy = (I)nx * ny;
-  const I col = (I)(blk * blockDim.x + threadIdx.x);
+  const int nxy = nx * ny;
+  const ResGrid rg = res_grid(nx, ny, nz);
+  const int chunk = (int)blk / rg.cols;
+  const int kb = chunk * rg.planes, ke = min(kb + rg.planes, nz);
+  const unsigned col = (unsigned)((int)blk - chunk * rg.cols) * kResBlock + threadIdx.x;
   float vmax = 0.0f;
-  DoubleFloat macc{0.0f, 0.0f};  // sum_k dz_k delta_k of the column
-  if (col < nxy) {
+  DoubleFloat macc{0.0f, 0.0f};  // sum_k dz_k delta_k of the column's chunk
+  if (col < (unsigned)nxy) {
     const double mu = mean ? *mean : 0.0;
-    const int i = (int)(col % nx), j = (int)(col / nx);
-    const I ip = (i + 1 == nx) ? col - i : col + 1;
-    const I im = (i == 0) ? col + nx - 1 : col - 1;
-    // y neighbours: periodic, or the mirror ghost of a wall (+d Neumann, -d Dirichlet)
-    I jp, jm;
-    bool np_ = false, nm_ = false;  // negate the ghost
-    if (ybc == CFS_Y_PERIODIC) {
-      jp = (j + 1 == ny) ? col - (I)j * nx : col + nx;
-      jm = (j == 0) ? col + (I)(ny - 1) * nx : col - nx;
-    } else {
-      jp = (j + 1 == ny) ? col : col + nx;
-      jm = (j == 0) ? col : col - nx;
-      np_ = (ybc == CFS_Y_DIRICHLET) && (j + 1 == ny);
-      nm_ = (ybc == CFS_Y_DIRICHLET) && (j == 0);
-    }
+    const ResCol q = res_col(col, nx, ny, ybc);
     const float4 axy = zk[3 * nz];
-    // the loads of plane k + 1 are issued one iteration ahead
-    float dkm = 0.0f, dk = dlt[col];
-    float dkp = (nz > 1) ? dlt[nxy + col] : 0.0f;
-    float xp = dlt[ip], xm = dlt[im], yp = dlt[jp], ym = dlt[jm];
-    double fk = f[col];
-    for (int k = 0; k < nz; ++k) {
-      const I o = (I)k * nxy;
-      const I on = (k + 1 < nz) ? o + nxy : o;  // plane k + 1 (clamped)
-      const float dkp2 = (k + 2 < nz) ? dlt[on + nxy + col] : 0.0f;
-      const float xpn = dlt[on + ip], xmn = dlt[on + im], ypn = dlt[on + jp], ymn = dlt[on + jm];
-      const double fkn = f[on + col];
-      const float4 ac = zk[3 * k], dw = zk[3 * k + 2];
-      DoubleFloat acc;
-      diff_acc<true>(acc, ac.x, ac.y, dkm, dk);  // dkm = 0 below the first row
-      diff_acc<false>(acc, ac.z, ac.w, dkp, dk);
-      diff_acc<false>(acc, axy.x, axy.y, xp, dk);
-      diff_acc<false>(acc, axy.x, axy.y, xm, dk);
-      diff_acc<false>(acc, axy.z, axy.w, np_ ? -yp : yp, dk);
-      diff_acc<false>(acc, axy.z, axy.w, nm_ ? -ym : ym, dk);
-      df_acc<false>(acc, dw.x, dw.y, dk);
-      // ((f - mean) split) - (s + e), renormalised as in the update
-      float fh, fl, sh, se, hi, lo;
-      f64_split(fk - mu, &fh, &fl);
-      two_sum(fh, -acc.s, sh, se);
-      se = __fadd_rn(se, __fsub_rn(fl, acc.e));
-      two_sum(sh, se, hi, lo);
-      rhi[o + col] = hi;  // also the next FP32 right-hand side
-      rlo[o + col] = lo;
-      if (dcopy) dcopy[o + col] = dk;  // the correction, for the pass that writes p
-      vmax = fmaxf(vmax, fabsf(hi));
-      if (mpart) df_acc<false>(macc, dw.z, dw.w, dk);
-      dkm = dk;
-      dk = dkp;
-      dkp = dkp2;
-      xp = xpn;
-      xm = xmn;
-      yp = ypn;
-      ym = ymn;
-      fk = fkn;
-    }
+    const float* start = dlt + (size_t)kb * nxy;
+    float dk = ldf(start, q.c);
+    float gh, gl;  // d_k - d_{k-1}, exact (d_{-1} = 0): what the plane below took as d_{k+1} - d_k
+    two_sum(dk, kb ? -ldf(start - nxy, q.c) : 0.0f, gh, gl);
+    by_planes<kFirstPlanes>(kb, ke, nz, [&](auto ng, int k0) {
+      constexpr int G = decltype(ng)::value;
+      float d[G], xp[G], xm[G], yp[G], ym[G];
+      double fk[G];
+#pragma unroll
+      for (int g = 0; g < G; ++g) {  // every load of the group before its first use
+        const size_t o = (size_t)(k0 + g) * nxy;
+        d[g] = (G > 1 || k0 + 1 < nz) ? ldf(dlt + o + nxy, q.c) : 0.0f;
+        fk[g] = *reinterpret_cast<const double*>(reinterpret_cast<const char*>(f + o) + 2u * q.c);
+        xp[g] = ldf(dlt + o, q.ip);
+        xm[g] = ldf(dlt + o, q.im);
+        yp[g] = ldf(dlt + o, q.jp);
+        ym[g] = ldf(dlt + o, q.jm);
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int k = k0 + g;
+        const size_t o = (size_t)k * nxy;
+        const float4 ac = zk[3 * k], dw = zk[3 * k + 2];
+        const float twice = -2.0f * dk;
+        DoubleFloat acc;
+        term_acc<true>(acc, ac.x, ac.y, -gh, -gl);
+        two_sum(d[g], -dk, gh, gl);  // the plane's upper difference
+        term_acc<false>(acc, ac.z, ac.w, gh, gl);
+        second_diff_acc(acc, axy.x, axy.y, xp[g], xm[g], twice);
+        second_diff_acc(acc, axy.z, axy.w, q.np ? -yp[g] : yp[g], q.nm ? -ym[g] : ym[g], twice);
+        if (k == 0 || k == nz - 1)
+          df_acc<false>(acc, dw.x, dw.y, dk);  // the wall terms
+        else
+          acc.e = __fmaf_rn(dw.x, dk, acc.e);  // a residue of 2^-52 of the coefficients
+        // ((f - mean) split) - (s + e), renormalised as in the update
+        float fh, fl, sh, se, hi, lo;
+        f64_split(fk[g] - mu, &fh, &fl);
+        two_sum(fh, -acc.s, sh, se);
+        se = __fadd_rn(se, __fsub_rn(fl, acc.e));
+        two_sum(sh, se, hi, lo);
+        stf(rhi + o, q.c, hi);  // also the next FP32 right-hand side
+        stf(rlo + o, q.c, lo);
+        if (dcopy) stf(dcopy + o, q.c, dk);  // the correction, for the pass that writes p
+        vmax = fmaxf(vmax, fabsf(hi));
+        if (mpart) df_acc<false>(macc, dw.z, dw.w, dk);
+        dk = d[g];
+      }
+    });
   }
   if (mpart) block_sum_to(f32_to_f64(macc.s) + f32_to_f64(macc.e), mpart + blk);
   block_max_to(vmax, rmax);
 }
 
-template <class I>
-__global__ void __launch_bounds__(kResBlock) poisson_first_kernel(
+__global__ void __launch_bounds__(kResBlock, kFirstMinBlocks) poisson_first_kernel(
     const double* __restrict__ f, const double* __restrict__ mean, const float* __restrict__ dlt,
     float* __restrict__ rhi, float* __restrict__ rlo, const float4* __restrict__ zk,
     unsigned int* rmax, int nx, int ny, int nz, int ybc, double* mpart, float* __restrict__ dcopy) {
-  poisson_first_body<I>(f, mean, dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x,
-                        dcopy);
+  poisson_first_body(f, mean, dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x, dcopy);
 }
 
 // The dz-weighted sum of a correction, from the per-block sums of the
@@ -534,7 +580,7 @@ __global__ void mean_final_group_kernel(const ResBox* boxes, GroupMap g) {
   mean_final_body(r.partial, r.nz, start_chunks(r.nz), r.dzf, (long long)r.nx * r.ny, r.mean);
 }
 
-__global__ void __launch_bounds__(kResBlock) poisson_first_group_kernel(const ResBox* boxes,
+__global__ void __launch_bounds__(kResBlock, kFirstMinBlocks) poisson_first_group_kernel(const ResBox* boxes,
                                                                         GroupMap g,
                                                                         const GroupIo* io) {
   int b, blk;
@@ -542,12 +588,8 @@ __global__ void __launch_bounds__(kResBlock) poisson_first_group_kernel(const Re
   const ResBox& r = boxes[b];
   const double* mean = r.neumann ? r.mean : nullptr;
   double* mpart = r.neumann ? r.mpart : nullptr;
-  if (res_idx32(r.nx, r.ny, r.nz))
-    poisson_first_body<int>(io[b].f, mean, r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz,
-                            r.ybc, mpart, blk, r.dcopy);
-  else
-    poisson_first_body<long long>(io[b].f, mean, r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny,
-                                  r.nz, r.ybc, mpart, blk, r.dcopy);
+  poisson_first_body(io[b].f, mean, r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz, r.ybc,
+                     mpart, blk, r.dcopy);
 }
 
 // One block per box (Neumann boxes; the others have nothing to sum).
@@ -557,7 +599,7 @@ __global__ void mean_acc_group_kernel(const ResBox* boxes, GroupMap g) {
   const ResBox& r = boxes[b];
   if (!r.neumann) return;
   const long long nxy = (long long)r.nx * r.ny;
-  mean_acc_body(r.mpart, (int)((nxy + kResBlock - 1) / kResBlock), r.mnum);
+  mean_acc_body(r.mpart, res_grid(r.nx, r.ny, r.nz).blocks(), r.mnum);
 }
 
 __global__ void mean_from_num_group_kernel(const ResBox* boxes, GroupMap g) {
@@ -578,18 +620,13 @@ __global__ void __launch_bounds__(kResBlock) helm_residual_group_kernel(const Re
                      mode, blk);
 }
 
-__global__ void __launch_bounds__(kResBlock) poisson_update_group_kernel(const ResBox* boxes,
+__global__ void __launch_bounds__(kResBlock, kUpdateMinBlocks) poisson_update_group_kernel(const ResBox* boxes,
                                                                          GroupMap g) {
   int b, blk;
   if (!group_block(g, &b, &blk)) return;
   const ResBox& r = boxes[b];
   double* mpart = r.neumann ? r.mpart : nullptr;
-  if (res_idx32(r.nx, r.ny, r.nz))
-    poisson_update_body<int>(r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz, r.ybc, mpart,
-                             blk);
-  else
-    poisson_update_body<long long>(r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz, r.ybc,
-                                   mpart, blk);
+  poisson_update_body(r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz, r.ybc, mpart, blk);
 }
 
 __global__ void first_only_group_kernel(const ResBox* boxes, GroupMap g, const GroupIo* io) {
@@ -834,8 +871,7 @@ static double* mean_num(cfs_plan* P) { return P->d_red + 2; }
 
 int refine_poisson(cfs_plan* P, const double* f, double* p, cudaStream_t st) {
   const long long nxy = (long long)P->nx * P->ny;
-  const unsigned grid = (unsigned)((nxy + kResBlock - 1) / kResBlock);
-  const bool idx32 = res_idx32(P->nx, P->ny, P->nz);
+  const unsigned grid = (unsigned)res_grid(P->nx, P->ny, P->nz).blocks();
   double* mean = nullptr;
   // one pass over f: r_0 = f as FP32, the extremes of r_0 and (Neumann) the
   // plane sums of the compatibility mean; then the reference norm
@@ -890,14 +926,14 @@ int refine_poisson(cfs_plan* P, const double* f, double* p, cudaStream_t st) {
     // (Neumann: each kernel also sums its correction, dz-weighted, per block)
     double* mpart = P->has_null ? P->d_mpart : nullptr;
     if (e == cudaSuccess && it == 0) {  // r = (f - mean) - L delta, by differences
-      auto k = idx32 ? poisson_first_kernel<int> : poisson_first_kernel<long long>;
-      k<<<grid, kResBlock, 0, st>>>(f, mean, W, P->d_r32b, P->d_rlo, P->d_zk, max_word(P),
-                                    P->nx, P->ny, P->nz, P->ybc, mpart, nullptr);
+      poisson_first_kernel<<<grid, kResBlock, 0, st>>>(f, mean, W, P->d_r32b, P->d_rlo, P->d_zk,
+                                                       max_word(P), P->nx, P->ny, P->nz, P->ybc,
+                                                       mpart, nullptr);
       e = cudaGetLastError();
     } else if (e == cudaSuccess) {  // r -= L delta
-      auto k = idx32 ? poisson_update_kernel<int> : poisson_update_kernel<long long>;
-      k<<<grid, kResBlock, 0, st>>>(W, P->d_r32b, P->d_rlo, P->d_zk, max_word(P), P->nx, P->ny,
-                                    P->nz, P->ybc, mpart);
+      poisson_update_kernel<<<grid, kResBlock, 0, st>>>(W, P->d_r32b, P->d_rlo, P->d_zk,
+                                                        max_word(P), P->nx, P->ny, P->nz, P->ybc,
+                                                        mpart);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess && mpart) {  // the weighted sum of p, correction by correction

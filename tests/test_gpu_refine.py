@@ -123,6 +123,35 @@ def test_refined_residual_is_evaluated_to_fp64_accuracy(chanfs, bc, beta, kind):
         assert rel(p, ref) < 10 * tol, rel(p, ref)
 
 
+# The residual kernels split a box's planes into chunks and a chunk into groups of
+# four: one chunk and several, chunks of one plane and up, every remainder of a group,
+# columns that end inside a block, each y boundary.
+CHUNKS = [(32, 24, 5, 0, 0), (32, 24, 16, 1, 0), (32, 24, 17, 0, 0), (36, 27, 35, 1, 1), (64, 48, 50, 0, 2),
+          (48, 36, 67, 1, 2), (64, 54, 96, 0, 1), (1024, 384, 7, 0, 0), (768, 648, 19, 1, 0)]
+
+
+@pytest.mark.parametrize("nx,ny,nz,bc,ybc", CHUNKS)
+def test_refined_residual_in_chunks_of_planes(chanfs, nx, ny, nz, bc, ybc):
+    """The residual the library stopped at is the residual of what it returned: a term taken
+    from the wrong plane would leave an error of the size of the right-hand side."""
+    lx, ly = 12.8, 6.4
+    dz = synth.tanh_dz(nz, 1.6)
+    f = synth.normal(7 * nx + nz, (nz, ny, nx))
+    has_null = bc == 0 and ybc != 2
+    if has_null:
+        f = synth.remove_weighted_mean(f, dz)
+    with chanfs.Plan(nx, ny, nz, lx, ly, dz, bc, chanfs.F32_REFINED, ybc) as plan:
+        p = host(plan.poisson_solve(dev(f)))
+        iters, rho = plan.last_info()
+    assert rho <= TOL and 1 <= iters <= 4, (iters, rho)
+    r = f - oracle.apply_poisson_walls(p, lx, ly, dz, bc, ybc)
+    if has_null:
+        r -= (np.repeat(dz, nx * ny) @ r.ravel()) / (dz.sum() * nx * ny)
+    # FP64 rounding of the operator itself: eight terms of at most 4 |p| / h^2 each
+    h2 = min(lx / nx, ly / ny, dz.min()) ** 2
+    assert np.max(np.abs(r)) <= TOL * np.max(np.abs(f)) + 32 * 2.0**-53 * np.max(np.abs(p)) / h2
+
+
 @pytest.mark.parametrize("tw", [-1, 1, 8, 16])
 def test_refined_poisson_thomas_shapes(chanfs, tw):
     nx, ny, nz = 64, 48, 300   # two TMA boxes along z, near-singular FP64 columns
