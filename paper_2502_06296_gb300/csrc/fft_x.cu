@@ -302,8 +302,24 @@ cudaError_t launch_rfft_x32_sum(const cfs_plan* P, const float* in, double* out,
                                    first);
 }
 
+// Lines per block of a box in a group: 1536 complex points.  The count that is
+// best for the box alone is not: a group's launch takes the shared memory of
+// its largest block for every block, so that one box tuned to 64 lines left
+// room for one block per SM (a group of 16: 645 us a pass instead of 100), and
+// the other boxes fill the chip.  Two groups of 16 boxes of 128-384 x 96-192 x
+// 64-192 by points per block: 256 3563 and 4148 us a solve, 512 3162 and 3697,
+// 1024 3001 and 3495, 1536 2997 and 3493, 2048 3007 and 3498, 3072 3070 and
+// 3565; with each box's own choice 3051 and 3592 at best.  (A line's bits do
+// not depend on the count.)
+static int x_group_lines(const cfs_plan* P) {
+  const int own = x_lines_per_cta(P, sizeof(float2));
+  if (x_smem_bytes(P, own, sizeof(float2)) > kMaxDynSmem) return own;  // refused as alone
+  const int lb = 1536 / P->M;
+  return lb < 1 ? 1 : (lb > 64 ? 64 : lb);
+}
+
 size_t x_group_box(const cfs_plan* P, bool inverse, XBox* box, int* blocks) {
-  const int lb = x_lines_per_cta(P, sizeof(float2));
+  const int lb = x_group_lines(P);
   box->d = P->fx;
   box->in = P->d_r32;
   box->in2 = P->d_r32b;

@@ -269,8 +269,22 @@ cudaError_t launch_fft_y32(const cfs_plan* P, float* data, bool inverse, cudaStr
   return launch_y<float2>(P, data, inverse, P->tk32, P->d_twy32, P->d_wy32, st);
 }
 
+// Columns per tile of a box in a group: the widest tile of at most 3072 points
+// (the widest that lets four tiles share an SM), for the reason given at
+// x_group_lines.  The same two groups by points per tile: 512 4191 and 4746 us
+// a solve, 1024 3414 and 3959, 1536 3123 and 3764, 2048 3082 and 3621, 3072
+// 2974 and 3547, 4096 3000 and 3537.
+static int y_group_tile(const cfs_plan* P) {
+  int tk = P->tk32;
+  if (!y_tile_ok(P, tk, true)) return tk;  // refused as alone
+  int best = 0;
+  for (int c = 2; c <= 32; c *= 2)
+    if (c * P->ny <= 3072 && y_tile_ok(P, c, true)) best = c;
+  return best ? best : tk;
+}
+
 size_t y_group_box(const cfs_plan* P, YBox* box, int* blocks) {
-  const int tk = P->tk32;
+  const int tk = y_group_tile(P);
   const cuuint64_t gdim[3] = {(cuuint64_t)(2 * P->M), (cuuint64_t)P->ny, (cuuint64_t)P->nz};
   const cuuint64_t gstride[2] = {(cuuint64_t)(2 * P->M) * sizeof(float),
                                  (cuuint64_t)(2 * P->M) * P->ny * sizeof(float)};
