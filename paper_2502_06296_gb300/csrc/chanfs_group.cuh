@@ -88,7 +88,7 @@ struct ZPartArgs {
 struct ResBox {  // refinement residual and norms (refine.cu)
   const double* abc;   // Helmholtz: A' | B' | C'
   const double* dzf;   // cell widths
-  double* partial;     // nz * start_chunks(nz) plane-chunk sums of the start pass
+  double* partial;     // nz * start_chunks plane-chunk sums of the start pass
   double* mean;        // dz-weighted mean
   float* r32;          // FP32 residual / correction
   float* r32b;         // FP32 residual of the later iterations
@@ -104,10 +104,13 @@ struct ResBox {  // refinement residual and norms (refine.cu)
   double inv_wn;       // 1 / (sum of the cell widths * Nx * Ny)
 };
 
-// Blocks of the grouped mean subtraction for a field of n points.
+// Blocks per box of the grouped passes that most boxes leave at once (zero
+// solutions, solutions of one FP32 solve): two per SM, since starting a block
+// costs as much as it does for one with work (16 boxes of 1216 blocks, all
+// idle: 42 us a launch; 13 with these).
 inline __host__ __device__ long long group_sub_blocks(long long n) {
   const long long b = (n + 255) / 256;
-  return b < 1216 ? b : 1216;
+  return b < 304 ? b : 304;
 }
 
 struct HThomasBox {  // Helmholtz Thomas sweep of one box (helm_thomas.cu)

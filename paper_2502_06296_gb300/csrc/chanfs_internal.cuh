@@ -112,14 +112,18 @@ struct Helm3Coef {
 };
 
 // Chunks per z plane of the refined Poisson start pass (refine.cu): about
-// 2432 blocks (16 per SM) over the nz planes, at most kMaxStartChunks.
+// 2432 blocks (16 per SM) over the nz planes, at most kMaxStartChunks, and
+// 4096 points or more each where the plane has them: a thread then has eight
+// pairs to load, and a block's reductions and start are spread over them (a
+// group of 16 small boxes took 298 us in blocks of 2000 points, 191 in these).
 constexpr int kMaxStartChunks = 16;
 // Rows appended to the FP32 z-operator table for the partitioned z solve (its
 // partitions have 8 or 16 rows; the last one may extend past nz).
 constexpr int kZPartRowPad = 16;
-inline __host__ __device__ int start_chunks(int nz) {
+inline __host__ __device__ int start_chunks(int nz, long long nxy) {
   const int c = (2432 + nz - 1) / nz;
-  return c < 1 ? 1 : (c > kMaxStartChunks ? kMaxStartChunks : c);
+  const int most = (int)(nxy / 4096 < kMaxStartChunks ? nxy / 4096 : kMaxStartChunks);
+  return c > most ? (most < 1 ? 1 : most) : c;
 }
 
 // The blocks of a refined Poisson residual (refine.cu): 128 columns each, and
@@ -216,7 +220,7 @@ struct cfs_plan {
   double inv_wn;     // 1 / (sum of the cell widths * Nx * Ny)
   double* d_red;     // reduction scratch: [0] two 32-bit words (max |r| as float bits; the
                      // start pass's extreme keys), [1] mean, [2] running weighted sum of
-                     // the solution, [3..) nz * start_chunks(nz) plane partials
+                     // the solution, [3..) nz * start_chunks plane partials
   double tol;        // relative residual target
   int maxit;         // at most this many corrections
   int last_iters;

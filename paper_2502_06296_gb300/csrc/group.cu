@@ -389,7 +389,7 @@ static int group_bind(cfs_group* G, int nplans, const cfs_plan_t* plans, cudaStr
     G->res[b] = r;
     bres[b] = (int)((nxy + 127) / 128);
     bpres[b] = res_grid(P->nx, P->ny, P->nz).blocks();
-    bplane[b] = P->nz * start_chunks(P->nz);
+    bplane[b] = P->nz * start_chunks(P->nz, nxy);
     bsub[b] = (int)group_sub_blocks(nxy * P->nz);
   }
   auto put = [&](size_t at, const std::vector<int>& v) {

@@ -513,7 +513,7 @@ extern "C" int cfs_plan_create_walls(cfs_plan_t* out, int nx, int ny, int nz, do
     }
     if (!rc) rc = dev_alloc_guarded(P, &P->d_r32, (size_t)nx * ny * nz);
     if (!rc)
-      rc = dev_alloc_guarded(P, &P->d_red, (size_t)nz * start_chunks(nz) + 8);
+      rc = dev_alloc_guarded(P, &P->d_red, (size_t)nz * start_chunks(nz, (long long)nx * ny) + 8);
     // The residual kernels' coefficients, each split as hi = fl32(v),
     // lo = fl32(v - hi), packed per plane (three float4: (A, C), (B', dz),
     // (D, dz)) and then (1/dx^2, 1/dy^2).  D_k = A_k + B'_k + C_k + 2/dx^2 +
