@@ -47,12 +47,12 @@ CFG = synth.CHANNEL
 STAGES = ["x_forward", "y_forward", "z_thomas", "y_inverse", "x_inverse", "helm_u", "helm_v",
           "helm_w"]
 HELM_STAGES = ("helm_u", "helm_v", "helm_w")
-KERNEL_OF_STAGE = {"x_forward": "rfft_x_kernel<false>", "y_forward": "fft_y_kernel<false>",
-                   "z_thomas": "thomas_kernel", "y_inverse": "fft_y_kernel<true>",
-                   "x_inverse": "rfft_x_kernel<true>", "helm_u": "pcr_kernel",
+KERNEL_OF_STAGE = {"x_forward": "fix_x_kernel<false>", "y_forward": "fix_y_kernel<false>",
+                   "z_thomas": "thomas_kernel", "y_inverse": "fix_y_kernel<true>",
+                   "x_inverse": "fix_x_kernel<true>", "helm_u": "pcr_kernel",
                    "helm_v": "pcr_kernel", "helm_w": "pcr_kernel"}
-SOURCE_OF_STAGE = {"x_forward": "fft_x.cu", "x_inverse": "fft_x.cu", "y_forward": "fft_y.cu",
-                   "y_inverse": "fft_y.cu", "z_thomas": "thomas.cu", "helm_u": "pcr.cu",
+SOURCE_OF_STAGE = {"x_forward": "fix_x.cu", "x_inverse": "fix_x.cu", "y_forward": "fix_y.cu",
+                   "y_inverse": "fix_y.cu", "z_thomas": "thomas.cu", "helm_u": "pcr.cu",
                    "helm_v": "pcr.cu", "helm_w": "pcr.cu"}
 
 
@@ -914,7 +914,8 @@ def run_probe_only(args):
 
 def run_f64_adds_sweep(args):
     """The FP64 transforms of the channel Poisson solve with each level of
-    integer-unit butterfly additions (CFS_OPT_F64_ADDS_X / _Y): median
+    CFS_OPT_F64_ADDS_X / _Y (without effect on lines of nine points and more,
+    which are transformed in block fixed point: the levels agree): median
     CUDA-event ms per stage over --steps solves (stage by stage, both options
     at the level), the bits of each solve against level 0's, and the pair
     rates of the FP64 pipe and of the integer-unit additions."""
@@ -1216,6 +1217,9 @@ def run_ours(args):
             "peak_source": "FP64: 152 SMs x 2 DFMA/clk x 2 flops x 2070 MHz (1.26 TFLOP/s), the "
                            "2 DFMA/clk/SM measured by cfs_probe_fma (line's fma_probe; "
                            "profiles/fp64_fma_probe.md); HBM: MEASURED_PEAKS.json hbm_gbs"}
+    if dom_stage[:2] in ("x_", "y_"):  # 64-bit fixed point on the integer units: no FP64 flops
+        roof.update(bound="hbm", achieved=roof["hbm_gbs"], unit="GB/s",
+                    peak=float(peaks.get("hbm_gbs", 6800.0)), frac=roof["hbm_frac"])
     line = {
         "metric": METRIC, "value": agg["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": agg["ms_per_step"], "higher_is_better": False,
