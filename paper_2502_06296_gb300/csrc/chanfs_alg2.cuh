@@ -208,11 +208,13 @@ __host__ __device__ inline void alg2_reduced_twisted(int J, const double* sub, c
     u = diag[j + 1] - fu * sup[j];
     v = diag[t - 1] - fv * sub[t];
   }
-  const T det = u * v - T(sup[h - 1]) * sub[h];
-  rip[h - 1] = (double)(v / det);
-  ripc[h - 1] = (double)(sup[h - 1] / det);
-  rip[h] = (double)(u / det);
-  ripc[h] = (double)(sub[h] / det);
+  // (not through u v - sup sub: that product overflows where the rows, which
+  // grow as c / dz^2, pass the square root of the largest number)
+  const T f = sub[h] / u, g = sup[h - 1] / u, w = v - f * sup[h - 1];
+  rip[h - 1] = (double)(v / w / u);
+  ripc[h - 1] = (double)(g / w);
+  rip[h] = (double)(T(1) / w);
+  ripc[h] = (double)(f / w);
 }
 
 // The reduced system solved in parallel instead (Step 3 again): parallel

@@ -56,3 +56,22 @@ def test_twisted_factors_solve_the_reduced_system(lib, J, margin):
     M = np.diag(b) + np.diag(a[1:], -1) + np.diag(c[:-1], 1)
     # backward error of a stable elimination: J roundings of 2^-53 each, a few per row
     assert np.max(np.abs(M @ x - d)) < 8 * J * 2.0**-53 * np.max(np.abs(M) @ np.abs(x) + np.abs(d))
+
+
+@pytest.mark.parametrize("J", [2, 4, 32])
+@pytest.mark.parametrize("e", [-900, -600, 600, 1000])
+def test_twisted_factors_follow_a_power_of_two(lib, J, e):
+    """Rows times 2^e (coefficients c / dz^2 of any size): multipliers unchanged, inverse pivots and the two middle
+    rows, which multiply right-hand sides, times 2^-e."""
+    rng = np.random.default_rng(J)
+    a, c = -rng.random(J), -rng.random(J)
+    a[0] = c[-1] = 0.0
+    b = 1.5 * (np.abs(a) + np.abs(c)) + 1e-3
+    p = lambda x: x.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+    f, g = np.zeros((3, J)), np.zeros((3, J))
+    lib.twisted(J, p(a), p(b), p(c), p(f))
+    s = [np.ldexp(x, e) for x in (a, b, c)]
+    lib.twisted(J, *map(p, s), p(g))
+    f[1] = np.ldexp(f[1], -e)
+    f[2, J // 2 - 1 : J // 2 + 1] = np.ldexp(f[2, J // 2 - 1 : J // 2 + 1], -e)
+    assert np.isfinite(g).all() and np.array_equal(g, f)
