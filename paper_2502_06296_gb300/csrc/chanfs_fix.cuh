@@ -9,19 +9,28 @@
 //
 // Range.  Let B be the largest sum of |re| + |im| over the inputs of one
 // first-pass butterfly and S the sum over the line.  The twiddle products come
-// out divided by 4 (a 62-bit value times a 62-bit twiddle, the high half), so
-// every pass after the first grows its values by R / 4 at most, and none exceeds
-// S / 4.  The scale 2^s is the largest with 2^s C < 2^headroom, C = max(B, min(B G,
-// S / 4)), G = max(1, R_2/4, R_2 R_3/16, ..): no overflow for any input.  The
-// pass by pass division keeps the bits below a long line's sums that a bound on
+// out divided by D = 4 (a 62-bit value times a 62-bit twiddle, the high half), so
+// every pass after the first grows its values by R / D at most, and none exceeds
+// S / D.  The scale 2^s is the largest with 2^s C < 2^headroom, C = max(B, min(B G,
+// S / D_2)), G = max(1, R_2/D_2, R_2 R_3/(D_2 D_3), ..): no overflow for any input.
+// The pass by pass division keeps the bits below a long line's sums that a bound on
 // the whole line at the start (N max|x|, or S) would give away.  Transforms with few
 // passes leave S out (C = B G), which costs them at most two bits.
-// Precision.  Values carry 61 bits less that growth below B against the 53 of a
-// double, twiddles 62; additions are exact, a product is rounded to the last
-// place, the result is rounded to a double once.
+// Precision.  Values start with 61 bits less the growth G below B and lose what the
+// passes divide by beyond what they gain; additions are exact, a product is rounded
+// to the last place of 62, the result is rounded to a double once.  D = 4 suits
+// radix 8 and 6 and costs a radix-3 pass up to two bits of its values: a few such
+// passes fit the eight bits over a double's 53, more do not, so D = 2 in the
+// radix-3 passes of lengths that have four or more of them.  Relative L2 errors in
+// units of 2^-53 of columns like 1/k^2, one dominant value, white noise and
+// magnitudes over 12 decades, D = 4 against 2: 729 7.9 8.7 1.8 3.3 against 0.7 0.6
+// 0.9 1.4; 2187 24 34 4.0 9.5 against 0.8 1.1 2.0 4.5; FP64 passes 1.5 to 4.4.
 #pragma once
 
-#include "chanfs_internal.cuh"
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include <vector>
 
 namespace chanfs {
 
@@ -89,12 +98,34 @@ template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_twoff(int n
   return o;
 }
 
-// ceil(log2) of the largest growth max(1, R_2/4, R_2 R_3/16, ..) after the first pass.
+// Whether the radix-3 passes divide by 2: where there are four or more of them
+// (lengths with four and more factors 3, none of which has a compiled kernel).
+template <bool PAIR> __host__ __device__ constexpr bool fix_halves(int n) {
+  int threes = 0;
+  for (int p = 0; p < fix_npass<PAIR>(n); ++p) threes += fix_radix<PAIR>(n, p) == 3;
+  return threes >= 4;
+}
+// Kernels of their own, radix 6 and 3 only (a test per pass in the general ones would
+// cost the other lengths 2 %): y at 64 x 729 x 64 103.6 us (96.5 dividing by 4), x at
+// 1458 x 64 x 64 105 us forward and 82 inverse (125 and 86).
+constexpr int kHalved = -1;  // (as a length)
+// The bits that a pass p after the first divides by, and those of all of them.
+template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_div(int n, int p) {
+  return fix_halves<PAIR>(n) && fix_rad<PAIR, INV>(n, p) == 3 ? 1 : 2;
+}
+template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_drop(int n) {
+  int d = 0;
+  for (int p = 1; p < fix_npass<PAIR>(n); ++p) d += fix_div<PAIR, INV>(n, p);
+  return d;
+}
+
+// ceil(log2) of the largest growth max(1, R_2/D_2, R_2 R_3/(D_2 D_3), ..) after the
+// first pass.
 template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_growth(int n) {
   int lg = 0;
   double g = 1.0;
   for (int p = 1; p < fix_npass<PAIR>(n); ++p) {
-    g *= fix_rad<PAIR, INV>(n, p) / 4.0;
+    g *= (double)fix_rad<PAIR, INV>(n, p) / (1 << fix_div<PAIR, INV>(n, p));
     while (g > (double)(1 << lg)) ++lg;
   }
   return lg;
@@ -104,7 +135,7 @@ template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_growth(int 
 // divisions take 7 bits or more, a line with one dominant value would otherwise
 // keep fewer than a double's bits.
 template <bool PAIR, bool INV> __host__ __device__ constexpr bool fix_uses_sum(int n) {
-  return fix_growth<PAIR, INV>(n) + 2 * (fix_npass<PAIR>(n) - 1) >= 7;
+  return fix_growth<PAIR, INV>(n) + fix_drop<PAIR, INV>(n) >= 7;
 }
 
 // The lengths with kernels of their own (every radix, span and offset a constant:
@@ -123,7 +154,52 @@ template <bool PAIR, bool INV> __host__ __device__ constexpr bool fix_uses_sum(i
 // the first pass's stride-R writes.
 __host__ __device__ constexpr int fix_pad(int e) { return e + (e >> 3); }
 
-#ifdef __CUDACC__
+// exp(-+2 pi i e / n) in units of 2^-62, the low words signed.  The values of
+// an eighth of the circle are computed once, in long double; the others are
+// their reflections.
+class FixRoots {
+ public:
+  explicit FixRoots(int n) : n_(n) {
+    const long double half_pi = 1.57079632679489661923132169163975144L;
+    for (int r = 0; 2 * r <= n; r += 4) add(half_pi * (long double)r / (long double)n);
+    if (n % 4) {  // the remainders of 4 e / n run over more than multiples of 4
+      cs_.clear();
+      for (int r = 0; 2 * r <= n; ++r) add(half_pi * (long double)r / (long double)n);
+    }
+  }
+  int4 at(long long e, bool conj) const {
+    e %= n_;
+    const long long q = 4 * e / n_, rest = 4 * e - q * n_;  // quarter turns, rest / n of the next
+    const bool swap = 2 * rest > n_;
+    const long long i = swap ? n_ - rest : rest;
+    const longlong2 cs = cs_[n_ % 4 ? i : i / 4];
+    const long long u = swap ? cs.y : cs.x, v = swap ? cs.x : cs.y;
+    const long long re = q == 0 ? u : q == 1 ? -v : q == 2 ? -u : v;
+    const long long im = q == 0 ? v : q == 1 ? u : q == 2 ? -v : -u;  // e^{+i angle}
+    int4 w;
+    split(re, &w.x, &w.y);
+    split(conj ? im : -im, &w.z, &w.w);
+    return w;
+  }
+
+ private:
+  void add(long double a) {
+    cs_.push_back(make_longlong2(llroundl(cosl(a) * 4611686018427387904.0L),
+                                 llroundl(sinl(a) * 4611686018427387904.0L)));
+  }
+  static void split(long long x, int* hi, int* lo) {
+    long long l = (long long)(int)(x & 0xffffffffll);
+    if (l == -2147483648ll) l = -2147483647ll;  // its negative is used too
+    *hi = (int)((x - l) >> 32);
+    *lo = (int)l;
+  }
+  long long n_;
+  std::vector<longlong2> cs_;
+};
+
+// (CHANFS_FIX_ON_HOST: a host test compiles the arithmetic with its own
+// definitions of the intrinsics.)
+#if defined(__CUDACC__) || defined(CHANFS_FIX_ON_HOST)
 
 __device__ __forceinline__ Fix fadd(Fix a, Fix b) { return {a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ Fix fsub(Fix a, Fix b) { return {a.x - b.x, a.y - b.y}; }
@@ -132,9 +208,13 @@ template <bool INV> __device__ __forceinline__ Fix frot(Fix a) {  // times -i (f
 }
 
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
   long long d;
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
   return d;
+#else
+  return (long long)((unsigned long long)((long long)a * b) + (unsigned long long)c);
+#endif
 }
 
 // v = h 2^32 + l with a signed low word.
@@ -313,13 +393,13 @@ __device__ __forceinline__ unsigned fix_quanta(float sum, unsigned top, unsigned
 // the maximum is far from 1, from the maximum and the points of a butterfly.  A
 // line of zeros takes s = 0.
 __device__ __forceinline__ FixScale fix_scale_of(unsigned top, unsigned most, unsigned quanta,
-                                                 int lgpts, int growth, int headroom) {
+                                                 int lgpts, int growth, int headroom, int div) {
   const int e = (int)(top >> 20);
   if (fix_summed(top)) {
     const int eb = (int)((most + 256u) >> 23) - 126;  // B < 2^eb
     int ec = eb + growth;
-    // S / 4 < 2^(eb - 19 + bits(quanta) - 2)
-    if (quanta) ec = max(eb, min(ec, eb + 11 - __clz((int)quanta)));
+    // S / D_2 < 2^(eb - 19 + bits(quanta) - div)
+    if (quanta) ec = max(eb, min(ec, eb + 13 - div - __clz((int)quanta)));
     return {headroom - ec, 0};
   }
   if (top == 0u) return {0, 0};
@@ -361,33 +441,43 @@ __device__ __forceinline__ double2 fix_to(Fix v, int s, int kind) {
   return make_double2(fix_to(v.x, s, kind), fix_to(v.y, s, kind));
 }
 
-// The DFT of a pass after the first: v[r] w[r - 1] / 4, transformed.
-template <int R, bool INV>
+// The DFT of a pass after the first: v[r] w[r - 1] / D, transformed.  (HALF, for
+// radix 3, D = 2: whole products and sums, which stay below 3 x 2^61, then the
+// division, towards zero: no common sign.)
+template <int R, bool INV, bool HALF>
 __device__ __forceinline__ void fix_twiddle_dft(Fix* v, const int4* __restrict__ tw, int stride) {
-  v[0] = fquarter(v[0]);
+  if constexpr (HALF) {
 #pragma unroll
-  for (int r = 1; r < R; ++r) v[r] = fmul4(v[r], __ldg(tw + (r - 1) * stride));
-  fdft<R, INV>(v);
-  v[0].x -= R * kFixBias;
-  v[0].y -= R * kFixBias;
+    for (int r = 1; r < R; ++r) v[r] = fmul(v[r], __ldg(tw + (r - 1) * stride));
+    fdft<R, INV>(v);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = {v[r].x / 2, v[r].y / 2};
+  } else {
+    v[0] = fquarter(v[0]);
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[r] = fmul4(v[r], __ldg(tw + (r - 1) * stride));
+    fdft<R, INV>(v);
+    v[0].x -= R * kFixBias;
+    v[0].y -= R * kFixBias;
+  }
 }
 
 // One Stockham radix-R butterfly: item j of a batch whose element e lives at
-// at(e): points j + r q of `in`, twiddles (over 4), DFT, positions (j - k) R + k
+// at(e): points j + r q of `in`, twiddles (over D), DFT, positions (j - k) R + k
 // + r L of `out`, k = j mod L.
-template <int R, bool INV, class At>
+template <int R, bool INV, bool HALF, class At>
 __device__ __forceinline__ void fix_butterfly(const Fix* in, Fix* out, int j, int q, int L,
                                               const int4* __restrict__ tw, At at) {
   Fix v[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) v[r] = in[at(j + r * q)];
   const int k = j % L;
-  fix_twiddle_dft<R, INV>(v, tw + k, L);
+  fix_twiddle_dft<R, INV, HALF>(v, tw + k, L);
   const int o = (j - k) * R + k;
 #pragma unroll
   for (int r = 0; r < R; ++r) out[at(o + r * L)] = v[r];
 }
 
-#endif  // __CUDACC__
+#endif
 
 }  // namespace chanfs

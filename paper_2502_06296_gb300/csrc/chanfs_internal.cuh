@@ -70,6 +70,9 @@ struct FixDesc {
   int growth;  // bits that the values may grow by after the first pass
   int sums;    // whether the scale uses the sum over the line
   int radix[kFixMaxPass], span[kFixMaxPass], twoff[kFixMaxPass];
+  int half;    // whether the radix-3 passes divide by 2
+  int div;     // bits of the second pass's division
+  int drop;    // bits of all divisions
 };
 
 // ----------------------------------------------------------------------------

@@ -19,6 +19,7 @@
 // with a power of two of items per line, at most 32, a warp owns its lines and
 // never waits for another.
 #include "chanfs_fix.cuh"
+#include "chanfs_internal.cuh"
 
 namespace chanfs {
 
@@ -120,8 +121,8 @@ struct XGroup {
   int nl;              // its lines
   long long line0;     // the first one
   long long nlines;    // lines of the field
-  int n, ps, headroom, growth;
-  int drop;            // 2^-drop: the passes' divisions by 4 (and the factor 2 of 2 X or 2 Z)
+  int n, ps, headroom, growth, div;
+  int drop;            // 2^-drop: the passes' divisions (and the factor 2 of 2 X or 2 Z)
   Fix *A, *B;          // two buffers of nl padded lines
   unsigned *top, *most, *quanta;
   FixScale* scale;
@@ -277,26 +278,27 @@ __device__ __forceinline__ void first_pass(const XGroup& g, const double2* in, b
   if (sums)
     quanta = line_sum<WARP, T>(g, l, on, on ? (INV ? 2u : 1u) * fix_quanta(sum, top, most) : 0u);
   if (on) {
-    const FixScale f = fix_scale_of(top, most, quanta, fix_ceil_log2(4 * R), g.growth, g.headroom);
+    const FixScale f =
+        fix_scale_of(top, most, quanta, fix_ceil_log2(4 * R), g.growth, g.headroom, g.div);
     if (i == 0) g.scale[l] = f;
     first_item<R, INV>(g, g.A + l * g.ps, g.n, Q, i, raw, f, post);
   }
 }
 
 // A middle pass over the group's lines, from one buffer to the other.
-template <int R, bool INV>
+template <int R, bool INV, bool HALF>
 __device__ __forceinline__ void middle_pass(const XGroup& g, const Fix* in, Fix* out, int L,
                                             const int4* __restrict__ tw) {
   const int Q = g.n / R, items = g.nl * Q;
   for (int it = g.lane; it < items; it += g.G) {
     const int l = it / Q, j = it - l * Q;
-    fix_butterfly<R, INV>(in + l * g.ps, out + l * g.ps, j, Q, L, tw,
+    fix_butterfly<R, INV, HALF>(in + l * g.ps, out + l * g.ps, j, Q, L, tw,
                           [](int e) { return fix_pad(e); });
   }
 }
 
 // The last forward pass with the untangling: pairs to global memory.
-template <int R>
+template <int R, bool HALF>
 __device__ __forceinline__ void last_forward(const XGroup& g, const Fix* in, double2* out,
                                              const int4* __restrict__ tw,
                                              const int4* __restrict__ post) {
@@ -314,8 +316,8 @@ __device__ __forceinline__ void last_forward(const XGroup& g, const Fix* in, dou
       a[r] = x[fix_pad(i + r * Q)];
       b[r] = x[fix_pad(jb + r * Q)];
     }
-    fix_twiddle_dft<R, false>(a, tw + i, Q);
-    fix_twiddle_dft<R, false>(b, tw + jb, Q);
+    fix_twiddle_dft<R, false, HALF>(a, tw + i, Q);
+    fix_twiddle_dft<R, false, HALF>(b, tw + jb, Q);
     const FixScale f = g.scale[l];
     const int sh = f.s - g.drop;
     double2* o = out + (g.line0 + l) * n;
@@ -340,7 +342,7 @@ static __device__ __noinline__ double2 scaled_by(double2 z, double mul) {
 // The last inverse pass: plain butterflies to global memory.
 // (The factor `mul`, where a caller wants one, goes on last: its FP64 products
 // are kept out of the plain code, where they would be most of the FP64 work.)
-template <int R>
+template <int R, bool HALF>
 __device__ __forceinline__ void last_inverse(const XGroup& g, const Fix* in, double2* out,
                                              const int4* __restrict__ tw, double mul, int scaled) {
   const int n = g.n, Q = n / R, items = g.nl * Q;
@@ -351,7 +353,7 @@ __device__ __forceinline__ void last_inverse(const XGroup& g, const Fix* in, dou
     Fix v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = x[fix_pad(j + r * Q)];
-    fix_twiddle_dft<R, true>(v, tw + j, Q);
+    fix_twiddle_dft<R, true, HALF>(v, tw + j, Q);
     const FixScale f = g.scale[l];
     const int sh = f.s - g.drop;
     double2* o = out + (g.line0 + l) * n;
@@ -379,8 +381,8 @@ __device__ __forceinline__ void fixed_middle(const XGroup& g, Fix* a, Fix* b, co
   constexpr int NP = fix_npass<true>(N);
   constexpr bool WARP = warp_lines(x_items<INV>(N));
   if constexpr (P + 1 < NP) {
-    middle_pass<fix_rad<true, INV>(N, P), INV>(g, a, b, fix_span<true, INV>(N, P),
-                                               tw + fix_twoff<true, INV>(N, P));
+    middle_pass<fix_rad<true, INV>(N, P), INV, false>(g, a, b, fix_span<true, INV>(N, P),
+                                                      tw + fix_twoff<true, INV>(N, P));
     group_sync<WARP>();
     fixed_middle<N, INV, P + 1>(g, b, a, tw, end);
   } else {
@@ -389,16 +391,17 @@ __device__ __forceinline__ void fixed_middle(const XGroup& g, Fix* a, Fix* b, co
 }
 
 // N > 0: the compile-time length; N = 0: any length, from d (at most 384 items
-// of the first pass per line).
+// of the first pass per line); N = kHalved: one whose radix-3 passes divide by 2.
 template <int N, bool INV>
-__global__ void __launch_bounds__(N ? 256 : 384, N ? 3 : 2)
+__global__ void __launch_bounds__(N > 0 ? 256 : 384, N > 0 ? 3 : 2)
     fix_x_kernel(const double2* in, double2* out, long long nlines, FixDesc d,
                  const int4* __restrict__ tw, const int4* __restrict__ post, int lb, double mul,
                  int scaled) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int T = N ? x_items<INV>(N ? N : 8) : 0;
+  constexpr int T = N > 0 ? x_items<INV>(N > 0 ? N : 8) : 0;
   constexpr bool WARP = N > 0 && warp_lines(T);
-  const int n = N ? N : d.n;
+  constexpr bool HALF = N == kHalved;
+  const int n = N > 0 ? N : d.n;
   const int ps = n + (n >> 3);
   XGroup g;
   g.n = n;
@@ -406,7 +409,8 @@ __global__ void __launch_bounds__(N ? 256 : 384, N ? 3 : 2)
   // forward: 2 X is up to 4 times a value of the last pass; inverse: a butterfly
   // of 2 Z is up to twice its item's sum, and nothing follows the last pass
   g.headroom = INV ? 61 : 60;
-  g.growth = N ? fix_growth<true, INV>(N ? N : 9) : d.growth;
+  g.growth = N > 0 ? fix_growth<true, INV>(N > 0 ? N : 9) : d.growth;
+  g.div = HALF ? d.div : 2;
   g.nlines = nlines;
   const int grp = WARP ? (int)(threadIdx.x >> 5) : 0;
   g.nl = WARP ? 32 / (T ? T : 32) : lb;
@@ -415,8 +419,8 @@ __global__ void __launch_bounds__(N ? 256 : 384, N ? 3 : 2)
   g.line0 = (long long)blockIdx.x * lb + grp * g.nl;
   Fix* buf = reinterpret_cast<Fix*>(smem_raw);
   g.A = buf + grp * g.nl * ps;
-  const int npass = N ? fix_npass<true>(N ? N : 8) : d.npass;
-  g.drop = 2 * (npass - 1) - 1;
+  const int npass = N > 0 ? fix_npass<true>(N > 0 ? N : 8) : d.npass;
+  g.drop = (HALF ? d.drop : 2 * (npass - 1)) - 1;
   g.B = g.A + (npass > 2 ? lb * ps : 0);
   int* cells = reinterpret_cast<int*>(buf + (npass > 2 ? 2 : 1) * lb * ps);
   g.scale = reinterpret_cast<FixScale*>(cells) + grp * g.nl;
@@ -433,20 +437,24 @@ __global__ void __launch_bounds__(N ? 256 : 384, N ? 3 : 2)
     fixed_middle<N, INV, 1>(g, g.A, g.B, tw, &end);
     constexpr int PL = fix_npass<true>(N) - 1;
     if constexpr (INV)
-      last_inverse<fix_rad<true, true>(N, PL)>(g, end, out, tw + fix_twoff<true, true>(N, PL),
-                                               mul, scaled);
+      last_inverse<fix_rad<true, true>(N, PL), false>(
+          g, end, out, tw + fix_twoff<true, true>(N, PL), mul, scaled);
     else
-      last_forward<fix_rad<true, false>(N, PL)>(g, end, out, tw + fix_twoff<true, false>(N, PL),
-                                                post);
+      last_forward<fix_rad<true, false>(N, PL), false>(
+          g, end, out, tw + fix_twoff<true, false>(N, PL), post);
   } else {
     switch (d.radix[0]) {
       case 8:
-        if constexpr (!INV) first_pass<8, INV, false, 0>(g, in, d.sums, post);
+        if constexpr (!INV && !HALF) first_pass<8, INV, false, 0>(g, in, d.sums, post);
         break;
       case 6: first_pass<6, INV, false, 0>(g, in, d.sums, post); break;
-      case 4: first_pass<4, INV, false, 0>(g, in, d.sums, post); break;
+      case 4:
+        if constexpr (!HALF) first_pass<4, INV, false, 0>(g, in, d.sums, post);
+        break;
       case 3: first_pass<3, INV, false, 0>(g, in, d.sums, post); break;
-      default: first_pass<2, INV, false, 0>(g, in, d.sums, post); break;
+      default:
+        if constexpr (!HALF) first_pass<2, INV, false, 0>(g, in, d.sums, post);
+        break;
     }
     __syncthreads();
     Fix *a = g.A, *b = g.B;
@@ -454,11 +462,17 @@ __global__ void __launch_bounds__(N ? 256 : 384, N ? 3 : 2)
       const int L = d.span[p];
       const int4* t = tw + d.twoff[p];
       switch (d.radix[p]) {
-        case 8: middle_pass<8, INV>(g, a, b, L, t); break;
-        case 6: middle_pass<6, INV>(g, a, b, L, t); break;
-        case 4: middle_pass<4, INV>(g, a, b, L, t); break;
-        case 3: middle_pass<3, INV>(g, a, b, L, t); break;
-        default: middle_pass<2, INV>(g, a, b, L, t); break;
+        case 8:
+          if constexpr (!HALF) middle_pass<8, INV, false>(g, a, b, L, t);
+          break;
+        case 6: middle_pass<6, INV, false>(g, a, b, L, t); break;
+        case 4:
+          if constexpr (!HALF) middle_pass<4, INV, false>(g, a, b, L, t);
+          break;
+        case 3: middle_pass<3, INV, HALF>(g, a, b, L, t); break;
+        default:
+          if constexpr (!HALF) middle_pass<2, INV, false>(g, a, b, L, t);
+          break;
       }
       __syncthreads();
       Fix* s = a;
@@ -468,23 +482,25 @@ __global__ void __launch_bounds__(N ? 256 : 384, N ? 3 : 2)
     const int4* t = tw + d.twoff[npass - 1];
     switch (d.radix[npass - 1]) {
       case 8:
-        if constexpr (INV) last_inverse<8>(g, a, out, t, mul, scaled);
+        if constexpr (INV && !HALF) last_inverse<8, false>(g, a, out, t, mul, scaled);
         break;
       case 6:
-        if constexpr (INV) last_inverse<6>(g, a, out, t, mul, scaled);
-        else last_forward<6>(g, a, out, t, post);
+        if constexpr (INV) last_inverse<6, false>(g, a, out, t, mul, scaled);
+        else last_forward<6, false>(g, a, out, t, post);
         break;
       case 4:
-        if constexpr (INV) last_inverse<4>(g, a, out, t, mul, scaled);
-        else last_forward<4>(g, a, out, t, post);
+        if constexpr (HALF) break;
+        else if constexpr (INV) last_inverse<4, false>(g, a, out, t, mul, scaled);
+        else last_forward<4, false>(g, a, out, t, post);
         break;
       case 3:
-        if constexpr (INV) last_inverse<3>(g, a, out, t, mul, scaled);
-        else last_forward<3>(g, a, out, t, post);
+        if constexpr (INV) last_inverse<3, HALF>(g, a, out, t, mul, scaled);
+        else last_forward<3, HALF>(g, a, out, t, post);
         break;
       default:
-        if constexpr (INV) last_inverse<2>(g, a, out, t, mul, scaled);
-        else last_forward<2>(g, a, out, t, post);
+        if constexpr (HALF) break;
+        else if constexpr (INV) last_inverse<2, false>(g, a, out, t, mul, scaled);
+        else last_forward<2, false>(g, a, out, t, post);
         break;
     }
   }
@@ -529,7 +545,9 @@ static cudaError_t dispatch(const cfs_plan* P, const double* in, double* out, do
     default: break;
   }
   const int T = x_items<INV>(P->M), lb = T >= 192 ? 1 : 192 / T;
-  return go<0, INV>(P, in, out, mul, nl, (lb * T + 31) / 32 * 32, lb, st);
+  const int threads = (lb * T + 31) / 32 * 32;
+  if (P->xfwd.half) return go<kHalved, INV>(P, in, out, mul, nl, threads, lb, st);
+  return go<0, INV>(P, in, out, mul, nl, threads, lb, st);
 }
 
 cudaError_t launch_fix_x(const cfs_plan* P, const double* in, double* out, bool inverse, double mul,

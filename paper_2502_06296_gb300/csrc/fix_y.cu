@@ -10,6 +10,7 @@
 // ALU pipe and by the barriers between the passes of a tile; 3456 x 3072 x 30 11 ms
 // and 3.7 ms (tiles of two columns, one CTA of 24 warps per SM).
 #include "chanfs_fix.cuh"
+#include "chanfs_internal.cuh"
 
 namespace chanfs {
 
@@ -18,15 +19,16 @@ struct YTile {
   int M;           // columns of the field (row stride)
   int valid;       // columns of this tile inside it
   int tk, sh;      // columns of the tile (a power of two), its logarithm
-  int n, headroom, growth, lgpts;
-  int drop;        // 2^-drop: the passes' divisions by 4
+  int n, headroom, growth, lgpts, div;
+  int drop;        // 2^-drop: the passes' divisions
   bool first;      // the tile holds the packed column kx = 0
   Fix *A, *B;
   unsigned *top, *most, *quanta;
 };
 
 __device__ __forceinline__ FixScale scale_of(const YTile& t, int c) {
-  return fix_scale_of(t.top[c], t.most[c], t.quanta[c], t.lgpts, t.growth, t.headroom);
+  return fix_scale_of(t.top[c], t.most[c], t.quanta[c], t.lgpts, t.growth, t.headroom,
+                      t.div);
 }
 
 // Rows of a wall transform: element t of the FFT is row wall_row(t).
@@ -141,21 +143,21 @@ __device__ __forceinline__ void first_pass(const YTile& t, int ytype, bool sums,
   if (on) first_points<R, INV, WALL>(t, j, c, ytype, raw, scale_of(t, c), wy);
 }
 
-template <int R, bool INV>
+template <int R, bool INV, bool HALF>
 __device__ __forceinline__ void middle_pass(const YTile& t, const Fix* in, Fix* out, int L,
                                             const int4* __restrict__ tw) {
   const int Q = t.n / R, items = Q << t.sh;
   for (int it = threadIdx.x; it < items; it += blockDim.x) {
     const int c = it & (t.tk - 1), j = it >> t.sh;
     const int sh = t.sh;
-    fix_butterfly<R, INV>(in, out, j, Q, L, tw, [=](int e) { return fix_pad((e << sh) + c); });
+    fix_butterfly<R, INV, HALF>(in, out, j, Q, L, tw, [=](int e) { return fix_pad((e << sh) + c); });
   }
 }
 
 // The last pass: plain columns to global memory.  A forward wall transform
 // leaves every column in shared memory for the mixing pass, the tile of the
 // packed column leaves that one.
-template <int R, bool INV, bool WALL>
+template <int R, bool INV, bool WALL, bool HALF>
 __device__ __forceinline__ void last_pass(const YTile& t, const Fix* in, Fix* keep, int ytype,
                                           const int4* __restrict__ tw) {
   const int n = t.n, Q = n / R, items = Q << t.sh;
@@ -165,7 +167,7 @@ __device__ __forceinline__ void last_pass(const YTile& t, const Fix* in, Fix* ke
     Fix v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = in[fix_pad(((j + r * Q) << t.sh) + c)];
-    fix_twiddle_dft<R, INV>(v, tw + j, Q);
+    fix_twiddle_dft<R, INV, HALF>(v, tw + j, Q);
     if (!INV && (WALL || (t.first && c == 0))) {
 #pragma unroll
       for (int r = 0; r < R; ++r) keep[fix_pad(((j + r * Q) << t.sh) + c)] = v[r];
@@ -233,7 +235,7 @@ template <int N, bool INV, int P>
 __device__ __forceinline__ void fixed_middle(const YTile& t, Fix* a, Fix* b, const int4* tw,
                                              Fix** end) {
   if constexpr (P + 1 < fix_npass<false>(N)) {
-    middle_pass<fix_rad<false, INV>(N, P), INV>(t, a, b, fix_span<false, INV>(N, P),
+    middle_pass<fix_rad<false, INV>(N, P), INV, false>(t, a, b, fix_span<false, INV>(N, P),
                                                 tw + fix_twoff<false, INV>(N, P));
     __syncthreads();
     fixed_middle<N, INV, P + 1>(t, b, a, tw, end);
@@ -256,17 +258,20 @@ constexpr int y_threads(int n) {
   return ((items << y_shift(items)) + 31) / 32 * 32;
 }
 
-// N > 0: the compile-time length (periodic y); N = 0: any length, from d.  Both
-// ask for 24 warps per SM (80 registers).
+// N > 0: the compile-time length (periodic y); N = 0: any length, from d; N =
+// kHalved: one whose radix-3 passes divide by 2.  All ask for 24 warps per SM (80
+// registers).
 template <int N, bool INV, bool WALL>
-__global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : 768,
-                                  N ? 768 / y_threads(N ? N : 9) : 1)
+__global__ void __launch_bounds__(N > 0 ? y_threads(N > 0 ? N : 9) : 768,
+                                  N > 0 ? 768 / y_threads(N > 0 ? N : 9) : 1)
     fix_y_kernel(double2* data, int M, FixDesc d, const int4* __restrict__ tw,
                  const int4* __restrict__ wy, int shift, int ytype) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int n = N ? N : d.n;
-  const int npass = N ? fix_npass<false>(N ? N : 8) : d.npass;
-  const int sh = N ? y_shift((N ? N : 9) / fix_radix<false>(N ? N : 9, 0)) : shift;
+  constexpr bool HALF = N == kHalved;
+  const int n = N > 0 ? N : d.n;
+  const int npass = N > 0 ? fix_npass<false>(N > 0 ? N : 8) : d.npass;
+  const int sh =
+      N > 0 ? y_shift((N > 0 ? N : 9) / fix_radix<false>(N > 0 ? N : 9, 0)) : shift;
   YTile t;
   t.n = n;
   t.M = M;
@@ -278,9 +283,10 @@ __global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : 768,
   t.col = data + (size_t)blockIdx.y * n * M + x0;
   // (an inverse wall transform's V_e is up to |X_e| + |X_{N-e}|)
   t.headroom = INV && WALL ? 60 : 61;
-  t.growth = N ? fix_growth<false, INV>(N ? N : 9) : d.growth;
-  t.lgpts = fix_ceil_log2(4 * (N ? fix_rad<false, INV>(N ? N : 9, 0) : d.radix[0]));
-  t.drop = 2 * (npass - 1);
+  t.growth = N > 0 ? fix_growth<false, INV>(N > 0 ? N : 9) : d.growth;
+  t.div = HALF ? d.div : 2;
+  t.drop = HALF ? d.drop : 2 * (npass - 1);
+  t.lgpts = fix_ceil_log2(4 * (N > 0 ? fix_rad<false, INV>(N > 0 ? N : 9, 0) : d.radix[0]));
   const int pts = n << sh, buf = pts + (pts >> 3);
   t.A = reinterpret_cast<Fix*>(smem_raw);
   t.B = t.A + buf;
@@ -296,26 +302,38 @@ __global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : 768,
     fixed_middle<N, INV, 1>(t, t.A, t.B, tw, &a);
     b = a == t.A ? t.B : t.A;
     constexpr int PL = fix_npass<false>(N) - 1;
-    last_pass<fix_rad<false, INV>(N, PL), INV, false>(t, a, b, ytype,
-                                                      tw + fix_twoff<false, INV>(N, PL));
+    last_pass<fix_rad<false, INV>(N, PL), INV, false, false>(t, a, b, ytype,
+                                                             tw + fix_twoff<false, INV>(N, PL));
   } else {
     switch (d.radix[0]) {
-      case 8: first_pass<8, INV, WALL>(t, ytype, d.sums, wy); break;
+      case 8:
+        if constexpr (!HALF) first_pass<8, INV, WALL>(t, ytype, d.sums, wy);
+        break;
       case 6: first_pass<6, INV, WALL>(t, ytype, d.sums, wy); break;
-      case 4: first_pass<4, INV, WALL>(t, ytype, d.sums, wy); break;
+      case 4:
+        if constexpr (!HALF) first_pass<4, INV, WALL>(t, ytype, d.sums, wy);
+        break;
       case 3: first_pass<3, INV, WALL>(t, ytype, d.sums, wy); break;
-      default: first_pass<2, INV, WALL>(t, ytype, d.sums, wy); break;
+      default:
+        if constexpr (!HALF) first_pass<2, INV, WALL>(t, ytype, d.sums, wy);
+        break;
     }
     __syncthreads();
     for (int p = 1; p + 1 < npass; ++p) {
       const int L = d.span[p];
       const int4* w = tw + d.twoff[p];
       switch (d.radix[p]) {
-        case 8: middle_pass<8, INV>(t, a, b, L, w); break;
-        case 6: middle_pass<6, INV>(t, a, b, L, w); break;
-        case 4: middle_pass<4, INV>(t, a, b, L, w); break;
-        case 3: middle_pass<3, INV>(t, a, b, L, w); break;
-        default: middle_pass<2, INV>(t, a, b, L, w); break;
+        case 8:
+          if constexpr (!HALF) middle_pass<8, INV, false>(t, a, b, L, w);
+          break;
+        case 6: middle_pass<6, INV, false>(t, a, b, L, w); break;
+        case 4:
+          if constexpr (!HALF) middle_pass<4, INV, false>(t, a, b, L, w);
+          break;
+        case 3: middle_pass<3, INV, HALF>(t, a, b, L, w); break;
+        default:
+          if constexpr (!HALF) middle_pass<2, INV, false>(t, a, b, L, w);
+          break;
       }
       __syncthreads();
       Fix* s = a;
@@ -324,11 +342,17 @@ __global__ void __launch_bounds__(N ? y_threads(N ? N : 9) : 768,
     }
     const int4* w = tw + d.twoff[npass - 1];
     switch (d.radix[npass - 1]) {
-      case 8: last_pass<8, INV, WALL>(t, a, b, ytype, w); break;
-      case 6: last_pass<6, INV, WALL>(t, a, b, ytype, w); break;
-      case 4: last_pass<4, INV, WALL>(t, a, b, ytype, w); break;
-      case 3: last_pass<3, INV, WALL>(t, a, b, ytype, w); break;
-      default: last_pass<2, INV, WALL>(t, a, b, ytype, w); break;
+      case 8:
+        if constexpr (!HALF) last_pass<8, INV, WALL, false>(t, a, b, ytype, w);
+        break;
+      case 6: last_pass<6, INV, WALL, false>(t, a, b, ytype, w); break;
+      case 4:
+        if constexpr (!HALF) last_pass<4, INV, WALL, false>(t, a, b, ytype, w);
+        break;
+      case 3: last_pass<3, INV, WALL, HALF>(t, a, b, ytype, w); break;
+      default:
+        if constexpr (!HALF) last_pass<2, INV, WALL, false>(t, a, b, ytype, w);
+        break;
     }
   }
   if constexpr (!INV) {
@@ -373,6 +397,7 @@ static cudaError_t dispatch(const cfs_plan* P, double* data, cudaStream_t st) {
       default: break;
     }
   }
+  if (P->yfwd.half) return go<kHalved, INV, WALL>(P, data, sh, threads, st);
   return go<0, INV, WALL>(P, data, sh, threads, st);
 }
 

@@ -56,49 +56,6 @@ bool make_fft_desc(int n, FftDesc* d, std::vector<double2>* tw, int max_radix) {
   return true;
 }
 
-// exp(-+2 pi i e / n) in units of 2^-62, the low words signed.  The values of
-// an eighth of the circle are computed once, in long double; the others are
-// their reflections.
-class FixRoots {
- public:
-  explicit FixRoots(int n) : n_(n) {
-    const long double half_pi = 1.57079632679489661923132169163975144L;
-    for (int r = 0; 2 * r <= n; r += 4) add(half_pi * (long double)r / (long double)n);
-    if (n % 4) {  // the remainders of 4 e / n run over more than multiples of 4
-      cs_.clear();
-      for (int r = 0; 2 * r <= n; ++r) add(half_pi * (long double)r / (long double)n);
-    }
-  }
-  int4 at(long long e, bool conj) const {
-    e %= n_;
-    const long long q = 4 * e / n_, rest = 4 * e - q * n_;  // quarter turns, rest / n of the next
-    const bool swap = 2 * rest > n_;
-    const long long i = swap ? n_ - rest : rest;
-    const longlong2 cs = cs_[n_ % 4 ? i : i / 4];
-    const long long u = swap ? cs.y : cs.x, v = swap ? cs.x : cs.y;
-    const long long re = q == 0 ? u : q == 1 ? -v : q == 2 ? -u : v;
-    const long long im = q == 0 ? v : q == 1 ? u : q == 2 ? -v : -u;  // e^{+i angle}
-    int4 w;
-    split(re, &w.x, &w.y);
-    split(conj ? im : -im, &w.z, &w.w);
-    return w;
-  }
-
- private:
-  void add(long double a) {
-    cs_.push_back(make_longlong2(llroundl(cosl(a) * 4611686018427387904.0L),
-                                 llroundl(sinl(a) * 4611686018427387904.0L)));
-  }
-  static void split(long long x, int* hi, int* lo) {
-    long long l = (long long)(int)(x & 0xffffffffll);
-    if (l == -2147483648ll) l = -2147483647ll;  // its negative is used too
-    *hi = (int)((x - l) >> 32);
-    *lo = (int)l;
-  }
-  long long n_;
-  std::vector<longlong2> cs_;
-};
-
 // Passes of a block fixed-point transform, and its twiddles appended to tw.
 // (roots: of a multiple of n)
 template <bool PAIR, bool INV>
@@ -109,6 +66,9 @@ static void make_fix_desc(int n, FixDesc* d, std::vector<int4>* tw, const FixRoo
   d->npass = fix_npass<PAIR>(n);
   d->growth = fix_growth<PAIR, INV>(n);
   d->sums = fix_uses_sum<PAIR, INV>(n);
+  d->half = fix_halves<PAIR>(n);
+  d->div = fix_div<PAIR, INV>(n, 1);
+  d->drop = fix_drop<PAIR, INV>(n);
   for (int p = 0; p < d->npass; ++p) {
     const int R = d->radix[p] = fix_rad<PAIR, INV>(n, p);
     const int L = d->span[p] = fix_span<PAIR, INV>(n, p);
