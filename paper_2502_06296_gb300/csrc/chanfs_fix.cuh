@@ -357,12 +357,6 @@ template <int R, bool INV> __device__ __forceinline__ void fdft(Fix* v) {
 
 // --- the scale of a line ----------------------------------------------------
 
-__host__ __device__ constexpr int fix_ceil_log2(int v) {
-  int b = 0;
-  while ((1 << b) < v) ++b;
-  return b;
-}
-
 // Adds |v| to a butterfly's maximum (as the high word of a double) and to its sum
 // (as a float from the double's leading bits; values outside the range of
 // floats are below every bound that the sum is used for, or switch it off).
@@ -371,63 +365,104 @@ __device__ __forceinline__ void fix_gather(double v, unsigned& top, float& sum) 
   top = max(top, u);
   sum += __uint_as_float((max(u, 0x38100000u) - 0x38000000u) << 3);
 }
+template <int N> __device__ __forceinline__ void fix_gather(const double2* v, unsigned& top, float& sum) {
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    fix_gather(v[r].x, top, sum);
+    fix_gather(v[r].y, top, sum);
+  }
+}
 
-// A line's scale.  kind 0: the conversions by shifts; kind 1: by the library's
-// scalbn (a line of subnormals, or with values beyond 2^+-900); kind 2: an
-// infinity or NaN (every output of the line is then NaN).
+// A line's scale, and how its results leave.  kind 0: by a shift of the exponent;
+// kind 1: by the library's scalbn (a line that was moved first, see fix_move); kind
+// 2: an infinity or NaN (every output of the line is then NaN).
 struct FixScale {
   int s, kind;
 };
 
-__device__ __forceinline__ bool fix_summed(unsigned top) { return (top >> 20) - 933u <= 180u; }
+// Whether a line whose largest value has this high word is scaled as it is: within
+// 2^+-90, where its sums fit the floats.
+__device__ __forceinline__ bool fix_near(unsigned top) { return (top >> 20) - 933u <= 180u; }
+
+// A line farther from 1 is moved first: all its values times 2^k, which brings its
+// largest near 1, exactly (what that takes below the subnormals is below 2^-1000 of
+// the largest).  So a power of two in the data comes out as that power of two, to
+// the last bit.  A line of subnormals moves to 1 .. 2^52.  (In registers, between two
+// reductions: the conversions have one form then.  Stages at 512 x 384 x 384 x 330 us
+// forward and 341 inverse, y 438 and 441, without any move 324, 333, 432 and 439; at
+// 384 x 256 x 192 between walls in y 161 and 170 against 167 and 186.)
+__device__ __forceinline__ int fix_move(unsigned top) {
+  const int e = (int)(top >> 20);
+  return fix_near(top) || e == 0x7ff ? 0 : e ? 1023 - e : 1074;
+}
+__device__ __forceinline__ double fix_moved(double v, int k) {  // |k| <= 1074
+  const int h = k / 2;
+  return v * __hiloint2double((1023 + h) << 20, 0) * __hiloint2double((1023 + k - h) << 20, 0);
+}
+// A thread's values moved, and gathered again.
+template <int N>
+__device__ __forceinline__ void fix_gather_moved(double2* v, int k, unsigned& top, float& sum) {
+  if (k) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) v[r] = make_double2(fix_moved(v[r].x, k), fix_moved(v[r].y, k));
+  }
+  top = 0u;
+  sum = 0.0f;
+  fix_gather<N>(v, top, sum);
+}
+// Whether a line must be moved, as far as one thread knows: from its largest value,
+// or, where that is 0 or below 2^-1042, from the thread's own.
+template <int N> __device__ __forceinline__ bool fix_far(unsigned top, const double2* v) {
+  if (top) return fix_move(top) != 0;
+  int low = 0;
+#pragma unroll
+  for (int r = 0; r < N; ++r) low |= __double2loint(v[r].x) | __double2loint(v[r].y);
+  return low != 0;
+}
 
 // A butterfly's sum in units of 2^-19 of the power of two above the largest one
 // (integers add up to the same in any order); 0 if the line does not use it.
 __device__ __forceinline__ unsigned fix_quanta(float sum, unsigned top, unsigned most) {
-  if (!fix_summed(top)) return 0u;
+  if (!fix_near(top)) return 0u;
   return __float2uint_ru(sum * __uint_as_float((272u - ((most + 256u) >> 23)) << 23));
 }
 
-// The scale, from the line's largest value (high word), largest butterfly sum B
-// (float bits) and, unless it is 0, the sum of the butterflies' quanta; where
-// the maximum is far from 1, from the maximum and the points of a butterfly.  A
+// The scale of a (moved) line, from its largest value (high word), largest butterfly
+// sum B (float bits) and, unless it is 0, the sum of the butterflies' quanta.  A
 // line of zeros takes s = 0.
 __device__ __forceinline__ FixScale fix_scale_of(unsigned top, unsigned most, unsigned quanta,
-                                                 int lgpts, int growth, int headroom, int div) {
-  const int e = (int)(top >> 20);
-  if (fix_summed(top)) {
-    const int eb = (int)((most + 256u) >> 23) - 126;  // B < 2^eb
-    int ec = eb + growth;
-    // S / D_2 < 2^(eb - 19 + bits(quanta) - div)
-    if (quanta) ec = max(eb, min(ec, eb + 13 - div - __clz((int)quanta)));
-    return {headroom - ec, 0};
-  }
-  if (top == 0u) return {0, 0};
-  return {e == 0x7ff ? 0 : headroom - growth - (max(e, 1) - 1022 + lgpts),
-          e == 0x7ff ? 2 : (e < 123 || e > 1923) ? 1 : 0};
+                                                 int growth, int headroom, int div) {
+  if (!fix_near(top)) return {0, top >= 0x7ff00000u ? 2 : 0};
+  const int eb = (int)((most + 256u) >> 23) - 126;  // B < 2^eb
+  int ec = eb + growth;
+  // S / D_2 < 2^(eb - 19 + bits(quanta) - div)
+  if (quanta) ec = max(eb, min(ec, eb + 13 - div - __clz((int)quanta)));
+  return {headroom - ec, 0};
+}
+// The scale of the line before it was moved by 2^k.
+__device__ __forceinline__ FixScale fix_moved_back(FixScale f, int k) {
+  return {f.s + k, k ? 1 : f.kind};
 }
 
-static __device__ __noinline__ long long fix_from_far(double v, FixScale f) {
-  return f.kind == 2 ? 0ll : __double2ll_rn(scalbn(v, f.s));
-}
 static __device__ __noinline__ double fix_to_far(long long v, int s, int kind) {
   return kind == 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)v, -s);
 }
 
-// trunc(v 2^s): the significand, its leading bit at 62, shifted down.
-__device__ __forceinline__ long long fix_from(double v, FixScale f) {
-  if (f.kind) return fix_from_far(v, f);
+// trunc(v 2^s): the significand, its leading bit at 62, shifted down.  (In a line
+// with an infinity or NaN the shift may be out of range: any value will do.)
+__device__ __forceinline__ long long fix_from(double v, int s) {
   const int hi = __double2hiint(v);
   const unsigned lo = (unsigned)__double2loint(v);
-  const int t = 1085 - f.s - (int)(((unsigned)hi & 0x7fffffffu) >> 20);
+  const int t = 1085 - s - (int)(((unsigned)hi & 0x7fffffffu) >> 20);
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
   const unsigned long long m =
-      ((((unsigned long long)__funnelshift_l(lo, mh, 10)) << 32) | (lo << 10)) >> min(t, 63);
+      ((((unsigned long long)__funnelshift_l(lo, mh, 10)) << 32) | (lo << 10)) >>
+      min((unsigned)t, 63u);
   const long long sg = hi >> 31;
   return ((long long)m ^ sg) - sg;
 }
-__device__ __forceinline__ Fix fix_from(double2 v, FixScale f) {
-  return {fix_from(v.x, f), fix_from(v.y, f)};
+__device__ __forceinline__ Fix fix_from(double2 v, int s) {
+  return {fix_from(v.x, s), fix_from(v.y, s)};
 }
 
 // v 2^-s, rounded to nearest (the exponent is adjusted on the encoding).

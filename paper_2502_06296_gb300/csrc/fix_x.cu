@@ -133,26 +133,35 @@ template <bool WARP> __device__ __forceinline__ void group_sync() {
   else __syncthreads();
 }
 
+template <bool WARP> __device__ __forceinline__ bool group_any(bool v) {
+  if constexpr (WARP) return __any_sync(~0u, v);
+  else return __syncthreads_or(v);
+}
+
 // The maxima over the T items of each line (item lane of the group in line lane
 // / T) of the values' magnitudes and of the butterflies' sums, and the sum of
-// their quanta: the same on every thread of a line.
+// their quanta: the same on every thread of a line.  line_max also says whether a
+// line of the group may have to be moved (fix_move), the same to the whole group.
 template <bool WARP, int T>
 __device__ __forceinline__ bool warp_lead(const XGroup& g) {  // a warp's items share a line
   return T ? T % 32 == 0 : g.nl == 1;
 }
 template <bool WARP, int T>
-__device__ __forceinline__ void line_max(const XGroup& g, int l, bool on, unsigned& top,
+__device__ __forceinline__ bool line_max(const XGroup& g, int l, bool on, unsigned& top,
                                          unsigned& most) {
   if constexpr (WARP && T == 32) {
     top = __reduce_max_sync(~0u, top);
     most = __reduce_max_sync(~0u, most);
+    return !fix_near(top);
   } else if constexpr (WARP) {
 #pragma unroll
     for (int o = 1; o < T; o *= 2) {
       top = max(top, __shfl_xor_sync(~0u, top, o));
       most = max(most, __shfl_xor_sync(~0u, most, o));
     }
+    return __any_sync(~0u, !fix_near(top));
   } else {
+    const bool odd = on && !fix_near(top);
     if (warp_lead<WARP, T>(g)) {
       top = __reduce_max_sync(~0u, top);
       most = __reduce_max_sync(~0u, most);
@@ -162,9 +171,10 @@ __device__ __forceinline__ void line_max(const XGroup& g, int l, bool on, unsign
       atomicMax(g.top + l, top);
       atomicMax(g.most + l, most);
     }
-    __syncthreads();
+    const bool any = __syncthreads_or(odd);
     top = g.top[l];
     most = g.most[l];
+    return any;
   }
 }
 template <bool WARP, int T>
@@ -188,9 +198,8 @@ __device__ __forceinline__ unsigned line_sum(const XGroup& g, int l, bool on, un
 
 // Item it of the first pass: forward, butterfly j of line l (R points j + r Q);
 // inverse, the pairs of item i (2 R points, and the point 0 of item 0).
-template <int R, bool INV, int NRAW>
-__device__ __forceinline__ void load_item(const double2* line, int n, int Q, int i, double2* raw,
-                                          unsigned& top, float& sum) {
+template <int R, bool INV>
+__device__ __forceinline__ void load_item(const double2* line, int n, int Q, int i, double2* raw) {
   if constexpr (!INV) {
 #pragma unroll
     for (int r = 0; r < R; ++r) raw[r] = line[i + r * Q];
@@ -205,22 +214,17 @@ __device__ __forceinline__ void load_item(const double2* line, int n, int Q, int
     }
     raw[2 * R] = z ? line[0] : make_double2(0.0, 0.0);
   }
-#pragma unroll
-  for (int r = 0; r < NRAW; ++r) {
-    fix_gather(raw[r].x, top, sum);
-    fix_gather(raw[r].y, top, sum);
-  }
 }
 
 // The first pass's arithmetic on a loaded item, written to buffer A.
 template <int R, bool INV>
 __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, int Q, int i,
-                                           const double2* raw, FixScale f,
+                                           const double2* raw, int s,
                                            const int4* __restrict__ post) {
   if constexpr (!INV) {
     Fix v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = fix_from(raw[r], f);
+    for (int r = 0; r < R; ++r) v[r] = fix_from(raw[r], s);
     fdft<R, false>(v);
 #pragma unroll
     for (int r = 0; r < R; ++r) line[fix_pad(i * R + r)] = v[r];
@@ -229,7 +233,7 @@ __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, in
     Fix a[R], b[R], p[R], q[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {  // 2 Z_k = E + i conj(W^k) T, T = X_k - conj X_{M-k}
-      const Fix xk = fix_from(raw[2 * r], f), xm = fix_from(raw[2 * r + 1], f);
+      const Fix xk = fix_from(raw[2 * r], s), xm = fix_from(raw[2 * r + 1], s);
       const Fix e = {xk.x + xm.x, xk.y - xm.y};
       const Fix u = fmul(Fix{xk.x - xm.x, xk.y + xm.y},
                          __ldg(post + pair_index<R>(z, i, r, Q)));
@@ -238,7 +242,7 @@ __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, in
     }
     pair_give<R>(z, p, q, a, b);
     if (z) {
-      const Fix x0 = fix_from(raw[2 * R], f);  // (X_0, X_M)
+      const Fix x0 = fix_from(raw[2 * R], s);  // (X_0, X_M)
       a[0] = {x0.x + x0.y, x0.x - x0.y};
     }
     fdft<R, true>(a);
@@ -271,17 +275,30 @@ __device__ __forceinline__ void first_pass(const XGroup& g, const double2* in, b
   double2 raw[NRAW];
   unsigned top = 0u, quanta = 0u;
   float sum = 0.0f;
-  if (on) load_item<R, INV, NRAW>(in + (g.line0 + l) * g.n, g.n, Q, i, raw, top, sum);
+  if (on) {
+    load_item<R, INV>(in + (g.line0 + l) * g.n, g.n, Q, i, raw);
+    fix_gather<NRAW>(raw, top, sum);
+  }
   if constexpr (!WARP) __syncthreads();  // the reduction's cells are cleared
   unsigned most = __float_as_uint(sum);
-  line_max<WARP, T>(g, l, on, top, most);
+  int k = 0;
+  if (line_max<WARP, T>(g, l, on, top, most) &&
+      group_any<WARP>(on && fix_far<NRAW>(top, raw))) {  // seldom: the group gathers again
+    k = fix_move(top);
+    if constexpr (!WARP) {
+      if (on && i == 0) g.top[l] = g.most[l] = 0u;
+      __syncthreads();
+    }
+    if (on) fix_gather_moved<NRAW>(raw, k, top, sum);
+    most = __float_as_uint(sum);
+    line_max<WARP, T>(g, l, on, top, most);
+  }
   if (sums)
     quanta = line_sum<WARP, T>(g, l, on, on ? (INV ? 2u : 1u) * fix_quanta(sum, top, most) : 0u);
   if (on) {
-    const FixScale f =
-        fix_scale_of(top, most, quanta, fix_ceil_log2(4 * R), g.growth, g.headroom, g.div);
-    if (i == 0) g.scale[l] = f;
-    first_item<R, INV>(g, g.A + l * g.ps, g.n, Q, i, raw, f, post);
+    const FixScale f = fix_scale_of(top, most, quanta, g.growth, g.headroom, g.div);
+    if (i == 0) g.scale[l] = fix_moved_back(f, k);
+    first_item<R, INV>(g, g.A + l * g.ps, g.n, Q, i, raw, f.s, post);
   }
 }
 

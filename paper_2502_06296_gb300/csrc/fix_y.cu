@@ -19,16 +19,20 @@ struct YTile {
   int M;           // columns of the field (row stride)
   int valid;       // columns of this tile inside it
   int tk, sh;      // columns of the tile (a power of two), its logarithm
-  int n, headroom, growth, lgpts, div;
+  int n, headroom, growth, div;
   int drop;        // 2^-drop: the passes' divisions
   bool first;      // the tile holds the packed column kx = 0
   Fix *A, *B;
   unsigned *top, *most, *quanta;
+  int* move;       // powers of two that the columns were moved by (fix_move)
 };
 
+// The scale of column c as it was moved, and of its results.
+__device__ __forceinline__ FixScale moved_scale(const YTile& t, int c) {
+  return fix_scale_of(t.top[c], t.most[c], t.quanta[c], t.growth, t.headroom, t.div);
+}
 __device__ __forceinline__ FixScale scale_of(const YTile& t, int c) {
-  return fix_scale_of(t.top[c], t.most[c], t.quanta[c], t.lgpts, t.growth, t.headroom,
-                      t.div);
+  return fix_moved_back(moved_scale(t, c), t.move[c]);
 }
 
 // Rows of a wall transform: element t of the FFT is row wall_row(t).
@@ -65,19 +69,13 @@ __device__ __forceinline__ double2 load_packed(const YTile& t, int e) {
 }
 
 template <int R, bool INV, bool WALL>
-__device__ __forceinline__ void load_points(const YTile& t, int j, int c, int ytype, double2* raw,
-                                            unsigned& top, float& sum) {
+__device__ __forceinline__ void load_points(const YTile& t, int j, int c, int ytype, double2* raw) {
   const int Q = t.n / R;
   if (INV && !WALL && t.first && c == 0) {
     for (int r = 0; r < R; ++r) raw[r] = load_packed(t, j + r * Q);
   } else {
 #pragma unroll
     for (int r = 0; r < R; ++r) raw[r] = load_elem<INV, WALL>(t, j + r * Q, c, ytype);
-  }
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    fix_gather(raw[r].x, top, sum);
-    fix_gather(raw[r].y, top, sum);
   }
 }
 
@@ -90,17 +88,17 @@ __device__ __forceinline__ Fix wall_unmix(Fix xe, Fix xn, int4 wconj) {
 
 template <int R, bool INV, bool WALL>
 __device__ __forceinline__ void first_points(const YTile& t, int j, int c, int ytype,
-                                             const double2* raw, FixScale f,
+                                             const double2* raw, int s,
                                              const int4* __restrict__ wy) {
   const int Q = t.n / R;
   Fix v[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    v[r] = fix_from(raw[r], f);
+    v[r] = fix_from(raw[r], s);
     if constexpr (INV && WALL) {
       const int e = j + r * Q;
       if (e > 0) {
-        const Fix xn = fix_from(load_elem<INV, WALL>(t, t.n - e, c, ytype), f);
+        const Fix xn = fix_from(load_elem<INV, WALL>(t, t.n - e, c, ytype), s);
         v[r] = wall_unmix(v[r], xn, __ldg(wy + e));
       }
     }
@@ -121,26 +119,51 @@ __device__ __forceinline__ void first_pass(const YTile& t, int ytype, bool sums,
   double2 raw[R];
   unsigned top = 0u;
   float sum = 0.0f;
-  if (on) load_points<R, INV, WALL>(t, j, c, ytype, raw, top, sum);
+  if (on) {
+    load_points<R, INV, WALL>(t, j, c, ytype, raw);
+    fix_gather<R>(raw, top, sum);
+  }
   __syncthreads();  // the reduction's cells are cleared
-  unsigned most = __float_as_uint(sum);
   const bool lead = (threadIdx.x & 31) < t.tk;
-  for (int o = t.tk; o < 32; o *= 2) {
-    top = max(top, __shfl_xor_sync(~0u, top, o));
-    most = max(most, __shfl_xor_sync(~0u, most, o));
+  const auto column_max = [&] {  // whether a column of the tile may have to be moved
+    unsigned u = top, v = __float_as_uint(sum);
+    for (int o = t.tk; o < 32; o *= 2) {
+      u = max(u, __shfl_xor_sync(~0u, u, o));
+      v = max(v, __shfl_xor_sync(~0u, v, o));
+    }
+    if (lead) {
+      atomicMax(t.top + c, u);
+      atomicMax(t.most + c, v);
+    }
+    return __syncthreads_or(on && !fix_near(top));
+  };
+  if (column_max()) {
+    const unsigned all = t.top[c];
+    if (__syncthreads_or(on && fix_far<R>(all, raw))) {  // seldom: the tile gathers again
+      const int k = fix_move(all);
+      if (threadIdx.x < t.tk) t.top[c] = t.most[c] = 0u;
+      __syncthreads();
+      if (on) {
+        fix_gather_moved<R>(raw, k, top, sum);
+        t.move[c] = k;  // the same from every thread of the column
+        if constexpr (INV && WALL) {  // mirrored points are read again
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int e = j + r * (t.n / R);
+            t.col[c + (size_t)(ytype == kSin ? t.n - 1 - e : e) * t.M] = raw[r];
+          }
+        }
+      }
+      column_max();
+    }
   }
-  if (lead) {
-    atomicMax(t.top + c, top);
-    atomicMax(t.most + c, most);
-  }
-  __syncthreads();
   if (sums) {
     unsigned q = on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
     for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
     if (lead) atomicAdd(t.quanta + c, q);
     __syncthreads();
   }
-  if (on) first_points<R, INV, WALL>(t, j, c, ytype, raw, scale_of(t, c), wy);
+  if (on) first_points<R, INV, WALL>(t, j, c, ytype, raw, moved_scale(t, c).s, wy);
 }
 
 template <int R, bool INV, bool HALF>
@@ -286,14 +309,14 @@ __global__ void __launch_bounds__(N > 0 ? y_threads(N > 0 ? N : 9) : 768,
   t.growth = N > 0 ? fix_growth<false, INV>(N > 0 ? N : 9) : d.growth;
   t.div = HALF ? d.div : 2;
   t.drop = HALF ? d.drop : 2 * (npass - 1);
-  t.lgpts = fix_ceil_log2(4 * (N > 0 ? fix_rad<false, INV>(N > 0 ? N : 9, 0) : d.radix[0]));
   const int pts = n << sh, buf = pts + (pts >> 3);
   t.A = reinterpret_cast<Fix*>(smem_raw);
   t.B = t.A + buf;
   t.top = reinterpret_cast<unsigned*>(t.B + buf);
   t.most = t.top + t.tk;
   t.quanta = t.most + t.tk;
-  for (int e = threadIdx.x; e < 3 * t.tk; e += blockDim.x) t.top[e] = 0u;
+  t.move = reinterpret_cast<int*>(t.quanta + t.tk);
+  for (int e = threadIdx.x; e < 4 * t.tk; e += blockDim.x) t.top[e] = 0u;
   Fix *a = t.A, *b = t.B;
   if constexpr (N > 0) {
     first_pass<fix_rad<false, INV>(N, 0), INV, false>(t, ytype, fix_uses_sum<false, INV>(N),
@@ -366,7 +389,7 @@ __global__ void __launch_bounds__(N > 0 ? y_threads(N > 0 ? N : 9) : 768,
 
 static size_t y_smem(int n, int sh) {
   const size_t pts = (size_t)n << sh;
-  return 2 * (pts + (pts >> 3)) * sizeof(Fix) + ((size_t)3 << sh) * sizeof(unsigned);
+  return 2 * (pts + (pts >> 3)) * sizeof(Fix) + ((size_t)4 << sh) * sizeof(unsigned);
 }
 
 template <int N, bool INV, bool WALL>

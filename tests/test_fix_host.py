@@ -38,7 +38,6 @@ static unsigned __funnelshift_l(unsigned lo, unsigned hi, unsigned s) {
 static unsigned __float2uint_ru(float f) { return (unsigned)ceilf(f); }
 static int __clz(int v) { return v ? __builtin_clz((unsigned)v) : 32; }
 static double __ll2double_rn(long long v) { return (double)v; }
-static long long __double2ll_rn(double v) { return llrint(v); }
 template <class T> static T __ldg(const T* p) { return *p; }
 #include "chanfs_fix.cuh"
 using namespace chanfs;
@@ -62,19 +61,16 @@ template <bool PAIR, bool INV> static void run(int n, const double2* in, double2
     std::vector<float> sums;
     for (int j = 0; j < Q; ++j) {
       float sum = 0;
-      for (int r = 0; r < R; ++r) {
-        fix_gather(in[j + r * Q].x, top, sum);
-        fix_gather(in[j + r * Q].y, top, sum);
-      }
+      for (int r = 0; r < R; ++r) fix_gather<1>(in + j + r * Q, top, sum);
       most = max(most, __float_as_uint(sum));
       sums.push_back(sum);
     }
     if (fix_uses_sum<PAIR, INV>(n))
       for (float s : sums) quanta += fix_quanta(s, top, most);
-    f = fix_scale_of(top, most, quanta, fix_ceil_log2(4 * R), fix_growth<PAIR, INV>(n), 61, fix_div<PAIR, INV>(n, 1));
+    f = fix_scale_of(top, most, quanta, fix_growth<PAIR, INV>(n), 61, fix_div<PAIR, INV>(n, 1));
     for (int j = 0; j < Q; ++j) {
       Fix v[R];
-      for (int r = 0; r < R; ++r) v[r] = fix_from(in[j + r * Q], f);
+      for (int r = 0; r < R; ++r) v[r] = fix_from(in[j + r * Q], f.s);
       fdft<R, INV>(v);
       for (int r = 0; r < R; ++r) a[j * R + r] = v[r];
     }

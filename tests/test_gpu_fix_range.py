@@ -8,6 +8,7 @@ import pytest
 torch = pytest.importorskip("torch")
 fft = pytest.importorskip("scipy.fft")
 pytestmark = pytest.mark.gpu
+X_FORWARD, Y_FORWARD, Y_INVERSE = 0, 1, 3  # stages of cfs_poisson_stage
 
 
 @pytest.fixture(scope="module")
@@ -68,3 +69,63 @@ def check(chanfs, nx, ny, kind):
                                    (24, 243), (16, 486), (36, 729)])
 def test_lengths_of_many_radix_3_passes(chanfs, nx, ny, kind):
     check(chanfs, nx, ny, kind)
+
+
+def same_values(a, b):
+    return np.array_equal(a, b)  # (-0 and 0 alike)
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 3), (216, 48), (162, 27), (32, 3), (96, 243), (1536, 4), (24, 9), (64, 16)])
+def test_powers_of_two_come_out_as_they_went_in(chanfs, nx, ny):
+    """Every plane times its own power of two, near and far from 1: the same bits times that power, both ways.
+    Planes of one power fill blocks of lines; with few lines per plane, blocks hold several powers."""
+    e = np.array([0, 100, -100, 3, -300, 600, -700, 900, -950, 91, -91])
+    nz = e.size
+    f = np.random.default_rng(nx * ny).standard_normal((nz, ny, nx))
+    f[2, :, nx // 2:] = 0.0  # (lone threads with nothing but zeros, beside a far line)
+    f[3] *= 1e-40            # (a far line, as its own power leaves it)
+    g = np.ldexp(f, e[:, None, None])
+    with chanfs.Plan(nx, ny, nz, 2.0, 1.0, np.full(nz, 0.5)) as plan:
+        base = plan.spectral_forward(torch.from_numpy(f).cuda())
+        back = plan.spectral_inverse(base).cpu().numpy()
+        base = base.cpu().numpy()
+        s = plan.spectral_forward(torch.from_numpy(g).cuda()).cpu().numpy()
+        t = plan.spectral_inverse(torch.from_numpy(np.ldexp(base, e[:, None, None])).cuda()).cpu().numpy()
+        tiny = np.random.default_rng(1).integers(-9, 10, f.shape).astype(float)
+        tiny[1] = 0.0
+        x = lambda f: plan.poisson_stage(X_FORWARD, torch.from_numpy(f).cuda()).cpu().numpy()
+        base_tiny, low = x(tiny), x(np.ldexp(tiny, -1074))
+        assert plan.check() == 0
+    assert same_values(s, np.ldexp(base, e[:, None, None]))
+    assert same_values(t, np.ldexp(back, e[:, None, None]))
+    assert not low[1].any()
+    # subnormal data along x: the result rounded once to the units of the type (and once before, to 53 bits)
+    assert np.max(np.abs(np.ldexp(low, 1074) - base_tiny)) <= 0.5 + 2.0**-40
+
+
+@pytest.mark.parametrize("ybc", [0, 1, 2])
+@pytest.mark.parametrize("nx,ny", [(64, 16), (54, 27), (36, 48), (72, 243), (48, 162), (128, 512)])
+def test_columns_of_a_tile_keep_their_own_powers(chanfs, nx, ny, ybc):
+    """The y transforms alone, neighbouring columns far apart in magnitude."""
+    nz = 3
+    rng = np.random.default_rng(nx + ny)
+    e = np.repeat(rng.choice([0, 0, 120, -120, 700, -800], nx // 2), 2)
+    f = rng.standard_normal((nz, ny, nx))
+    with chanfs.Plan(nx, ny, nz, 2.0, 1.0, np.full(nz, 0.5), 0, 0, ybc) as plan:
+        for stage in (Y_FORWARD, Y_INVERSE):
+            base = plan.poisson_stage(stage, torch.from_numpy(f).cuda()).cpu().numpy()
+            got = plan.poisson_stage(stage, torch.from_numpy(np.ldexp(f, e)).cuda()).cpu().numpy()
+            assert same_values(got, np.ldexp(base, e)), stage
+        assert plan.check() == 0
+
+
+def test_far_long_columns_keep_their_bits(chanfs):
+    """White noise times 2^-100 along 768 and 1024 points, which the line's sum scales."""
+    for ny in (768, 1024):
+        f = np.random.default_rng(ny).standard_normal((3, ny, 16))
+        ref = packed(f)
+        with chanfs.Plan(16, ny, 3, 2.0, 1.0, np.full(3, 0.5)) as plan:
+            s = plan.spectral_forward(torch.from_numpy(np.ldexp(f, -100)).cuda()).cpu().numpy()
+        got = np.ldexp(s, 100).view(np.complex128).reshape(ref.shape)
+        err = float(np.sqrt(np.sum(np.abs(got - ref) ** 2) / np.sum(np.abs(ref) ** 2)))
+        assert err < 3 * 2.0**-53  # (the fixed-point error of white noise is 1.5 at 4096)
