@@ -502,6 +502,11 @@ int cfs_slab_helmholtz_finish(cfs_slab_t slab, double c, int loc, const double* 
  *       16 KB of data per buffer) or 1..64.
  *   CFS_OPT_Y_TILE  complex columns per y-transform tile (of the precision the
  *       solves transform in): 0 automatic or 1..32 (even for refined plans).
+ *       Both shape a refined plan's own FP32 transforms, and FP64 ones of fewer
+ *       than nine points (nx/2 or ny).  Longer FP64 transforms and the boxes of
+ *       a group choose their shapes by length; the options are then accepted
+ *       and reported, with no effect, and no FP64 solve fails for a default
+ *       tile that does not fit.
  *   CFS_OPT_PCR_PARTS  z-partitions of Algorithm 2 for Helmholtz sets that
  *       are prepared without an explicit count: 0 automatic (about 32 rows
  *       per partition) or 1..64, each partition at least 3 rows.

@@ -257,11 +257,7 @@ bool y_tile_ok(const cfs_plan* P, int tk, bool fp32) {
 }
 
 cudaError_t launch_fft_y(const cfs_plan* P, double* data, bool inverse, cudaStream_t st) {
-  if (P->ny >= kFixMinLen) {
-    // a tile that does not fit is an invalid plan option here as elsewhere
-    return y_tile_ok(P, P->tk, false) ? launch_fix_y(P, data, inverse, st)
-                                      : cudaErrorInvalidValue;
-  }
+  if (P->ny >= kFixMinLen) return launch_fix_y(P, data, inverse, st);  // (tiles of its own)
   return launch_y<double2>(P, data, inverse, P->tk, P->d_twy, P->d_wy, st);
 }
 

@@ -69,7 +69,7 @@ static bool fits(const cfs_plan* P, const Choice& c) {
   const bool fp32 = (P->dtype == CFS_F32_REFINED);
   const size_t cs = fp32 ? sizeof(float2) : sizeof(double2);
   if (c.x_lines < 1 || c.x_lines > 64 || x_smem_bytes(P, c.x_lines, cs) > 227 * 1024) return false;
-  if (!y_tile_ok(P, c.y_tile, fp32)) return false;
+  if ((fp32 || P->ny < kFixMinLen) && !y_tile_ok(P, c.y_tile, fp32)) return false;
   if (c.thomas != -1 && thomas_tile_width(P, fp32, c.thomas) != c.thomas) return false;
   if (c.pcr_parts < 0 || c.pcr_parts > kPcrMaxParts) return false;
   for (int n = P->nz - 1; c.pcr_parts > 0 && n <= P->nz; ++n)
@@ -185,7 +185,7 @@ extern "C" int cfs_plan_autotune(cfs_plan_t P, void* stream) {
     best.y_tile = tk0;
     for (int cand : {1, 2, 4, 8, 16, 32}) {
       if (!y_tile_ok(P, cand, fp32)) continue;
-      if (!shaped_y) {  // the option must still name a tile that fits
+      if (!shaped_y) {  // not used: the option still names a tile that fits, if there is one
         if (!y_tile_ok(P, best.y_tile, fp32)) best.y_tile = cand;
         continue;
       }

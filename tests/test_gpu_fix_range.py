@@ -5,6 +5,9 @@ Poisson solve receive) and columns with one dominant value."""
 import numpy as np
 import pytest
 
+import oracle
+from paper_2502_06296_gb300 import synth
+
 torch = pytest.importorskip("torch")
 fft = pytest.importorskip("scipy.fft")
 pytestmark = pytest.mark.gpu
@@ -129,3 +132,37 @@ def test_far_long_columns_keep_their_bits(chanfs):
         got = np.ldexp(s, 100).view(np.complex128).reshape(ref.shape)
         err = float(np.sqrt(np.sum(np.abs(got - ref) ** 2) / np.sum(np.abs(ref) ** 2)))
         assert err < 3 * 2.0**-53  # (the fixed-point error of white noise is 1.5 at 4096)
+
+
+@pytest.mark.parametrize("ny", [972, 1296, 1458, 1944, 2048, 2187, 2916, 3072, 3888, 4096])
+def test_default_plans_transform_long_columns(chanfs, ny):
+    """Every length runs on a plan as it is made: one to four columns per tile, compiled and general kernels."""
+    check(chanfs, 18, ny, "spectrum")
+
+
+@pytest.mark.parametrize("ybc", [1, 2])
+@pytest.mark.parametrize("ny", [384, 432, 768, 1536, 2187, 4096])
+def test_default_plans_solve_between_walls(chanfs, ny, ybc):
+    nx, nz = 16 if ny % 2 else 4, 3  # (an odd count of rows asks for eight columns)
+    dz = synth.tanh_dz(nz, 1.4)
+    f = synth.normal(ny + ybc, (nz, ny, nx))
+    if ybc == 1:
+        f = synth.remove_weighted_mean(f, dz)
+    ref = oracle.poisson_solve_walls(f, 2.0, 1.0, dz, 0, ybc)
+    with chanfs.Plan(nx, ny, nz, 2.0, 1.0, dz, 0, 0, ybc) as plan:
+        p = plan.poisson_solve(torch.from_numpy(f).cuda()).cpu().numpy()
+        assert plan.check() == 0
+    assert np.max(np.abs(p - ref)) / np.max(np.abs(ref)) < 1e-12  # (as the z sweeps' test)
+
+
+@pytest.mark.parametrize("ny", [2048, 2187])
+def test_a_tuned_plan_keeps_the_bits_and_the_choice(chanfs, ny):
+    nx, nz = 18, 4
+    f = torch.from_numpy(synth.normal(ny, (nz, ny, nx))).cuda()
+    with chanfs.Plan(nx, ny, nz, 2.0, 1.0, np.full(nz, 0.5)) as plan:
+        before = plan.spectral_forward(f)
+        chosen = plan.autotune()
+        assert torch.equal(before, plan.spectral_forward(f))
+        assert plan.autotune() == chosen
+        p = plan.poisson_solve(f)
+        assert plan.check() == 0 and bool(torch.isfinite(p).all())
