@@ -32,6 +32,12 @@ constexpr int kResBlock = 128;
 // that they leave room for, are 3 to 13% slower at both.
 constexpr int kFirstPlanes = 4, kFirstMinBlocks = 5;
 constexpr int kUpdatePlanes = 4, kUpdateMinBlocks = 6;
+// Boxes of few planes, most of which no whole group reaches (by_planes), take pairs
+// of planes and more blocks per SM: a solve at 2592 x 1296 x 3, 4, 5 and 8 1141, 1344,
+// 1535 and 2149 us (1221, 1435, 1561 and 2218 in groups of four; plane by plane, the
+// next one's loads ahead, 1099, 1320, 1529 and 2199).  At nine planes groups of four
+// are even with them.
+constexpr int kThinNz = 8, kThinPlanes = 2, kThinMinBlocks = 8;
 
 __device__ __forceinline__ void block_max_to(float v, unsigned int* out) {
   // non-negative floats order like their bit patterns
@@ -270,6 +276,7 @@ __device__ __forceinline__ void by_planes(int k, int end, int nz, F&& group) {
   for (; k < end; ++k) group(std::integral_constant<int, 1>{}, k);
 }
 
+template <int PLANES>
 __device__ __forceinline__ void poisson_update_body(const float* __restrict__ dlt,
                                                     float* __restrict__ rhi,
                                                     float* __restrict__ rlo,
@@ -288,7 +295,7 @@ __device__ __forceinline__ void poisson_update_body(const float* __restrict__ dl
     const float4 axy = zk[3 * nz];
     const float* start = dlt + (size_t)kb * nxy;
     float dkm = kb ? ldf(start - nxy, q.c) : 0.0f, dk = ldf(start, q.c);
-    by_planes<kUpdatePlanes>(kb, ke, nz, [&](auto ng, int k0) {
+    by_planes<PLANES>(kb, ke, nz, [&](auto ng, int k0) {
       constexpr int G = decltype(ng)::value;
       float d[G], xp[G], xm[G], yp[G], ym[G], rh[G], rl[G];
 #pragma unroll
@@ -332,11 +339,12 @@ __device__ __forceinline__ void poisson_update_body(const float* __restrict__ dl
   block_max_to(vmax, rmax);
 }
 
-__global__ void __launch_bounds__(kResBlock, kUpdateMinBlocks) poisson_update_kernel(
+template <int PLANES, int MINB>
+__global__ void __launch_bounds__(kResBlock, MINB) poisson_update_kernel(
     const float* __restrict__ dlt, float* __restrict__ rhi, float* __restrict__ rlo,
     const float4* __restrict__ zk, unsigned int* rmax, int nx, int ny, int nz, int ybc,
     double* mpart) {
-  poisson_update_body(dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x);
+  poisson_update_body<PLANES>(dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x);
 }
 
 // ----------------------------------------------------------------------------
@@ -376,6 +384,7 @@ __device__ __forceinline__ void second_diff_acc(DoubleFloat& acc, float ch, floa
 
 // zk as for the update.  r32 must not alias dlt (the neighbours of a column
 // are read from dlt).
+template <int PLANES>
 __device__ __forceinline__ void poisson_first_body(
     const double* __restrict__ f, const double* __restrict__ mean, const float* __restrict__ dlt,
     float* __restrict__ rhi, float* __restrict__ rlo, const float4* __restrict__ zk,
@@ -396,7 +405,7 @@ __device__ __forceinline__ void poisson_first_body(
     float dk = ldf(start, q.c);
     float gh, gl;  // d_k - d_{k-1}, exact (d_{-1} = 0): what the plane below took as d_{k+1} - d_k
     two_sum(dk, kb ? -ldf(start - nxy, q.c) : 0.0f, gh, gl);
-    by_planes<kFirstPlanes>(kb, ke, nz, [&](auto ng, int k0) {
+    by_planes<PLANES>(kb, ke, nz, [&](auto ng, int k0) {
       constexpr int G = decltype(ng)::value;
       float d[G], xp[G], xm[G], yp[G], ym[G];
       double fk[G];
@@ -445,11 +454,13 @@ __device__ __forceinline__ void poisson_first_body(
   block_max_to(vmax, rmax);
 }
 
-__global__ void __launch_bounds__(kResBlock, kFirstMinBlocks) poisson_first_kernel(
+template <int PLANES, int MINB>
+__global__ void __launch_bounds__(kResBlock, MINB) poisson_first_kernel(
     const double* __restrict__ f, const double* __restrict__ mean, const float* __restrict__ dlt,
     float* __restrict__ rhi, float* __restrict__ rlo, const float4* __restrict__ zk,
     unsigned int* rmax, int nx, int ny, int nz, int ybc, double* mpart, float* __restrict__ dcopy) {
-  poisson_first_body(f, mean, dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x, dcopy);
+  poisson_first_body<PLANES>(f, mean, dlt, rhi, rlo, zk, rmax, nx, ny, nz, ybc, mpart, blockIdx.x,
+                             dcopy);
 }
 
 // The dz-weighted sum of a correction, from the per-block sums of the
@@ -580,8 +591,8 @@ __global__ void __launch_bounds__(kResBlock, kFirstMinBlocks) poisson_first_grou
   const ResBox& r = boxes[b];
   const double* mean = r.neumann ? r.mean : nullptr;
   double* mpart = r.neumann ? r.mpart : nullptr;
-  poisson_first_body(io[b].f, mean, r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz, r.ybc,
-                     mpart, blk, r.dcopy);
+  poisson_first_body<kFirstPlanes>(io[b].f, mean, r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny,
+                                   r.nz, r.ybc, mpart, blk, r.dcopy);
 }
 
 // One block per box (Neumann boxes; the others have nothing to sum).
@@ -618,7 +629,8 @@ __global__ void __launch_bounds__(kResBlock, kUpdateMinBlocks) poisson_update_gr
   if (!group_block(g, &b, &blk)) return;
   const ResBox& r = boxes[b];
   double* mpart = r.neumann ? r.mpart : nullptr;
-  poisson_update_body(r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz, r.ybc, mpart, blk);
+  poisson_update_body<kUpdatePlanes>(r.r32, r.r32b, r.rlo, r.zk, r.rmax, r.nx, r.ny, r.nz, r.ybc,
+                                     mpart, blk);
 }
 
 __global__ void first_only_group_kernel(const ResBox* boxes, GroupMap g, const GroupIo* io) {
@@ -864,6 +876,7 @@ static double* mean_num(cfs_plan* P) { return P->d_red + 2; }
 int refine_poisson(cfs_plan* P, const double* f, double* p, cudaStream_t st) {
   const long long nxy = (long long)P->nx * P->ny;
   const unsigned grid = (unsigned)res_grid(P->nx, P->ny, P->nz).blocks();
+  const bool thin = P->nz <= kThinNz;
   double* mean = nullptr;
   // one pass over f: r_0 = f as FP32, the extremes of r_0 and (Neumann) the
   // plane sums of the compatibility mean; then the reference norm
@@ -918,12 +931,16 @@ int refine_poisson(cfs_plan* P, const double* f, double* p, cudaStream_t st) {
     // (Neumann: each kernel also sums its correction, dz-weighted, per block)
     double* mpart = P->has_null ? P->d_mpart : nullptr;
     if (e == cudaSuccess && it == 0) {  // r = (f - mean) - L delta, by differences
-      poisson_first_kernel<<<grid, kResBlock, 0, st>>>(f, mean, W, P->d_r32b, P->d_rlo, P->d_zk,
+      auto k = thin ? poisson_first_kernel<kThinPlanes, kThinMinBlocks>
+                    : poisson_first_kernel<kFirstPlanes, kFirstMinBlocks>;
+      k<<<grid, kResBlock, 0, st>>>(f, mean, W, P->d_r32b, P->d_rlo, P->d_zk,
                                                        max_word(P), P->nx, P->ny, P->nz, P->ybc,
                                                        mpart, nullptr);
       e = cudaGetLastError();
     } else if (e == cudaSuccess) {  // r -= L delta
-      poisson_update_kernel<<<grid, kResBlock, 0, st>>>(W, P->d_r32b, P->d_rlo, P->d_zk,
+      auto k = thin ? poisson_update_kernel<kThinPlanes, kThinMinBlocks>
+                    : poisson_update_kernel<kUpdatePlanes, kUpdateMinBlocks>;
+      k<<<grid, kResBlock, 0, st>>>(W, P->d_r32b, P->d_rlo, P->d_zk,
                                                         max_word(P), P->nx, P->ny, P->nz, P->ybc,
                                                         mpart);
       e = cudaGetLastError();
