@@ -21,6 +21,8 @@
  *   as void* (NULL = legacy default stream).  Solves are asynchronous; input
  *   and output may be the same buffer (in place).  Plans own their tables and
  *   workspace; one plan may be used from one host thread at a time.
+ *   An infinity or NaN in a field of an FP64 transform makes every output of
+ *   its line NaN (along x, then along y; lines of nine points and more).
  *
  * Errors
  *   Every call returns a cfs_status.  Argument errors are detected on the host
@@ -488,8 +490,8 @@ int cfs_slab_helmholtz_finish(cfs_slab_t slab, double c, int loc, const double* 
  * order), and defaults are picked per plan from the problem size.
  *   CFS_OPT_THOMAS_TILE  columns per shared-memory tile of the z sweeps of
  *       Eq. 12: 0 automatic (the default), 8 or 16, or -1 for the streaming
- *       kernel (one thread per column, rows through registers, the forward
- *       sweep's intermediate written to the spectrum and read back).  Tiles
+ *       kernel (one to four real columns per thread, rows through registers,
+ *       the forward sweep's intermediate written to the spectrum and read back).  Tiles
  *       apply to FP64 sweeps only: the FP32 sweeps of refined plans stream
  *       (grouped solves have no tile variant, and a box gives the same bits
  *       grouped as alone), and get_option reports their shape.  Or, for
@@ -640,8 +642,8 @@ int cfs_probe_fma(int bits, long long iters, double* fma_per_s, double* ms);
 /*
  * cfs_probe_addsub -- a measurement with no counterpart in the paper: the
  * rate of FP64 butterfly pairs (a + b, a - b) on the FP64 pipe
- * (on_integer_units = 0) or by the integer-unit additions (1).  Every thread of one full wave of 256-thread blocks runs 8
- * independent pair chains for `iters` steps (rounded up to a multiple of
+ * (on_integer_units = 0) or by the integer-unit additions (1).  Every thread
+ * of one full wave of 256-thread blocks runs 8 independent pair chains for `iters` steps (rounded up to a multiple of
  * 256; 1 <= iters <= 2^40), timed as cfs_probe_fma.  *pairs_per_s receives
  * pairs per second, *ms (may be NULL) the launch time.  Waits for the device.
  */

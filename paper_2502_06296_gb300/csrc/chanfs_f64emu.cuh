@@ -2,14 +2,11 @@
 // integer units, bit for bit the round-to-nearest-even result of the FP64
 // pipe.
 //
-// The FP64 transforms are bound by the FP64 pipe: GB300 executes two FP64
-// lanes per SM per clock, one warp instruction every 16 clocks, while the
-// same SM issues four warp instructions per clock to its integer and FP32
-// pipes.  A butterfly pair (a + b, a - b) computed here costs a few dozen
-// integer and logic instructions instead of two FP64 instructions, so a
-// transform that moves part of its additions here runs both kinds of units
-// at once.  The results are the FP64 pipe's, so a kernel gives the same bits
-// whichever additions it moves.
+// Reached by the library's probe and self-checks alone (probe.cu): the FP64
+// transforms, which moved part of their additions here once, run in block fixed
+// point as a whole (chanfs_fix.cuh).  A butterfly pair (a + b, a - b) costs a few
+// dozen integer and logic instructions here instead of two FP64 instructions,
+// of which a warp's hold their SM quarter's pipe for 64 clocks each.
 //
 // The arithmetic follows the definition of binary64 addition (IEEE 754,
 // round to nearest, ties to even): align the smaller magnitude to the
