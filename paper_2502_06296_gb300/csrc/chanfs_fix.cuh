@@ -21,10 +21,11 @@
 // to the last place of 62, the result is rounded to a double once.  D = 4 suits
 // radix 8 and 6 and costs a radix-3 pass up to two bits of its values: a few such
 // passes fit the eight bits over a double's 53, more do not, so D = 2 in the
-// radix-3 passes of lengths that have four or more of them.  Relative L2 errors in
+// radix-3 passes of long plans of them (fix_halves).  Relative L2 errors in
 // units of 2^-53 of columns like 1/k^2, one dominant value, white noise and
 // magnitudes over 12 decades, D = 4 against 2: 729 7.9 8.7 1.8 3.3 against 0.7 0.6
-// 0.9 1.4; 2187 24 34 4.0 9.5 against 0.8 1.1 2.0 4.5; FP64 passes 1.5 to 4.4.
+// 0.9 1.4; 2187 24 34 4.0 9.5 against 0.8 1.1 2.0 4.5; 972 along x, inverse, 3.1 3.2
+// 1.3 2.7 against 1.0 1.0 1.3 2.8; FP64 passes 1.5 to 4.4.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -98,12 +99,15 @@ template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_twoff(int n
   return o;
 }
 
-// Whether the radix-3 passes divide by 2: where there are four or more of them
-// (lengths with four and more factors 3, none of which has a compiled kernel).
+// Whether the radix-3 passes divide by 2: in plans of five and more passes of radix
+// 6 and 3 with two and more of radix 3 (243, 486, 729, 972, 1458, 1944, 2187, 2916;
+// none has a compiled kernel).  Shorter plans lose nothing by 4, and 3888, with one
+// radix-3 pass, gains nothing by 2.
 template <bool PAIR> __host__ __device__ constexpr bool fix_halves(int n) {
   int threes = 0;
   for (int p = 0; p < fix_npass<PAIR>(n); ++p) threes += fix_radix<PAIR>(n, p) == 3;
-  return threes >= 4;
+  const int first = fix_radix<PAIR>(n, 0);
+  return fix_npass<PAIR>(n) >= 5 && threes >= 2 && (first == 6 || first == 3);
 }
 // Kernels of their own, radix 6 and 3 only (a test per pass in the general ones would
 // cost the other lengths 2 %): y at 64 x 729 x 64 103.6 us (96.5 dividing by 4), x at

@@ -68,7 +68,7 @@ def check(chanfs, nx, ny, kind):
 
 
 @pytest.mark.parametrize("kind", ["spectrum", "one value"])
-@pytest.mark.parametrize("nx,ny", [(162, 3), (486, 3), (972, 3), (1458, 3), (2916, 3), (3888, 3), (16, 81),
+@pytest.mark.parametrize("nx,ny", [(162, 3), (486, 3), (972, 3), (1458, 3), (1944, 3), (2916, 3), (3888, 3), (16, 81),
                                    (24, 243), (16, 486), (36, 729)])
 def test_lengths_of_many_radix_3_passes(chanfs, nx, ny, kind):
     check(chanfs, nx, ny, kind)
