@@ -110,8 +110,8 @@ template <bool PAIR> __host__ __device__ constexpr bool fix_halves(int n) {
   return fix_npass<PAIR>(n) >= 5 && threes >= 2 && (first == 6 || first == 3);
 }
 // Kernels of their own, radix 6 and 3 only (a test per pass in the general ones would
-// cost the other lengths 2 %): y at 64 x 729 x 64 103.6 us (96.5 dividing by 4), x at
-// 1458 x 64 x 64 105 us forward and 82 inverse (125 and 86).
+// cost the other lengths 2 %): y at 64 x 729 x 64 103.6 us against 96.5 dividing by 4,
+// x at 1458 x 64 x 64 105 us forward and 82 inverse against 125 and 86.
 constexpr int kHalved = -1;  // (as a length)
 // The bits that a pass p after the first divides by, and those of all of them.
 template <bool PAIR, bool INV> __host__ __device__ constexpr int fix_div(int n, int p) {
@@ -369,12 +369,9 @@ __device__ __forceinline__ void fix_gather(double v, unsigned& top, float& sum) 
   top = max(top, u);
   sum += __uint_as_float((max(u, 0x38100000u) - 0x38000000u) << 3);
 }
-template <int N> __device__ __forceinline__ void fix_gather(const double2* v, unsigned& top, float& sum) {
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    fix_gather(v[r].x, top, sum);
-    fix_gather(v[r].y, top, sum);
-  }
+__device__ __forceinline__ void fix_gather(double2 v, unsigned& top, float& sum) {
+  fix_gather(v.x, top, sum);
+  fix_gather(v.y, top, sum);
 }
 
 // A line's scale, and how its results leave.  kind 0: by a shift of the exponent;
@@ -391,10 +388,11 @@ __device__ __forceinline__ bool fix_near(unsigned top) { return (top >> 20) - 93
 // A line farther from 1 is moved first: all its values times 2^k, which brings its
 // largest near 1, exactly (what that takes below the subnormals is below 2^-1000 of
 // the largest).  So a power of two in the data comes out as that power of two, to
-// the last bit.  A line of subnormals moves to 1 .. 2^52.  (In registers, between two
-// reductions: the conversions have one form then.  Stages at 512 x 384 x 384 x 330 us
-// forward and 341 inverse, y 438 and 441, without any move 324, 333, 432 and 439; at
-// 384 x 256 x 192 between walls in y 161 and 170 against 167 and 186.)
+// the last bit.  A line of subnormals moves to 1 .. 2^52.  (The kernels
+// do this in a call of their own.  With the moves among the code that every line runs,
+// the x and y stages took 330 / 341 and 438 / 441 us at 512 x 384 x 384, y at 64 x 729 x
+// 64 103; with the call 327 / 322, 428 / 436 and 63; with neither 324 / 333, 432 / 439
+// and 96, the conversions then testing every value for the far cases.)
 __device__ __forceinline__ int fix_move(unsigned top) {
   const int e = (int)(top >> 20);
   return fix_near(top) || e == 0x7ff ? 0 : e ? 1023 - e : 1074;
@@ -403,16 +401,8 @@ __device__ __forceinline__ double fix_moved(double v, int k) {  // |k| <= 1074
   const int h = k / 2;
   return v * __hiloint2double((1023 + h) << 20, 0) * __hiloint2double((1023 + k - h) << 20, 0);
 }
-// A thread's values moved, and gathered again.
-template <int N>
-__device__ __forceinline__ void fix_gather_moved(double2* v, int k, unsigned& top, float& sum) {
-  if (k) {
-#pragma unroll
-    for (int r = 0; r < N; ++r) v[r] = make_double2(fix_moved(v[r].x, k), fix_moved(v[r].y, k));
-  }
-  top = 0u;
-  sum = 0.0f;
-  fix_gather<N>(v, top, sum);
+__device__ __forceinline__ double2 fix_moved(double2 v, int k) {
+  return k ? make_double2(fix_moved(v.x, k), fix_moved(v.y, k)) : v;
 }
 // Whether a line must be moved, as far as one thread knows: from its largest value,
 // or, where that is 0 or below 2^-1042, from the thread's own.

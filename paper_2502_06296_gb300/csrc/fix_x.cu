@@ -14,7 +14,7 @@
 // point: 21 in additions, 17 in the conversion from double, the rest in the
 // products' halves; 68 % busy in ncu at 24 warps per SM), against 13.75
 // instructions per point on an FP64 pipe 32 times narrower: 2.03 / 1.99 ms forward
-// / inverse in FP64 at 512 x 384 x 384 on GB300, 0.34 / 0.35 ms here (3.6 TB/s).
+// / inverse in FP64 at 512 x 384 x 384 on GB300, 0.33 / 0.32 ms here (3.7 TB/s).
 // Lengths with up to three factors 3 are compiled with every radix, span and offset a constant;
 // with a power of two of items per line, at most 32, a warp owns its lines and
 // never waits for another.
@@ -196,35 +196,30 @@ __device__ __forceinline__ unsigned line_sum(const XGroup& g, int l, bool on, un
   }
 }
 
-// Item it of the first pass: forward, butterfly j of line l (R points j + r Q);
-// inverse, the pairs of item i (2 R points, and the point 0 of item 0).
+// Value r of item i of the first pass: forward, butterfly i of the line (R points i +
+// r Q); inverse, the pairs of item i (2 R points, and the point 0 of item 0).
 template <int R, bool INV>
-__device__ __forceinline__ void load_item(const double2* line, int n, int Q, int i, double2* raw) {
+__device__ __forceinline__ double2 item_value(const double2* line, int n, int Q, int i, int r) {
   if constexpr (!INV) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) raw[r] = line[i + r * Q];
+    return line[i + r * Q];
   } else {
     const bool z = i == 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const bool have = !z || (Q & 1) == 0 || !pair_second<R>(r);
-      const int k = pair_index<R>(z, i, r, Q);
-      raw[2 * r] = have ? line[k] : make_double2(0.0, 0.0);
-      raw[2 * r + 1] = have ? line[n - k] : make_double2(0.0, 0.0);
-    }
-    raw[2 * R] = z ? line[0] : make_double2(0.0, 0.0);
+    if (r == 2 * R) return z ? line[0] : make_double2(0.0, 0.0);
+    const int k = pair_index<R>(z, i, r / 2, Q);
+    const bool have = !z || (Q & 1) == 0 || !pair_second<R>(r / 2);
+    return have ? line[r % 2 ? n - k : k] : make_double2(0.0, 0.0);
   }
 }
 
-// The first pass's arithmetic on a loaded item, written to buffer A.
-template <int R, bool INV>
+// The first pass's arithmetic on an item of values raw(r), written to buffer A.
+template <int R, bool INV, class Raw>
 __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, int Q, int i,
-                                           const double2* raw, int s,
+                                           Raw raw, int s,
                                            const int4* __restrict__ post) {
   if constexpr (!INV) {
     Fix v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = fix_from(raw[r], s);
+    for (int r = 0; r < R; ++r) v[r] = fix_from(raw(r), s);
     fdft<R, false>(v);
 #pragma unroll
     for (int r = 0; r < R; ++r) line[fix_pad(i * R + r)] = v[r];
@@ -233,7 +228,7 @@ __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, in
     Fix a[R], b[R], p[R], q[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {  // 2 Z_k = E + i conj(W^k) T, T = X_k - conj X_{M-k}
-      const Fix xk = fix_from(raw[2 * r], s), xm = fix_from(raw[2 * r + 1], s);
+      const Fix xk = fix_from(raw(2 * r), s), xm = fix_from(raw(2 * r + 1), s);
       const Fix e = {xk.x + xm.x, xk.y - xm.y};
       const Fix u = fmul(Fix{xk.x - xm.x, xk.y + xm.y},
                          __ldg(post + pair_index<R>(z, i, r, Q)));
@@ -242,7 +237,7 @@ __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, in
     }
     pair_give<R>(z, p, q, a, b);
     if (z) {
-      const Fix x0 = fix_from(raw[2 * R], s);  // (X_0, X_M)
+      const Fix x0 = fix_from(raw(2 * R), s);  // (X_0, X_M)
       a[0] = {x0.x + x0.y, x0.x - x0.y};
     }
     fdft<R, true>(a);
@@ -259,47 +254,94 @@ __device__ __forceinline__ void first_item(const XGroup& g, Fix* line, int n, in
 
 // The first pass of the group's lines: at most one item per thread, kept in
 // registers from the scan of its magnitudes on.
-// (sums: whether the scale uses the sum over the line.  Inverse: the two
-// butterflies of an item are each bounded by twice its sum, one factor 2 of which
-// is in the headroom.)
+template <int R, bool INV, int T> struct XItem {  // this thread's
+  static constexpr int kRaw = INV ? 2 * R + 1 : R;
+  int Q, l, i;
+  bool on;
+  const double2* line;
+  __device__ __forceinline__ XItem(const XGroup& g, const double2* in) {
+    Q = g.n / R;
+    const int per = T ? T : (INV ? (Q + 1) / 2 : Q);
+    l = min(g.lane / per, g.nl - 1);
+    i = g.lane - l * per;
+    on = g.lane < g.nl * per && l < g.nlines - g.line0;
+    line = in + (g.line0 + l) * g.n;
+  }
+  __device__ __forceinline__ double2 value(const XGroup& g, int r) const {
+    return item_value<R, INV>(line, g.n, Q, i, r);
+  }
+};
+// Its scale and arithmetic, the line's values times 2^k.  (sums: whether the scale
+// uses the sum over the line.  Inverse: the two butterflies of an item are each
+// bounded by twice its sum, one factor 2 of which is in the headroom.)
+template <int R, bool INV, bool WARP, int T, class Raw>
+__device__ __forceinline__ void first_arith(const XGroup& g, const XItem<R, INV, T>& it, Raw raw,
+                                            unsigned top, unsigned most, float sum, int k,
+                                            bool sums, const int4* __restrict__ post) {
+  unsigned quanta = 0u;
+  if (sums)
+    quanta = line_sum<WARP, T>(g, it.l, it.on,
+                               it.on ? (INV ? 2u : 1u) * fix_quanta(sum, top, most) : 0u);
+  if (it.on) {
+    const FixScale f = fix_scale_of(top, most, quanta, g.growth, g.headroom, g.div);
+    if (it.i == 0) g.scale[it.l] = fix_moved_back(f, k);
+    first_item<R, INV>(g, g.A + it.l * g.ps, g.n, it.Q, it.i, raw, f.s, post);
+  }
+}
+// The pass again from its loads on, for a group with a line far from 1.  (A call that
+// reads its values twice rather than keep them: the registers and the schedule of
+// the others know nothing of it.)
+template <int R, bool INV, bool WARP, int T>
+static __device__ __noinline__ void first_pass_far(XGroup g, const double2* in, bool sums,
+                                                   const int4* __restrict__ post) {
+  using Item = XItem<R, INV, T>;
+  const Item it(g, in);
+  unsigned top = 0u, most = 0u;
+  float sum = 0.0f;
+  if constexpr (WARP) {
+    if (it.on)
+#pragma unroll 1
+      for (int r = 0; r < Item::kRaw; ++r) fix_gather(it.value(g, r), top, sum);
+    line_max<WARP, T>(g, it.l, it.on, top, most);
+  } else {
+    top = g.top[it.l];  // the line's, from the first attempt
+    __syncthreads();
+    if (it.on && it.i == 0) g.top[it.l] = g.most[it.l] = 0u;
+    __syncthreads();
+  }
+  const int k = fix_move(top);
+  const auto raw = [&](int r) { return fix_moved(it.value(g, r), k); };
+  top = 0u;
+  sum = 0.0f;
+  if (it.on)
+#pragma unroll 1
+    for (int r = 0; r < Item::kRaw; ++r) fix_gather(raw(r), top, sum);
+  most = __float_as_uint(sum);
+  line_max<WARP, T>(g, it.l, it.on, top, most);
+  first_arith<R, INV, WARP, T>(g, it, raw, top, most, sum, k, sums, post);
+}
 template <int R, bool INV, bool WARP, int T>
 __device__ __forceinline__ void first_pass(const XGroup& g, const double2* in, bool sums,
                                            const int4* __restrict__ post) {
-  constexpr int NRAW = INV ? 2 * R + 1 : R;
-  const int Q = g.n / R;
-  const int per = T ? T : (INV ? (Q + 1) / 2 : Q);
-  const int items = g.nl * per;
-  const long long left = g.nlines - g.line0;
-  const int l = min(g.lane / per, g.nl - 1), i = g.lane - l * per;
-  const bool on = g.lane < items && l < left;
-  double2 raw[NRAW];
-  unsigned top = 0u, quanta = 0u;
+  using Item = XItem<R, INV, T>;
+  const Item it(g, in);
+  double2 raw[Item::kRaw];
+  unsigned top = 0u;
   float sum = 0.0f;
-  if (on) {
-    load_item<R, INV>(in + (g.line0 + l) * g.n, g.n, Q, i, raw);
-    fix_gather<NRAW>(raw, top, sum);
+  if (it.on) {
+#pragma unroll
+    for (int r = 0; r < Item::kRaw; ++r) raw[r] = it.value(g, r);
+#pragma unroll
+    for (int r = 0; r < Item::kRaw; ++r) fix_gather(raw[r], top, sum);
   }
   if constexpr (!WARP) __syncthreads();  // the reduction's cells are cleared
   unsigned most = __float_as_uint(sum);
-  int k = 0;
-  if (line_max<WARP, T>(g, l, on, top, most) &&
-      group_any<WARP>(on && fix_far<NRAW>(top, raw))) {  // seldom: the group gathers again
-    k = fix_move(top);
-    if constexpr (!WARP) {
-      if (on && i == 0) g.top[l] = g.most[l] = 0u;
-      __syncthreads();
-    }
-    if (on) fix_gather_moved<NRAW>(raw, k, top, sum);
-    most = __float_as_uint(sum);
-    line_max<WARP, T>(g, l, on, top, most);
-  }
-  if (sums)
-    quanta = line_sum<WARP, T>(g, l, on, on ? (INV ? 2u : 1u) * fix_quanta(sum, top, most) : 0u);
-  if (on) {
-    const FixScale f = fix_scale_of(top, most, quanta, g.growth, g.headroom, g.div);
-    if (i == 0) g.scale[l] = fix_moved_back(f, k);
-    first_item<R, INV>(g, g.A + l * g.ps, g.n, Q, i, raw, f.s, post);
-  }
+  if (line_max<WARP, T>(g, it.l, it.on, top, most) &&
+      group_any<WARP>(it.on && fix_far<Item::kRaw>(top, raw)))
+    first_pass_far<R, INV, WARP, T>(g, in, sums, post);
+  else
+    first_arith<R, INV, WARP, T>(g, it, [&](int r) { return raw[r]; }, top, most, sum, 0, sums,
+                                 post);
 }
 
 // A middle pass over the group's lines, from one buffer to the other.

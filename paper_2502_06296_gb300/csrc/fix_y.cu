@@ -6,7 +6,7 @@
 // with its own scale.  The first pass reads its butterflies from global memory
 // into registers, the last one writes them back, so a tile visits shared
 // memory only between passes.  512 x 384 x 384 on GB300: 1.70 ms in FP64 on TMA
-// tiles (bound by the FP64 pipe), 0.45 ms here (2.7 TB/s), bound by the integer
+// tiles (bound by the FP64 pipe), 0.43 ms here (2.8 TB/s), bound by the integer
 // ALU pipe and by the barriers between the passes of a tile; 3456 x 3072 x 30 11 ms
 // and 3.7 ms (tiles of two columns, one CTA of 24 warps per SM).
 #include "chanfs_fix.cuh"
@@ -24,16 +24,8 @@ struct YTile {
   bool first;      // the tile holds the packed column kx = 0
   Fix *A, *B;
   unsigned *top, *most, *quanta;
-  int* move;       // powers of two that the columns were moved by (fix_move)
+  FixScale* scale;
 };
-
-// The scale of column c as it was moved, and of its results.
-__device__ __forceinline__ FixScale moved_scale(const YTile& t, int c) {
-  return fix_scale_of(t.top[c], t.most[c], t.quanta[c], t.growth, t.headroom, t.div);
-}
-__device__ __forceinline__ FixScale scale_of(const YTile& t, int c) {
-  return fix_moved_back(moved_scale(t, c), t.move[c]);
-}
 
 // Rows of a wall transform: element t of the FFT is row wall_row(t).
 __device__ __forceinline__ int wall_row(int t, int n) {
@@ -68,15 +60,11 @@ __device__ __forceinline__ double2 load_packed(const YTile& t, int e) {
   return 2 * e < n ? make_double2(v.x - w.y, v.y + w.x) : make_double2(w.x + v.y, v.x - w.y);
 }
 
-template <int R, bool INV, bool WALL>
-__device__ __forceinline__ void load_points(const YTile& t, int j, int c, int ytype, double2* raw) {
-  const int Q = t.n / R;
-  if (INV && !WALL && t.first && c == 0) {
-    for (int r = 0; r < R; ++r) raw[r] = load_packed(t, j + r * Q);
-  } else {
-#pragma unroll
-    for (int r = 0; r < R; ++r) raw[r] = load_elem<INV, WALL>(t, j + r * Q, c, ytype);
-  }
+// Point e of column c as the first pass reads it.
+template <bool INV, bool WALL>
+__device__ __forceinline__ double2 load_point(const YTile& t, int e, int c, int ytype) {
+  if (INV && !WALL && t.first && c == 0) return load_packed(t, e);
+  return load_elem<INV, WALL>(t, e, c, ytype);
 }
 
 // V_e of the inverse wall transform from its column's X: conj(w_e) (X_e - i
@@ -86,84 +74,134 @@ __device__ __forceinline__ Fix wall_unmix(Fix xe, Fix xn, int4 wconj) {
   return fmul(Fix{xe.x + xn.y, xe.y - xn.x}, wconj);
 }
 
-template <int R, bool INV, bool WALL>
-__device__ __forceinline__ void first_points(const YTile& t, int j, int c, int ytype,
-                                             const double2* raw, int s,
-                                             const int4* __restrict__ wy) {
-  const int Q = t.n / R;
-  Fix v[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    v[r] = fix_from(raw[r], s);
-    if constexpr (INV && WALL) {
-      const int e = j + r * Q;
-      if (e > 0) {
-        const Fix xn = fix_from(load_elem<INV, WALL>(t, t.n - e, c, ytype), s);
-        v[r] = wall_unmix(v[r], xn, __ldg(wy + e));
-      }
-    }
-  }
-  fdft<R, INV>(v);
-#pragma unroll
-  for (int r = 0; r < R; ++r) t.A[fix_pad(((j * R + r) << t.sh) + c)] = v[r];
-}
-
 // The first pass of a tile: at most one item per thread, kept in registers from
 // the scan of its magnitudes on.
+template <int R> struct YItem {  // this thread's
+  int c, j;
+  bool on;
+  __device__ __forceinline__ explicit YItem(const YTile& t) {
+    const int it = threadIdx.x;
+    c = it & (t.tk - 1);
+    j = it >> t.sh;
+    on = it < (t.n / R) << t.sh && c < t.valid;
+  }
+  template <bool INV, bool WALL>
+  __device__ __forceinline__ double2 value(const YTile& t, int ytype, int r) const {
+    return load_point<INV, WALL>(t, j + r * (t.n / R), c, ytype);
+  }
+  __device__ __forceinline__ int place(const YTile& t, int r) const {  // of result r, in A
+    return fix_pad(((j * R + r) << t.sh) + c);
+  }
+};
+// The columns' maxima from their threads' (to t.top and t.most); whether one of
+// them may have to be moved (fix_move), the same to the whole tile.
+__device__ __forceinline__ bool column_max(const YTile& t, int c, bool on, unsigned top, float sum) {
+  const bool odd = on && !fix_near(top);
+  unsigned most = __float_as_uint(sum);
+  for (int o = t.tk; o < 32; o *= 2) {
+    top = max(top, __shfl_xor_sync(~0u, top, o));
+    most = max(most, __shfl_xor_sync(~0u, most, o));
+  }
+  if ((threadIdx.x & 31) < t.tk) {
+    atomicMax(t.top + c, top);
+    atomicMax(t.most + c, most);
+  }
+  return __syncthreads_or(odd);
+}
+// The scale of a thread's column, its values times 2^k (to t.scale for the others).
+// (sums: whether it uses the sum over the column.)
+template <int R>
+__device__ __forceinline__ int first_scale(const YTile& t, const YItem<R>& it, float sum, int k,
+                                           bool sums) {
+  const int c = it.c;
+  if (sums) {
+    unsigned q = it.on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
+    for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
+    if ((threadIdx.x & 31) < t.tk) atomicAdd(t.quanta + c, q);
+    __syncthreads();
+  }
+  const FixScale f = fix_scale_of(t.top[c], t.most[c], t.quanta[c], t.growth, t.headroom, t.div);
+  if (it.on && it.j == 0) t.scale[c] = fix_moved_back(f, k);
+  return f.s;
+}
+// Point r of an item in fixed point, from its value x (times 2^k; the mirrored point
+// of a wall is read here).
+template <int R, bool INV, bool WALL>
+__device__ __forceinline__ Fix first_point(const YTile& t, const YItem<R>& it, int ytype, int r,
+                                           double2 x, int k, int s, const int4* __restrict__ wy) {
+  const Fix v = fix_from(x, s);
+  if constexpr (INV && WALL) {
+    const int e = it.j + r * (t.n / R);
+    if (e > 0) {
+      double2 xn = load_elem<INV, WALL>(t, t.n - e, it.c, ytype);
+      xn = fix_moved(xn, k);
+      return wall_unmix(v, fix_from(xn, s), __ldg(wy + e));
+    }
+  }
+  return v;
+}
+// The pass up to its points in fixed point, left at the item's places of A, for a
+// tile with a column far from 1.  (A call that reads its values twice and keeps few
+// registers: the schedule of the other tiles knows nothing of it.)
+template <int R, bool INV, bool WALL>
+static __device__ __noinline__ void first_far(YTile t, int ytype, bool sums,
+                                              const int4* __restrict__ wy) {
+  const YItem<R> it(t);
+  const int k = fix_move(t.top[it.c]);  // from the first attempt
+  __syncthreads();
+  if (threadIdx.x < t.tk) t.top[it.c] = t.most[it.c] = 0u;
+  __syncthreads();
+  unsigned top = 0u;
+  float sum = 0.0f;
+  if (it.on)
+#pragma unroll 1
+    for (int r = 0; r < R; ++r)
+      fix_gather(fix_moved(it.template value<INV, WALL>(t, ytype, r), k), top, sum);
+  column_max(t, it.c, it.on, top, sum);
+  const int s = first_scale<R>(t, it, sum, k, sums);
+  if (it.on)
+#pragma unroll 1
+    for (int r = 0; r < R; ++r) {
+      const double2 x = fix_moved(it.template value<INV, WALL>(t, ytype, r), k);
+      t.A[it.place(t, r)] = first_point<R, INV, WALL>(t, it, ytype, r, x, k, s, wy);
+    }
+}
 template <int R, bool INV, bool WALL>
 __device__ __forceinline__ void first_pass(const YTile& t, int ytype, bool sums,
                                            const int4* __restrict__ wy) {
-  const int items = (t.n / R) << t.sh;
-  const int it = threadIdx.x, c = it & (t.tk - 1), j = it >> t.sh;
-  const bool on = it < items && c < t.valid;
+  const YItem<R> it(t);
   double2 raw[R];
   unsigned top = 0u;
   float sum = 0.0f;
-  if (on) {
-    load_points<R, INV, WALL>(t, j, c, ytype, raw);
-    fix_gather<R>(raw, top, sum);
+  if (it.on) {
+    if (INV && !WALL && t.first && it.c == 0) {
+      for (int r = 0; r < R; ++r) raw[r] = load_packed(t, it.j + r * (t.n / R));
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        raw[r] = load_elem<INV, WALL>(t, it.j + r * (t.n / R), it.c, ytype);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) fix_gather(raw[r], top, sum);
   }
   __syncthreads();  // the reduction's cells are cleared
-  const bool lead = (threadIdx.x & 31) < t.tk;
-  const auto column_max = [&] {  // whether a column of the tile may have to be moved
-    unsigned u = top, v = __float_as_uint(sum);
-    for (int o = t.tk; o < 32; o *= 2) {
-      u = max(u, __shfl_xor_sync(~0u, u, o));
-      v = max(v, __shfl_xor_sync(~0u, v, o));
-    }
-    if (lead) {
-      atomicMax(t.top + c, u);
-      atomicMax(t.most + c, v);
-    }
-    return __syncthreads_or(on && !fix_near(top));
-  };
-  if (column_max()) {
-    const unsigned all = t.top[c];
-    if (__syncthreads_or(on && fix_far<R>(all, raw))) {  // seldom: the tile gathers again
-      const int k = fix_move(all);
-      if (threadIdx.x < t.tk) t.top[c] = t.most[c] = 0u;
-      __syncthreads();
-      if (on) {
-        fix_gather_moved<R>(raw, k, top, sum);
-        t.move[c] = k;  // the same from every thread of the column
-        if constexpr (INV && WALL) {  // mirrored points are read again
+  Fix v[R];
+  if (column_max(t, it.c, it.on, top, sum) &&
+      __syncthreads_or(it.on && fix_far<R>(t.top[it.c], raw))) {
+    first_far<R, INV, WALL>(t, ytype, sums, wy);
+    if (!it.on) return;
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const int e = j + r * (t.n / R);
-            t.col[c + (size_t)(ytype == kSin ? t.n - 1 - e : e) * t.M] = raw[r];
-          }
-        }
-      }
-      column_max();
-    }
+    for (int r = 0; r < R; ++r) v[r] = t.A[it.place(t, r)];
+  } else {
+    const int s = first_scale<R>(t, it, sum, 0, sums);
+    if (!it.on) return;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      v[r] = first_point<R, INV, WALL>(t, it, ytype, r, raw[r], 0, s, wy);
   }
-  if (sums) {
-    unsigned q = on ? fix_quanta(sum, t.top[c], t.most[c]) : 0u;
-    for (int o = t.tk; o < 32; o *= 2) q += __shfl_xor_sync(~0u, q, o);
-    if (lead) atomicAdd(t.quanta + c, q);
-    __syncthreads();
-  }
-  if (on) first_points<R, INV, WALL>(t, j, c, ytype, raw, moved_scale(t, c).s, wy);
+  fdft<R, INV>(v);
+#pragma unroll
+  for (int r = 0; r < R; ++r) t.A[it.place(t, r)] = v[r];
 }
 
 template <int R, bool INV, bool HALF>
@@ -195,7 +233,7 @@ __device__ __forceinline__ void last_pass(const YTile& t, const Fix* in, Fix* ke
 #pragma unroll
       for (int r = 0; r < R; ++r) keep[fix_pad(((j + r * Q) << t.sh) + c)] = v[r];
     } else {
-      const FixScale f = scale_of(t, c);
+      const FixScale f = t.scale[c];
       double2* o = t.col + c;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -220,7 +258,7 @@ __device__ __forceinline__ void wall_mix(const YTile& t, const Fix* in, int ytyp
   for (int it = threadIdx.x; it < items; it += blockDim.x) {
     const int c = it & (t.tk - 1), k = it >> t.sh;
     if (c >= t.valid) continue;
-    const FixScale f = scale_of(t, c);
+    const FixScale f = t.scale[c];
     double2* o = t.col + c;
     const auto slot = [&](int e) { return (size_t)(ytype == kSin ? n - 1 - e : e) * t.M; };
     const Fix vk = in[fix_pad((k << t.sh) + c)];
@@ -241,7 +279,7 @@ __device__ __forceinline__ void wall_mix(const YTile& t, const Fix* in, int ytyp
 // = -i (Z_ky - conj Z_{Ny-ky}) / 2; the self-conjugate slots keep the pair.
 __device__ __forceinline__ void untangle_column(const YTile& t, const Fix* in) {
   const int n = t.n;
-  const FixScale f = scale_of(t, 0);
+  const FixScale f = t.scale[0];
   for (int k = threadIdx.x; 2 * k <= n; k += blockDim.x) {
     const Fix z = in[fix_pad(k << t.sh)];
     if (k == 0 || 2 * k == n) {
@@ -281,12 +319,25 @@ constexpr int y_threads(int n) {
   return ((items << y_shift(items)) + 31) / 32 * 32;
 }
 
+constexpr size_t y_smem(int n, int sh) {
+  const size_t pts = (size_t)n << sh;
+  return 2 * (pts + (pts >> 3)) * sizeof(Fix) + ((size_t)5 << sh) * sizeof(unsigned);
+}
+// Launch bounds: 24 warps per SM (80 registers), or 28 (72) where that and shared
+// memory make room for a block more (108, 144, 216 and lengths up to 72: 216 forward
+// 37 us with three blocks of nine warps, 41 with two).
+constexpr bool y_tight(int n) {
+  const int warps = y_threads(n) / 32;
+  const int room = (int)(228 * 1024 / (y_smem(n, y_shift(n / fix_radix<false>(n, 0))) + 1024));
+  return room > 24 / warps && 28 / warps > 24 / warps;
+}
 // N > 0: the compile-time length (periodic y); N = 0: any length, from d; N =
-// kHalved: one whose radix-3 passes divide by 2.  All ask for 24 warps per SM (80
-// registers).
+// kHalved: one whose radix-3 passes divide by 2.
 template <int N, bool INV, bool WALL>
-__global__ void __launch_bounds__(N > 0 ? y_threads(N > 0 ? N : 9) : 768,
-                                  N > 0 ? 768 / y_threads(N > 0 ? N : 9) : 1)
+__global__ void __launch_bounds__(N <= 0 ? 768 : y_tight(N > 0 ? N : 9) ? 448 : y_threads(N > 0 ? N : 9),
+                                  N <= 0                      ? 1
+                                  : y_tight(N > 0 ? N : 9) ? 2
+                                                              : 768 / y_threads(N > 0 ? N : 9))
     fix_y_kernel(double2* data, int M, FixDesc d, const int4* __restrict__ tw,
                  const int4* __restrict__ wy, int shift, int ytype) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -315,8 +366,8 @@ __global__ void __launch_bounds__(N > 0 ? y_threads(N > 0 ? N : 9) : 768,
   t.top = reinterpret_cast<unsigned*>(t.B + buf);
   t.most = t.top + t.tk;
   t.quanta = t.most + t.tk;
-  t.move = reinterpret_cast<int*>(t.quanta + t.tk);
-  for (int e = threadIdx.x; e < 4 * t.tk; e += blockDim.x) t.top[e] = 0u;
+  t.scale = reinterpret_cast<FixScale*>(t.quanta + t.tk);
+  for (int e = threadIdx.x; e < 3 * t.tk; e += blockDim.x) t.top[e] = 0u;
   Fix *a = t.A, *b = t.B;
   if constexpr (N > 0) {
     first_pass<fix_rad<false, INV>(N, 0), INV, false>(t, ytype, fix_uses_sum<false, INV>(N),
@@ -385,11 +436,6 @@ __global__ void __launch_bounds__(N > 0 ? y_threads(N > 0 ? N : 9) : 768,
       else untangle_column(t, b);
     }
   }
-}
-
-static size_t y_smem(int n, int sh) {
-  const size_t pts = (size_t)n << sh;
-  return 2 * (pts + (pts >> 3)) * sizeof(Fix) + ((size_t)4 << sh) * sizeof(unsigned);
 }
 
 template <int N, bool INV, bool WALL>

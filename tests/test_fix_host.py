@@ -61,7 +61,7 @@ template <bool PAIR, bool INV> static void run(int n, const double2* in, double2
     std::vector<float> sums;
     for (int j = 0; j < Q; ++j) {
       float sum = 0;
-      for (int r = 0; r < R; ++r) fix_gather<1>(in + j + r * Q, top, sum);
+      for (int r = 0; r < R; ++r) fix_gather(in[j + r * Q], top, sum);
       most = max(most, __float_as_uint(sum));
       sums.push_back(sum);
     }
